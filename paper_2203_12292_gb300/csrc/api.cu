@@ -535,6 +535,7 @@ void upload_all_tables() {
   if (done[dev]) return;
   upload_tables_cell();
   upload_tables_lanes();
+  upload_tables_lattice();
   upload_tables_transfer();
   upload_tables_mlp();
   upload_tables_dwl();
@@ -711,6 +712,11 @@ void setup_handle(Handle& H, const std::vector<Octree>& gc_meshes, int lmax, con
     t.gstart_c = H.lev[l - 1]->gstart.as<int32_t>();
     t.mask_c = H.lev[l - 1]->mask.as<uint16_t>();
     t.coarse = H.lev[l - 1]->cl;
+    if (t.kind == 0) {
+      T->lattice.alloc(lattice_table_words(t.kf, t.n_coarse) * sizeof(int32_t));
+      launch_lattice_entities(t, T->lattice.as<int32_t>(), H.stream);
+      t.lattice = T->lattice.as<int32_t>();
+    }
     H.tr[l] = std::move(T);
   }
   if (H.ls) {

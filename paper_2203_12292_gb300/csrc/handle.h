@@ -40,7 +40,7 @@ struct LevelDev {
 
 struct TransferDev {
   TransferHost host;
-  DevBuf fine_of, refined;
+  DevBuf fine_of, refined, lattice;
   TransferLaunch tl{};
 };
 

@@ -119,6 +119,7 @@ struct TransferLaunch {
   const uint32_t* own_f;    // fine cells
   const int32_t* gstart_c;  // coarse cells x 27
   const uint16_t* mask_c;   // coarse cells
+  const int32_t* lattice;   // h: entity table of the lattice kernels (null: not built)
   CellLaunch coarse;        // coarse level tiles (restriction scatter)
 };
 void launch_prolongate_add(const TransferLaunch& T, bool fp64, const void* coarse, void* fine, cudaStream_t s);
@@ -128,6 +129,18 @@ void launch_restrict_add(const TransferLaunch& T, bool fp64, const void* fine, v
 // coarse = R (b - Ax), no zeroing of coarse needed
 void launch_restrict_residual(const TransferLaunch& T, bool fp64, const void* b, const void* Ax, void* coarse,
                               bool overwrite, cudaStream_t s);
+
+// the h transfer with one warp per coarse cell (kernels_lattice.cu); the table
+// (lattice_table_words words) is built once per transfer from the other members
+size_t lattice_table_words(int k, int n_coarse);
+void launch_lattice_entities(const TransferLaunch& T, int32_t* table, cudaStream_t s);
+bool lattice_prolong_ok(const TransferLaunch& T);
+bool lattice_restrict_ok(const TransferLaunch& T);
+void launch_prolong_lattice(const TransferLaunch& T, bool fp64, const void* coarse, void* fine, cudaStream_t s);
+// coarse (+)= R fine, or R (rhs - fine) with rhs set
+void launch_restrict_lattice(const TransferLaunch& T, bool fp64, const void* fine, const void* rhs, void* coarse,
+                             bool overwrite, cudaStream_t s);
+void upload_tables_lattice();
 
 // vector kernels
 void upload_tables();

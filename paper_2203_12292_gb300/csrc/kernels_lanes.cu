@@ -40,30 +40,16 @@
 //     direction by direction) between separate passes.
 // The sums are therefore reproducible bit for bit.
 #include <algorithm>
-#include <map>
-#include <vector>
 
 #include "device.cuh"
 #include "kernels.h"
+#include "lanes.cuh"
 
 namespace gcmg {
 
 GCMG_DEFINE_UPLOAD(upload_tables_lanes_1d)
 
 namespace {
-
-constexpr int LW = 8;  // table entries of x-lines per warp
-
-// x-line r = b + N c of degree K: slot of node (0, b, c) | byte offset of the
-// node in its entity << 8 | byte offset of node (1, b, c) in the slot after it
-// << 16; per warp the x-lines it gathers and scatters (-1: none),
-// class-partitioned
-struct LaneLines {
-  uint32_t line[KMAX + 1][NMAX * NMAX];
-  int8_t xw[KMAX + 1][NMAX][LW];
-  int32_t nx[KMAX + 1][NMAX];  // x-lines of each warp
-};
-__constant__ LaneLines c_ll;
 
 template <typename T>
 struct LaneArgsT {
@@ -86,28 +72,6 @@ struct LaneArgsT {
   int tile0;
 };
 using LaneArgs = LaneArgsT<float>;
-
-// child-side interpolation I_p (TRANS: its transpose) on one line in
-// registers.  I_1[a][b] = I_0[k-a][k-b] (Gauss-Lobatto points and Lagrange
-// basis are symmetric under x -> 1 - x), so p = 1 reverses the line, applies
-// I_0 and reverses back: one set of constant-operand multiply-adds
-template <int K, bool TRANS>
-__device__ __forceinline__ void interp_line_reg(float* v, int p) {
-  constexpr int N = K + 1;
-  const DevTables<float>& tb = tab<float>(K);
-  float x[N], y[N];
-#pragma unroll
-  for (int a = 0; a < N; ++a) x[a] = p ? v[K - a] : v[a];
-#pragma unroll
-  for (int r = 0; r < N; ++r) {
-    float s = 0.f;
-#pragma unroll
-    for (int a = 0; a < N; ++a) s += (TRANS ? tb.I[0][a][r] : tb.I[0][r][a]) * x[a];
-    y[r] = s;
-  }
-#pragma unroll
-  for (int a = 0; a < N; ++a) v[a] = p ? y[K - a] : y[a];
-}
 
 // one direction D of C_e (TRANS: C_e^T) on the lines of warp w: line
 // q = i + N w has the other coordinates (u, v) = (q % N, q / N) in increasing
@@ -136,30 +100,6 @@ __device__ __forceinline__ void hang_pass(float* cb, uint16_t m, uint32_t hlD, i
 #pragma unroll
     for (int a = 0; a < N; ++a) ptr[a * S] = x[a];
   }
-}
-
-// *x += v where lanes with the same address (siblings behind one hanging face
-// or edge) add one after another in lane order; absent DoFs (the zero region)
-// add nothing.  Only lanes whose slot hangs can share an address within one
-// instruction: without such a lane (hang_any = 0) the plain addition is exact.
-__device__ __noinline__ void add_ordered_slow(float* x, float v, bool real, int lane) {
-  const unsigned key = real ? (unsigned)__cvta_generic_to_shared(x) : ~(unsigned)lane;
-  const unsigned peers = __match_any_sync(0xffffffffu, key);
-  const int rank = __popc(peers & ((1u << lane) - 1u));
-  const int most = __reduce_max_sync(0xffffffffu, (unsigned)__popc(peers));
-  for (int q = 0; q < most; ++q) {
-    if (real && rank == q) *x += v;
-    __syncwarp();
-  }
-}
-
-// (the ordered path out of line: the unrolled scatter of the tiles with hanging cells calls it
-// at every node, and inlined it would multiply that code)
-__device__ __forceinline__ void add_ordered(float* x, float v, bool real, int lane, bool hang_any) {
-  if (!hang_any)
-    *x += v;
-  else
-    add_ordered_slow(x, v, real, lane);
 }
 
 // zero the accumulator (n floats from the 16-byte aligned x0)
@@ -484,31 +424,6 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 8 : 1) vmult_lanes(Lane
 // wider than its FP64 pipe.  Values are converted once on entry to and once
 // on exit from the tile; the cell buffer and the accumulator hold df pairs.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ df df_sel(bool p, df a, df b) { return df{p ? a.hi : b.hi, p ? a.lo : b.lo}; }
-
-// sum_j x_j c_j over T double-float values and double-float constants
-// (ch + cl) with one normalisation: the high products p_j = x_j.hi ch_j carry
-// their exact rounding errors (fused multiply-add), the p_j are summed by
-// error-free two-sums, and the low-order terms (product errors, cross terms
-// x.hi cl and x.lo ch, two-sum errors) go into one fp32 sum; 12 T - 5
-// operations instead of 18 T - 11 for a chain of df_fma
-template <int T>
-__device__ __forceinline__ df df_dot(const df* x, const float* ch, const float* cl) {
-  float S = __fmul_rn(x[0].hi, ch[0]);
-  float L = __fmaf_rn(x[0].hi, cl[0], __fmaf_rn(x[0].lo, ch[0], __fmaf_rn(x[0].hi, ch[0], -S)));
-#pragma unroll
-  for (int j = 1; j < T; ++j) {
-    const float p = __fmul_rn(x[j].hi, ch[j]);
-    const float l = __fmaf_rn(x[j].hi, cl[j], __fmaf_rn(x[j].lo, ch[j], __fmaf_rn(x[j].hi, ch[j], -p)));
-    const float s = __fadd_rn(S, p);
-    const float z = __fsub_rn(s, S);
-    const float t = __fadd_rn(__fsub_rn(S, __fsub_rn(s, z)), __fsub_rn(p, z));
-    S = s;
-    L = __fadd_rn(L, __fadd_rn(l, t));
-  }
-  return df_norm(S, L);
-}
-
 // even-odd forward transform with B (nodal -> modes in mode order) and its
 // backward transform, in double-float, rows as df_dot
 template <int K>
@@ -558,29 +473,6 @@ __device__ __forceinline__ void df_eo_bwd_fast(df* u) {
     u[N - 1 - j] = df_sub(E[j], O[j]);
   }
   if (N % 2) u[NH] = E[NH];
-}
-
-// I_p (TRANS: transposed) on one df line, by the mirror identity of interp_line_reg
-template <int K, bool TRANS>
-__device__ __forceinline__ void interp_line_df(df* v, int p) {
-  constexpr int N = K + 1;
-  const float(&Ih)[NMAX][NMAX] = c_tf[K].I[0];
-  const float(&Il)[NMAX][NMAX] = c_tflo[K].I[0];
-  df x[N], y[N];
-#pragma unroll
-  for (int a = 0; a < N; ++a) x[a] = df_sel(p, v[K - a], v[a]);
-  float ch[NMAX], cl[NMAX];
-#pragma unroll
-  for (int r = 0; r < N; ++r) {
-#pragma unroll
-    for (int a = 0; a < N; ++a) {
-      ch[a] = TRANS ? Ih[a][r] : Ih[r][a];
-      cl[a] = TRANS ? Il[a][r] : Il[r][a];
-    }
-    y[r] = df_dot<N>(x, ch, cl);
-  }
-#pragma unroll
-  for (int a = 0; a < N; ++a) v[a] = df_sel(p, y[K - a], y[a]);
 }
 
 template <int K, int D, bool TRANS, bool SWEEP = false>
@@ -646,21 +538,6 @@ __device__ __forceinline__ void sweep_scale_df(df* cb, int w, int lane, df h) {
     df_eo_bwd_fast<K>(v);
 #pragma unroll
     for (int c = 0; c < N; ++c) p[c * S] = v[c];
-  }
-}
-
-__device__ __forceinline__ void add_ordered_df(df* x, df v, bool real, int lane, bool hang_any) {
-  if (!hang_any) {
-    *x = df_add(*x, v);
-    return;
-  }
-  const unsigned key = real ? (unsigned)__cvta_generic_to_shared(x) : ~(unsigned)lane;
-  const unsigned peers = __match_any_sync(0xffffffffu, key);
-  const int rank = __popc(peers & ((1u << lane) - 1u));
-  const int most = __reduce_max_sync(0xffffffffu, (unsigned)__popc(peers));
-  for (int q = 0; q < most; ++q) {
-    if (real && rank == q) *x = df_add(*x, v);
-    __syncwarp();
   }
 }
 
@@ -816,66 +693,6 @@ __global__ void __launch_bounds__((K + 1) * 32) vmult_lanes_df(LaneArgsT<double>
     for (int i = threadIdx.x; i < ti.n_owned; i += NT) d[i] = df_to(xs[i]);
   const int32_t* hp = A.halo_pos + ti.foreign_begin;
   for (int i = threadIdx.x; i < ti.n_foreign; i += NT) A.halo[hp[i]] = df_to(xs[ti.n_owned + i]);
-}
-
-// host: entity slot and offset of local node (a, b, c) of a degree-k cell
-// (the numbering of the level set-up: slot cx + 3 cy + 9 cz, DoFs of an
-// entity lexicographic over its interior axes)
-void host_node_slot(int k, int a, int b, int c, int& slot, int& off) {
-  const int ca = a == 0 ? 0 : (a == k ? 2 : 1), cbb = b == 0 ? 0 : (b == k ? 2 : 1),
-            cc = c == 0 ? 0 : (c == k ? 2 : 1);
-  slot = ca + 3 * cbb + 9 * cc;
-  int o = 0, mul = 1;
-  if (ca == 1) {
-    o += a - 1;
-    mul *= k - 1;
-  }
-  if (cbb == 1) {
-    o += (b - 1) * mul;
-    mul *= k - 1;
-  }
-  if (cc == 1) o += (c - 1) * mul;
-  off = o;
-}
-
-// x-line tables: slots and offsets per line; the line classes (lines whose
-// nodes can share DoFs between cells) dealt to the k+1 warps, largest class
-// first to the least loaded warp
-void fill_lane_lines(LaneLines& t) {
-  t = LaneLines{};
-  for (int k = 0; k <= KMAX; ++k)
-    for (int w = 0; w < NMAX; ++w)
-      for (int i = 0; i < LW; ++i) t.xw[k][w][i] = -1;
-  for (int k = 1; k <= KMAX; ++k) {
-    const int n = k + 1;
-    for (int c = 0; c < n; ++c)
-      for (int b = 0; b < n; ++b) {
-        int s0, o0, s1, o1 = 0;
-        host_node_slot(k, 0, b, c, s0, o0);
-        if (k > 1) host_node_slot(k, 1, b, c, s1, o1);
-        t.line[k][b + n * c] = (uint32_t)s0 | ((uint32_t)(4 * o0) << 8) | ((uint32_t)(4 * o1) << 16);
-      }
-    auto cls = [&](int x) { return (x == 0 || x == k) ? -1 : x; };
-    std::map<std::pair<int, int>, std::vector<int>> classes;
-    for (int c = 0; c < n; ++c)
-      for (int b = 0; b < n; ++b) classes[{cls(b), cls(c)}].push_back(b + n * c);
-    std::vector<std::vector<int>> cl;
-    for (auto& kv : classes) cl.push_back(kv.second);
-    std::stable_sort(cl.begin(), cl.end(), [](const std::vector<int>& x, const std::vector<int>& y) {
-      return x.size() > y.size();
-    });
-    std::vector<int> load(n, 0);
-    for (const auto& c : cl) {
-      int w = 0;
-      for (int u = 1; u < n; ++u)
-        if (load[u] < load[w]) w = u;
-      for (int r : c) {
-        if (load[w] >= LW) throw std::runtime_error("lane line table overflow");
-        t.xw[k][w][load[w]++] = (int8_t)r;
-      }
-    }
-    for (int w = 0; w < n; ++w) t.nx[k][w] = load[w];
-  }
 }
 
 template <int K>

@@ -648,7 +648,19 @@ void restrict_any(const TransferLaunch& L, const T* src, T* dst, const T* rhs, b
 }  // namespace
 
 #ifndef GCMG_BODIES_ONLY
+// The h transfer runs one warp per coarse cell (kernels_lattice.cu).  The
+// kernels of this file take the p transfer, the restriction onto tiles above 32
+// cells and with a set chunk size, and the recorded launches of the persistent
+// batch, whose blocks all have the layout of these kernels.
+bool lattice_restrict(const TransferLaunch& L) {
+  return lattice_restrict_ok(L) && L.coarse.chunk == 0 && !dwl_recording();
+}
+
 void launch_prolongate_add(const TransferLaunch& L, bool fp64, const void* coarse, void* fine, cudaStream_t s) {
+  if (lattice_prolong_ok(L) && !dwl_recording()) {
+    launch_prolong_lattice(L, fp64, coarse, fine, s);
+    return;
+  }
   if (fp64)
     prolong_any<double>(L, static_cast<const double*>(coarse), static_cast<double*>(fine), s);
   else
@@ -656,6 +668,10 @@ void launch_prolongate_add(const TransferLaunch& L, bool fp64, const void* coars
 }
 
 void launch_restrict_add(const TransferLaunch& L, bool fp64, const void* fine, void* coarse, cudaStream_t s) {
+  if (lattice_restrict(L)) {
+    launch_restrict_lattice(L, fp64, fine, nullptr, coarse, false, s);
+    return;
+  }
   if (fp64)
     restrict_any<double>(L, static_cast<const double*>(fine), static_cast<double*>(coarse), nullptr, false, s);
   else
@@ -664,6 +680,10 @@ void launch_restrict_add(const TransferLaunch& L, bool fp64, const void* fine, v
 
 void launch_restrict_residual(const TransferLaunch& L, bool fp64, const void* b, const void* Ax, void* coarse,
                               bool overwrite, cudaStream_t s) {
+  if (lattice_restrict(L)) {
+    launch_restrict_lattice(L, fp64, Ax, b, coarse, overwrite, s);
+    return;
+  }
   if (fp64)
     restrict_any<double>(L, static_cast<const double*>(Ax), static_cast<double*>(coarse),
                          static_cast<const double*>(b), overwrite, s);
