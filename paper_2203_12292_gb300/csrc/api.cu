@@ -373,9 +373,24 @@ bool any_learned(const Handle& H) {
   return false;
 }
 
+// The levels 0 .. dense_top take their matrix unless one of them is observed or
+// changed on its own: timers, a learned smoother, a recorded launch list of the
+// persistent batch, the cycle stopped after the coarse-grid correction.
+bool dense_usable(const Handle& H, int l) {
+  if (l != H.dense_top || !H.dense_ok || H.prof.on || dwl_recording()) return false;
+  if (H.stop_after_cgc && l == (int)H.lev.size() - 1) return false;
+  for (int q = 0; q <= l; ++q)
+    if (H.lev[q]->smoother != GCMG_SMOOTHER_CHEBYSHEV) return false;
+  return true;
+}
+
 void vcycle_level(Handle& H, int l) {
   LevelDev& L = *H.lev[l];
   const bool f64 = !L.fp32;
+  if (dense_usable(H, l)) {
+    launch_dense_apply(f64, H.dense.p, (int)L.n(), L.b.p, L.x.p, H.stream);
+    return;
+  }
   if (l == 0) {
     const int r = prof_begin(H, 0, GCMG_STAGE_COARSE);
     if (H.n0) launch_coarse_solve(f64, H.Ainv.as<double>(), H.n0, L.b.p, L.x.p, H.stream);
@@ -536,11 +551,62 @@ void upload_all_tables() {
   upload_tables_cell();
   upload_tables_lanes();
   upload_tables_lattice();
+  upload_tables_dense();
   upload_tables_transfer();
   upload_tables_mlp();
   upload_tables_dwl();
   ck(cudaDeviceSynchronize(), "upload tables");
   done[dev] = 1;
+}
+
+// the V-cycle matrix of the smallest levels (kernels_dense.cu): global
+// coarsening on Cartesian cells, every level below included
+void setup_dense(Handle& H) {
+  H.dense_ok = false;
+  H.dense_top = -1;
+  if (H.ls) return;
+  int top = -1;
+  for (int l = 0; l <= H.top_mg && H.lev[l]->n() <= DENSE_MAX && !H.lev[l]->cl.geom; ++l)
+    if (l >= 1 && H.lev[l]->n() > 0) top = l;
+  if (top < 0) return;
+  int nmax = 1;
+  for (int l = 0; l <= top; ++l) nmax = std::max(nmax, (int)H.lev[l]->n());
+  const size_t q = (size_t)nmax * nmax;
+  DevBuf work;  // the products' scratch, A, P, M of the coarser level
+  work.alloc(dense_scratch_bytes(nmax) + 3 * q * sizeof(double));
+  double* A = work.as<double>() + dense_scratch_bytes(nmax) / sizeof(double);
+  double *P = A + q, *Mc = A + 2 * q;
+  int n_c = H.n0;
+  if (n_c) ck(cudaMemcpyAsync(Mc, H.Ainv.p, (size_t)n_c * n_c * sizeof(double), cudaMemcpyDeviceToDevice, H.stream), "copy");
+  for (int l = 1; l <= top; ++l) {
+    LevelDev& L = *H.lev[l];
+    const int n = (int)L.n();
+    if (n == 0) {
+      n_c = 0;
+      continue;
+    }
+    launch_dense_operator(L.cl, n, (int)L.host.cells.size(), L.gstart.as<int32_t>(), A, H.stream);
+    if (n_c) launch_dense_prolongation(H.tr[l]->tl, n, n_c, (int)L.host.cells.size(), P, H.stream);
+    std::vector<double> coef;
+    for (const ChebCoef& c : cheb_coefs(L.lam, H.cfg.smoothing_range, H.cfg.cheb_degree)) {
+      coef.push_back(c.c1);
+      coef.push_back(c.c2);
+    }
+    const double* M = dense_vcycle_matrix(n, A, L.dinv64.as<double>(), (int)coef.size() / 2, coef.data(), n_c, P, Mc,
+                                          work.as<double>(), H.stream);
+    if (l < top)
+      ck(cudaMemcpyAsync(Mc, M, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToDevice, H.stream), "copy");
+    else {
+      const size_t bytes = (size_t)n * n * (L.fp32 ? sizeof(float) : sizeof(double));
+      if (H.dense.bytes != bytes) H.dense.alloc(bytes);
+      launch_dense_store(!L.fp32, M, H.dense.p, (int64_t)n * n, H.stream);
+    }
+    n_c = n;
+  }
+  ck_launches("dense levels");
+  ck(cudaStreamSynchronize(H.stream), "dense levels");  // the scratch is freed on return
+  H.dense_top = top;
+  H.dense_ok = true;
 }
 
 void setup_numerics(Handle& H) {
@@ -568,6 +634,7 @@ void setup_numerics(Handle& H) {
     H.lev[l]->lam = H.cfg.eig_safety * estimate_lambda(H, l);
     ck_launches("eigenvalue estimate");
   }
+  setup_dense(H);
   H.g_core.reset();
   H.g_a.reset();
 }
@@ -1190,6 +1257,7 @@ int gcmg_set_lambda(gcmg_handle* h, int level, double lam) {
     if (!h || !(lam > 0)) throw Error(GCMG_ERR_ARG, "bad lambda");
     check_level(h->h, level);
     h->h.lev[level]->lam = lam;
+    if (level <= h->h.dense_top) h->h.dense_ok = false;  // that interval is not the matrix's: level by level from now on
     h->h.g_core.reset();
   });
 }

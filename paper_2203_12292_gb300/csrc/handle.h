@@ -93,6 +93,11 @@ struct Handle {
   int n_sm = 152;               // multiprocessors of the handle's device (set-up)
   bool stop_after_cgc = false;  // finest level: return after the prolongation
   bool ls = false;              // local smoothing: lev[0..top_mg] refinement levels, lev.back() the active mesh
+  // V-cycle of the levels 0 .. dense_top as one matrix (-1: none); dense_ok: it
+  // belongs to the levels' present operators and Chebyshev intervals
+  int dense_top = -1;
+  bool dense_ok = false;
+  DevBuf dense;
   int top_mg = 0;               // finest multigrid level (lev.size() - 1 for global coarsening)
   bool in_batch = false;        // owned by a batch, whose graph holds the kernels' arguments
   cudaStream_t cap_stream = nullptr;

@@ -142,6 +142,19 @@ void launch_restrict_lattice(const TransferLaunch& T, bool fp64, const void* fin
                              bool overwrite, cudaStream_t s);
 void upload_tables_lattice();
 
+// the V-cycle of the smallest levels as one dense matrix (kernels_dense.cu),
+// on levels of at most DENSE_MAX DoFs
+constexpr int DENSE_MAX = 1024;
+void upload_tables_dense();
+// A of a level (n x n, rows) and P of a transfer (n_f x n_c, rows), fp64
+void launch_dense_operator(const CellLaunch& L, int n, int n_cells, const int32_t* gstart, double* A, cudaStream_t s);
+void launch_dense_prolongation(const TransferLaunch& T, int n_f, int n_c, int cells_f, double* P, cudaStream_t s);
+size_t dense_scratch_bytes(int n);
+double* dense_vcycle_matrix(int n, const double* A, const double* dinv, int steps, const double* coef, int n_c,
+                            const double* P, const double* Mc, double* work, cudaStream_t s);
+void launch_dense_store(bool fp64, const double* M, void* out, int64_t n, cudaStream_t s);
+void launch_dense_apply(bool fp64, const void* M, int n, const void* b, void* x, cudaStream_t s);
+
 // vector kernels
 void upload_tables();
 void launch_cast(bool to64, const void* src, void* dst, int64_t n, cudaStream_t s);
