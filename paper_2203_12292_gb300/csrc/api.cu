@@ -559,15 +559,17 @@ void upload_all_tables() {
   done[dev] = 1;
 }
 
-// the V-cycle matrix of the smallest levels (kernels_dense.cu): global
-// coarsening on Cartesian cells, every level below included
+// the V-cycle matrix of the smallest levels (kernels_dense.cu): Cartesian cells,
+// every level below included; under local smoothing only while the levels below
+// take no copied values (their right-hand side is R r alone)
 void setup_dense(Handle& H) {
   H.dense_ok = false;
   H.dense_top = -1;
-  if (H.ls) return;
   int top = -1;
-  for (int l = 0; l <= H.top_mg && H.lev[l]->n() <= DENSE_MAX && !H.lev[l]->cl.geom; ++l)
+  for (int l = 0; l <= H.top_mg && H.lev[l]->n() <= DENSE_MAX && !H.lev[l]->cl.geom; ++l) {
     if (l >= 1 && H.lev[l]->n() > 0) top = l;
+    if (H.lev[l]->n_cp > 0) break;
+  }
   if (top < 0) return;
   int nmax = 1;
   for (int l = 0; l <= top; ++l) nmax = std::max(nmax, (int)H.lev[l]->n());
