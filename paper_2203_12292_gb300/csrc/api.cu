@@ -289,12 +289,13 @@ void smooth(Handle& H, int l, bool fp64, void* x, const void* b, void* d, void* 
   const auto c = cheb_coefs(L.lam, H.cfg.smoothing_range, H.cfg.cheb_degree);
   size_t it = 0;
   if (zero_init) {
-    launch_cheb_init(fp64, x, d, b, dinv, c[0].c2, n, H.stream);
+    launch_cheb_init(fp64, x, b, dinv, c[0].c2, n, H.stream);
     it = 1;
   }
   for (; it < c.size(); ++it) {
+    const int step = it == 0 ? CHEB_FIRST : (zero_init && it == 1 ? CHEB_AFTER_ZERO : CHEB_NEXT);
     vmult(H, l, fp64, x, t);
-    launch_cheb_step(fp64, x, d, b, t, dinv, c[it].c1, c[it].c2, n, H.stream);
+    launch_cheb_step(fp64, step, it + 1 == c.size(), x, d, b, t, dinv, c[it].c1, c[it].c2, n, H.stream);
   }
 }
 

@@ -156,7 +156,10 @@ bool dwl_record(const void* kernel, unsigned grid, unsigned block, size_t smem, 
 #define GCMG_DWL_VEC(X)                                                                             \
   X((cast_kernel<float, double>)) X((cast_kernel<double, float>)) X((copy_kernel))                  \
   X((zero_kernel<float>)) X((zero_kernel<double>)) X((cheb_init_kernel<float>))                     \
-  X((cheb_step_kernel<float, true>)) X((cheb_step_kernel<float, false>)) X((residual_kernel<float>)) \
+  X((cheb_step_kernel<float, CHEB_FIRST, false>)) \
+  X((cheb_step_kernel<float, CHEB_FIRST, true>)) X((cheb_step_kernel<float, CHEB_AFTER_ZERO, false>)) \
+  X((cheb_step_kernel<float, CHEB_AFTER_ZERO, true>)) X((cheb_step_kernel<float, CHEB_NEXT, false>)) \
+  X((cheb_step_kernel<float, CHEB_NEXT, true>)) X((residual_kernel<float>))                         \
   X((coarse_kernel<float>)) X((dot_partial_b<double>)) X((dot_partial_b<float>)) X((dot_final))     \
   X((cg_xr_b<false>)) X((cg_xr_b<true>)) X((cg_p_kernel<double>)) X((cg_p_kernel<float>))
 #define GCMG_DWL_VEC_SERIAL(X) X((scalar_set_kernel)) X((cg_stats_kernel))

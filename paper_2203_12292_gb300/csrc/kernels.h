@@ -172,9 +172,12 @@ void launch_copy_from_level(bool fp64, const void* src, const int32_t* g, const 
 // a[idx[i]] = b[idx[i]] = 0 (Jacobi inverse on refinement-edge DoFs)
 void launch_zero_at(const int32_t* idx, int64_t n, double* a, float* b, cudaStream_t s);
 void launch_invert(const double* d, double* inv64, float* inv32, int64_t n, cudaStream_t s);
-void launch_cheb_init(bool fp64, void* x, void* d, const void* b, const void* dinv, double c2, int64_t n, cudaStream_t s);
-void launch_cheb_step(bool fp64, void* x, void* d, const void* b, const void* Ax, const void* dinv, double c1,
-                      double c2, int64_t n, cudaStream_t s);
+// a Chebyshev step: the first of a smoother, the one after the start from zero
+// (d = x on entry), or a later one; last: d is not written
+enum ChebStep { CHEB_FIRST, CHEB_AFTER_ZERO, CHEB_NEXT };
+void launch_cheb_init(bool fp64, void* x, const void* b, const void* dinv, double c2, int64_t n, cudaStream_t s);
+void launch_cheb_step(bool fp64, int step, bool last, void* x, void* d, const void* b, const void* Ax, const void* dinv,
+                      double c1, double c2, int64_t n, cudaStream_t s);
 void launch_residual(bool fp64, void* r, const void* b, const void* Ax, int64_t n, cudaStream_t s);
 void launch_axpy(bool fp64, void* y, const void* x, double a, int64_t n, cudaStream_t s);
 void launch_fill(double* x, double v, int64_t n, cudaStream_t s);

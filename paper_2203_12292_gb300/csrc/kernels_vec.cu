@@ -2,7 +2,8 @@
 //
 // * Chebyshev iteration around point Jacobi (Sec. 3.3): one fused pass per
 //   step, d <- c1 d + c2 D^{-1} (b - A x), x <- x + d (c1 = 0 starts the
-//   recurrence).  Reads b, Ax, D^{-1}, d, x and writes d, x.
+//   recurrence).  Reads b, Ax, D^{-1}, d, x and writes d, x; d only between the
+//   first and the last step.
 // * Algorithm 1: casts between the fp64 CG vectors and the fp32 levels.
 // * Sec. 3.4: the level-0 solve is a dense product with the inverse of the
 //   (small, fp64) level-0 matrix.
@@ -139,28 +140,30 @@ __global__ void invert_kernel(const double* d, double* i64, float* i32, int64_t 
   }
 }
 
+// the start from zero: x = c2 D^-1 b.  d equals x there, so it is not stored:
+// the next step takes d from x (12 instead of 16 B per DoF in fp32)
 template <typename T>
-__global__ void cheb_init_kernel(T* x, T* d, const T* b, const T* dinv, T c2, int64_t n) {
+__global__ void cheb_init_kernel(T* x, const T* b, const T* dinv, T c2, int64_t n) {
   pdl_begin();
-  grid_stride4(
-      n, [&](int64_t i) { return c2 * dinv[i] * b[i]; },
-      [&](int64_t i, T v) {
-        d[i] = v;
-        x[i] = v;
-      });
+  grid_stride4(n, [&](int64_t i) { return c2 * dinv[i] * b[i]; }, [&](int64_t i, T v) { x[i] = v; });
 }
 
-template <typename T, bool FIRST>
+// one Chebyshev step; STEP: CHEB_FIRST (c1 = 0, d not read), CHEB_AFTER_ZERO (d
+// is x), CHEB_NEXT; LAST: d is not needed again and not written.  fp32 bytes
+// per DoF of three presmoothing and three postsmoothing steps: 136 instead of
+// 152 (every step read and wrote d)
+template <typename T, int STEP, bool LAST>
 __global__ void cheb_step_kernel(T* x, T* d, const T* b, const T* Ax, const T* dinv, T c1, T c2, int64_t n) {
   pdl_begin();
   struct V {
     T r, di, d, x;
   };
   grid_stride4(
-      n, [&](int64_t i) { return V{b[i] - Ax[i], dinv[i], FIRST ? T(0) : d[i], x[i]}; },
+      n, [&](int64_t i) { return V{b[i] - Ax[i], dinv[i], STEP == CHEB_NEXT ? d[i] : T(0), x[i]}; },
       [&](int64_t i, V e) {
-        const T v = FIRST ? c2 * e.di * e.r : c1 * e.d + c2 * e.di * e.r;
-        d[i] = v;
+        const T dp = STEP == CHEB_AFTER_ZERO ? e.x : e.d;
+        const T v = STEP == CHEB_FIRST ? c2 * e.di * e.r : c1 * dp + c2 * e.di * e.r;
+        if (!LAST) d[i] = v;
         x[i] = e.x + v;
       });
 }
@@ -494,38 +497,46 @@ void launch_invert(const double* d, double* inv64, float* inv32, int64_t n, cuda
   { launch_pdl(invert_kernel, grid_for(n), BLOCK, 0, s, d, inv64, inv32, n); note_launches(1); }
 }
 
-void launch_cheb_init(bool fp64, void* x, void* d, const void* b, const void* dinv, double c2, int64_t n,
-                      cudaStream_t s) {
+void launch_cheb_init(bool fp64, void* x, const void* b, const void* dinv, double c2, int64_t n, cudaStream_t s) {
   if (n <= 0) return;
   if (fp64)
-    { launch_pdl(cheb_init_kernel<double>, grid_for(n), BLOCK, 0, s, (double*)x, (double*)d, (const double*)b,
-                                                            (const double*)dinv, c2, n); note_launches(1); }
+    launch_pdl(cheb_init_kernel<double>, grid_for(n), BLOCK, 0, s, (double*)x, (const double*)b, (const double*)dinv, c2, n);
   else
-    { launch_pdl(cheb_init_kernel<float>, grid_for(n), BLOCK, 0, s, (float*)x, (float*)d, (const float*)b, (const float*)dinv,
-                                                           (float)c2, n); note_launches(1); }
+    launch_pdl(cheb_init_kernel<float>, grid_for(n), BLOCK, 0, s, (float*)x, (const float*)b, (const float*)dinv, (float)c2,
+               n);
+  note_launches(1);
 }
 
-void launch_cheb_step(bool fp64, void* x, void* d, const void* b, const void* Ax, const void* dinv, double c1,
-                      double c2, int64_t n, cudaStream_t s) {
+namespace {
+template <typename T, int STEP>
+void cheb_step(bool last, T* x, T* d, const T* b, const T* Ax, const T* dinv, T c1, T c2, int64_t n, cudaStream_t s) {
+  if (last)
+    launch_pdl(cheb_step_kernel<T, STEP, true>, grid_for(n), BLOCK, 0, s, x, d, b, Ax, dinv, c1, c2, n);
+  else
+    launch_pdl(cheb_step_kernel<T, STEP, false>, grid_for(n), BLOCK, 0, s, x, d, b, Ax, dinv, c1, c2, n);
+  note_launches(1);
+}
+template <typename T>
+void cheb_step_any(int step, bool last, T* x, T* d, const T* b, const T* Ax, const T* dinv, T c1, T c2, int64_t n,
+                   cudaStream_t s) {
+  if (step == CHEB_FIRST)
+    cheb_step<T, CHEB_FIRST>(last, x, d, b, Ax, dinv, c1, c2, n, s);
+  else if (step == CHEB_AFTER_ZERO)
+    cheb_step<T, CHEB_AFTER_ZERO>(last, x, d, b, Ax, dinv, c1, c2, n, s);
+  else
+    cheb_step<T, CHEB_NEXT>(last, x, d, b, Ax, dinv, c1, c2, n, s);
+}
+}  // namespace
+
+void launch_cheb_step(bool fp64, int step, bool last, void* x, void* d, const void* b, const void* Ax, const void* dinv,
+                      double c1, double c2, int64_t n, cudaStream_t s) {
   if (n <= 0) return;
-  const bool first = (c1 == 0.0);
-  if (fp64) {
-    if (first)
-      { launch_pdl(cheb_step_kernel<double, true>, grid_for(n), BLOCK, 0, s, (double*)x, (double*)d, (const double*)b,
-                                                                   (const double*)Ax, (const double*)dinv, c1, c2, n); note_launches(1); }
-    else
-      { launch_pdl(cheb_step_kernel<double, false>, grid_for(n), BLOCK, 0, s, (double*)x, (double*)d, (const double*)b,
-                                                                    (const double*)Ax, (const double*)dinv, c1, c2, n); note_launches(1); }
-  } else {
-    if (first)
-      { launch_pdl(cheb_step_kernel<float, true>, grid_for(n), BLOCK, 0, s, (float*)x, (float*)d, (const float*)b,
-                                                                  (const float*)Ax, (const float*)dinv, (float)c1,
-                                                                  (float)c2, n); note_launches(1); }
-    else
-      { launch_pdl(cheb_step_kernel<float, false>, grid_for(n), BLOCK, 0, s, (float*)x, (float*)d, (const float*)b,
-                                                                   (const float*)Ax, (const float*)dinv, (float)c1,
-                                                                   (float)c2, n); note_launches(1); }
-  }
+  if (fp64)
+    cheb_step_any<double>(step, last, (double*)x, (double*)d, (const double*)b, (const double*)Ax, (const double*)dinv, c1,
+                          c2, n, s);
+  else
+    cheb_step_any<float>(step, last, (float*)x, (float*)d, (const float*)b, (const float*)Ax, (const float*)dinv,
+                         (float)c1, (float)c2, n, s);
 }
 
 void launch_residual(bool fp64, void* r, const void* b, const void* Ax, int64_t n, cudaStream_t s) {
@@ -700,8 +711,11 @@ void dwl_register_vec() {
 #define GCMG_DWL_COARSEN(fn) dwl_set_coarsen(reinterpret_cast<const void*>(fn), 4);
   GCMG_DWL_COARSEN((cast_kernel<float, double>)) GCMG_DWL_COARSEN((cast_kernel<double, float>))
   GCMG_DWL_COARSEN((copy_kernel)) GCMG_DWL_COARSEN((zero_kernel<float>)) GCMG_DWL_COARSEN((zero_kernel<double>))
-  GCMG_DWL_COARSEN((cheb_init_kernel<float>)) GCMG_DWL_COARSEN((cheb_step_kernel<float, true>))
-  GCMG_DWL_COARSEN((cheb_step_kernel<float, false>)) GCMG_DWL_COARSEN((residual_kernel<float>))
+  GCMG_DWL_COARSEN((cheb_init_kernel<float>)) GCMG_DWL_COARSEN((residual_kernel<float>))
+  GCMG_DWL_COARSEN((cheb_step_kernel<float, CHEB_FIRST, false>)) GCMG_DWL_COARSEN((cheb_step_kernel<float, CHEB_FIRST, true>))
+  GCMG_DWL_COARSEN((cheb_step_kernel<float, CHEB_AFTER_ZERO, false>))
+  GCMG_DWL_COARSEN((cheb_step_kernel<float, CHEB_AFTER_ZERO, true>))
+  GCMG_DWL_COARSEN((cheb_step_kernel<float, CHEB_NEXT, false>)) GCMG_DWL_COARSEN((cheb_step_kernel<float, CHEB_NEXT, true>))
   GCMG_DWL_COARSEN((cg_p_kernel<double>)) GCMG_DWL_COARSEN((cg_p_kernel<float>))
 #undef GCMG_DWL_COARSEN
   dwl_register(reinterpret_cast<const void*>(cg_check_kernel), DWL_OP_CHECK, dwl_args_size(cg_check_kernel));
