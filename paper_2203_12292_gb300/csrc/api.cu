@@ -128,6 +128,13 @@ void vmult(Handle& H, int l, bool fp64, const void* src, void* dst, int stage) {
   prof_end(H, r);
 }
 
+// the cell vectors of A x on a level of few cells (the pass that adds them up follows)
+void cell_vectors(Handle& H, int l, bool fp64, const void* x) {
+  const int r = prof_begin(H, l, GCMG_STAGE_VMULT);
+  launch_cell_vectors(H.lev[l]->cl, fp64, x, H.stream);
+  prof_end(H, r);
+}
+
 double dot_host(Handle& H, const double* x, const double* y, int64_t n) {
   if (n == 0) return 0.0;
   launch_dot(x, y, n, H.scratch.as<double>(), H.scal.as<double>(), 8, DOT_STORE, H.stream);
@@ -281,21 +288,33 @@ std::vector<ChebCoef> cheb_coefs(double lam_max, double range, int degree) {
   return c;
 }
 
-// Chebyshev smoother on level l with vectors x, b, d, t (precision fp64)
-void smooth(Handle& H, int l, bool fp64, void* x, const void* b, void* d, void* t, const void* dinv, bool zero_init) {
+// Chebyshev smoother on level l with vectors x, b, d, t (precision fp64);
+// pending (zero_init only): b is formed from the level's cell vectors first
+void smooth(Handle& H, int l, bool fp64, void* x, const void* b, void* d, void* t, const void* dinv, bool zero_init,
+            void* pending = nullptr) {
   LevelDev& L = *H.lev[l];
   const int64_t n = L.n();
   if (n == 0) return;
   const auto c = cheb_coefs(L.lam, H.cfg.smoothing_range, H.cfg.cheb_degree);
+  const bool cells = cells_ok(L.cl);
   size_t it = 0;
   if (zero_init) {
-    launch_cheb_init(fp64, x, b, dinv, c[0].c2, n, H.stream);
+    if (pending)
+      launch_cell_sum_start(L.cl, fp64, pending, x, dinv, c[0].c2, H.stream);
+    else
+      launch_cheb_init(fp64, x, b, dinv, c[0].c2, n, H.stream);
     it = 1;
   }
   for (; it < c.size(); ++it) {
     const int step = it == 0 ? CHEB_FIRST : (zero_init && it == 1 ? CHEB_AFTER_ZERO : CHEB_NEXT);
+    const bool last = it + 1 == c.size();
+    if (cells) {
+      cell_vectors(H, l, fp64, x);
+      launch_cell_sum_cheb(L.cl, fp64, step, last, x, d, b, dinv, c[it].c1, c[it].c2, H.stream);
+      continue;
+    }
     vmult(H, l, fp64, x, t);
-    launch_cheb_step(fp64, step, it + 1 == c.size(), x, d, b, t, dinv, c[it].c1, c[it].c2, n, H.stream);
+    launch_cheb_step(fp64, step, last, x, d, b, t, dinv, c[it].c1, c[it].c2, n, H.stream);
   }
 }
 
@@ -385,9 +404,10 @@ bool dense_usable(const Handle& H, int l) {
   return true;
 }
 
-void vcycle_level(Handle& H, int l) {
+void vcycle_level(Handle& H, int l, bool pending) {
   LevelDev& L = *H.lev[l];
   const bool f64 = !L.fp32;
+  if (pending && (l == 0 || dense_usable(H, l))) launch_cell_sum(L.cl, f64, L.b.p, false, H.stream);
   if (dense_usable(H, l)) {
     launch_dense_apply(f64, H.dense.p, (int)L.n(), L.b.p, L.x.p, H.stream);
     return;
@@ -400,19 +420,33 @@ void vcycle_level(Handle& H, int l) {
   }
   const void* dinv = f64 ? L.dinv64.p : L.dinv32.p;
   int r = prof_begin(H, l, GCMG_STAGE_PRESMOOTH);
-  smooth(H, l, f64, L.x.p, L.b.p, L.d.p, L.t.p, dinv, true);  // presmoothing
+  smooth(H, l, f64, L.x.p, L.b.p, L.d.p, L.t.p, dinv, true, pending ? L.b.p : nullptr);  // presmoothing
   prof_end(H, r);
   r = prof_begin(H, l, GCMG_STAGE_RESIDUAL);
-  vmult(H, l, f64, L.x.p, L.t.p);  // A x for the residual
+  // A x for the residual; on a level of few cells the residual itself (its pass over the DoFs forms it)
+  const bool formed = cells_ok(L.cl);
+  if (formed) {
+    cell_vectors(H, l, f64, L.x.p);
+    launch_cell_sum_residual(L.cl, f64, L.b.p, L.t.p, H.stream);
+  } else {
+    vmult(H, l, f64, L.x.p, L.t.p);
+  }
   prof_end(H, r);
   LevelDev& C = *H.lev[l - 1];
   r = prof_begin(H, l, GCMG_STAGE_RESTRICT);
   // the residual r = b - A x is formed in the restriction's gather; global coarsening:
   // b^(l-1) = R r; local smoothing: b^(l-1) += R (r_S, r_E) on top of the values Algorithm 1
   // copied to level l-1 (r_E = -A_ES x_S: b_E is zero on level l)
-  if (C.n()) launch_restrict_residual(H.tr[l]->tl, f64, L.b.p, L.t.p, C.b.p, !H.ls, H.stream);
+  // onto a level of few cells the result stays in its cell vectors until its presmoothing starts
+  // (local smoothing: added to the copied values now)
+  const bool to_cells = C.n() && cells_ok(C.cl) && lattice_prolong_ok(H.tr[l]->tl);
+  if (to_cells) {
+    launch_restrict_cells(H.tr[l]->tl, f64, L.t.p, formed ? nullptr : L.b.p, H.stream);
+    if (H.ls) launch_cell_sum(C.cl, f64, C.b.p, true, H.stream);
+  } else if (C.n())
+    launch_restrict_residual(H.tr[l]->tl, f64, formed ? nullptr : L.b.p, L.t.p, C.b.p, !H.ls, H.stream);
   prof_end(H, r);
-  vcycle_level(H, l - 1);
+  vcycle_level(H, l - 1, to_cells && !H.ls);
   r = prof_begin(H, l, GCMG_STAGE_PROLONGATE);
   if (C.n()) launch_prolongate_add(H.tr[l]->tl, f64, C.x.p, L.x.p, H.stream);  // prolongation
   prof_end(H, r);
@@ -553,6 +587,7 @@ void upload_all_tables() {
   upload_tables_lanes();
   upload_tables_lattice();
   upload_tables_dense();
+  upload_tables_small();
   upload_tables_transfer();
   upload_tables_mlp();
   upload_tables_dwl();
@@ -640,6 +675,43 @@ void setup_numerics(Handle& H) {
   setup_dense(H);
   H.g_core.reset();
   H.g_a.reset();
+}
+
+// per DoF the positions of its entries in the cell vectors (node n of cell c at
+// c (k+1)^3 + n, x fastest), increasing
+void cell_vector_lists(const LevelHost& L, std::vector<int32_t>& ptr, std::vector<int32_t>& pos) {
+  const int n1 = L.k + 1, n3 = n1 * n1 * n1;
+  std::vector<int> slot(n3), off(n3);
+  for (int n = 0; n < n3; ++n) {
+    const int x[3] = {n % n1, (n / n1) % n1, n / (n1 * n1)};
+    int s = 0, o = 0, ms = 1, mo = 1;
+    for (int d = 0; d < 3; ++d) {
+      const int c = x[d] == 0 ? 0 : (x[d] == L.k ? 2 : 1);
+      s += c * ms;
+      ms *= 3;
+      if (c == 1) {
+        o += (x[d] - 1) * mo;
+        mo *= L.k - 1;
+      }
+    }
+    slot[n] = s;
+    off[n] = o;
+  }
+  const size_t nc = L.cells.size();
+  ptr.assign((size_t)L.n_free + 1, 0);
+  for (size_t c = 0; c < nc; ++c)
+    for (int n = 0; n < n3; ++n) {
+      const int32_t g = L.gstart[c * NSLOT + slot[n]];
+      if (g >= 0) ++ptr[g + off[n] + 1];
+    }
+  for (int64_t i = 0; i < L.n_free; ++i) ptr[i + 1] += ptr[i];
+  pos.assign(ptr[L.n_free], 0);
+  std::vector<int32_t> at(ptr.begin(), ptr.end() - 1);
+  for (size_t c = 0; c < nc; ++c)
+    for (int n = 0; n < n3; ++n) {
+      const int32_t g = L.gstart[c * NSLOT + slot[n]];
+      if (g >= 0) pos[at[g + off[n]]++] = (int32_t)(c * n3 + n);
+    }
 }
 
 void setup_handle(Handle& H, const std::vector<Octree>& gc_meshes, int lmax, const gcmg_config& cfg) {
@@ -734,6 +806,23 @@ void setup_handle(Handle& H, const std::vector<Octree>& gc_meshes, int lmax, con
     c.lane_tiles_lo = lh.lane.empty() ? nullptr : L->lane_tiles_lo.p;
     c.lane_hang_lo = lh.lane.empty() ? nullptr : L->lane_hang_lo.p;
     c.n_hang_tiles = lh.n_hang_tiles;
+    // levels of few cells, unless the operator kernel was chosen: the entries of every DoF in the
+    // cell vectors, in cell order
+    if (cfg.cell_kernel == 0 && cfg.cell_threads == 0 && lh.n_free > 0 &&
+        cell_vectors_pay((int64_t)lh.cells.size(), k, H.n_sm)) {
+      std::vector<int32_t> ptr, pos;
+      cell_vector_lists(lh, ptr, pos);
+      L->sum_ptr.upload(ptr, H.stream);
+      L->sum_pos.upload(pos, H.stream);
+      ck(cudaStreamSynchronize(H.stream), "upload");  // the lists are freed on return
+      L->cell_vec.alloc(lh.cells.size() * (size_t)((k + 1) * (k + 1) * (k + 1)) * sizeof(double));
+      c.sum_ptr = L->sum_ptr.as<int32_t>();
+      c.sum_pos = L->sum_pos.as<int32_t>();
+      c.cell_vec = L->cell_vec.p;
+    }
+    c.gstart = L->gstart.as<int32_t>();
+    c.n_cells = (int)lh.cells.size();
+    c.n_dofs = (int)lh.n_free;
     c.cell_ijk = L->cell_ijk.as<int32_t>();
     c.k = k;
     c.tc = tc;

@@ -30,6 +30,10 @@ __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
+// The same after a kernel has loaded what no kernel of the cycle writes (index
+// lists, tile records, diagonals): those loads overlap the predecessor's tail.
+// Their values are written by set-up calls only, which synchronise.
+__device__ __forceinline__ void pdl_wait() { pdl_begin(); }
 
 // asynchronous global -> shared copies (cp.async): a thread issues all its
 // copies of a tile before waiting once, so the latency of the tile's loads is

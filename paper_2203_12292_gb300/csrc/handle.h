@@ -18,6 +18,7 @@ struct LevelDev {
   bool fp32 = true;
   DevBuf tiles, meta, foreign, subptr, perm, cell_ijk, gstart, own, mask, lane_tiles, lane_order, lane_hang, tiles_lo,
       lane_tiles_lo, lane_hang_lo;
+  DevBuf sum_ptr, sum_pos, cell_vec;  // levels of few cells
   DevBuf halo, halo_dofs, halo_ptr, halo_src, halo_pos;
   DevBuf diag64, dinv64, dinv32;
   DevBuf x, b, d, t;        // V-cycle vectors in level precision
@@ -146,7 +147,8 @@ void check_level(const Handle& h, int level);
 int prof_begin(Handle& H, int level, int stage);
 void prof_end(Handle& H, int rec);
 void vmult(Handle& H, int l, bool fp64, const void* src, void* dst, int stage = GCMG_STAGE_VMULT);
-void vcycle_level(Handle& H, int l);
+// pending: the level's right-hand side is still in its cell vectors (a restricted residual)
+void vcycle_level(Handle& H, int l, bool pending = false);
 bool any_learned(const Handle& H);
 
 }  // namespace gcmg

@@ -47,6 +47,14 @@ struct CellLaunch {
   const void* lane_tiles_lo;
   const void* lane_hang_lo;
   int n_hang_tiles;           // tiles with hanging cells
+  // levels of few cells (kernels_small.cu): per DoF its entries in the cell
+  // vectors (null: the level has none)
+  const int32_t* sum_ptr;
+  const int32_t* sum_pos;
+  void* cell_vec;             // n_cells (k+1)^3 values of the launch precision
+  const int32_t* gstart;
+  int n_cells;
+  int n_dofs;
   double lo, dom;
   const double* coef;  // per cell coefficient nu_e (element matrix nu_e h A_ref); null: 1
   int geom;            // 0: Cartesian cells; GEOM_WARP: the cells mapped by the warp below
@@ -140,7 +148,35 @@ void launch_prolong_lattice(const TransferLaunch& T, bool fp64, const void* coar
 // coarse (+)= R fine, or R (rhs - fine) with rhs set
 void launch_restrict_lattice(const TransferLaunch& T, bool fp64, const void* fine, const void* rhs, void* coarse,
                              bool overwrite, cudaStream_t s);
+// the restriction of fine (rhs - fine with rhs set) to the coarse level's cell vectors
+void launch_restrict_cells(const TransferLaunch& T, bool fp64, const void* fine, const void* rhs, cudaStream_t s);
 void upload_tables_lattice();
+
+// the operator of a level of few cells: cell vectors, then one pass over the
+// DoFs that adds them up and goes on (kernels_small.cu)
+// Levels that take them: those too small for 32-cell tiles (fewer than two tiles
+// per SM), and larger ones of low degree up to CELL_VEC_MAX entries.  Postsmoothing
+// in fp32, tiles -> cell vectors: Q4 4,712 cells 61 -> 56 us, 7,680 cells 76 -> 51;
+// Q1 37,871 cells (0.30 M entries) 46 -> 23, 82,776 cells (0.66 M) 58 -> 36; Q2
+// 21,512 cells (0.58 M) 59 -> 50, but 32,768 cells (0.88 M) 40 -> 45 and Q4 21,512
+// cells (2.7 M) 111 -> 128 (fp64 crosses at the same sizes)
+constexpr int64_t CELL_VEC_MAX = 850000;
+inline bool cell_vectors_pay(int64_t cells, int k, int n_sm) {
+  return cells < 2 * (int64_t)n_sm * 32 || cells * (k + 1) * (k + 1) * (k + 1) <= CELL_VEC_MAX;
+}
+bool cells_ok(const CellLaunch& L);
+void launch_cell_vectors(const CellLaunch& L, bool fp64, const void* src, cudaStream_t s);
+void launch_cell_sum(const CellLaunch& L, bool fp64, void* dst, bool add, cudaStream_t s);
+void launch_cell_sum_residual(const CellLaunch& L, bool fp64, const void* b, void* r, cudaStream_t s);
+// a Chebyshev step on b - sum: the first of a smoother, the one after the start
+// from zero (d = x on entry), or a later one; last: d is not written
+enum ChebStep { CHEB_FIRST, CHEB_AFTER_ZERO, CHEB_NEXT };
+void launch_cell_sum_cheb(const CellLaunch& L, bool fp64, int step, bool last, void* x, void* d, const void* b,
+                          const void* dinv, double c1, double c2, cudaStream_t s);
+// b = sum (a restricted residual), x = c2 dinv b
+void launch_cell_sum_start(const CellLaunch& L, bool fp64, void* b, void* x, const void* dinv, double c2,
+                           cudaStream_t s);
+void upload_tables_small();
 
 // the V-cycle of the smallest levels as one dense matrix (kernels_dense.cu),
 // on levels of at most DENSE_MAX DoFs
@@ -172,9 +208,6 @@ void launch_copy_from_level(bool fp64, const void* src, const int32_t* g, const 
 // a[idx[i]] = b[idx[i]] = 0 (Jacobi inverse on refinement-edge DoFs)
 void launch_zero_at(const int32_t* idx, int64_t n, double* a, float* b, cudaStream_t s);
 void launch_invert(const double* d, double* inv64, float* inv32, int64_t n, cudaStream_t s);
-// a Chebyshev step: the first of a smoother, the one after the start from zero
-// (d = x on entry), or a later one; last: d is not written
-enum ChebStep { CHEB_FIRST, CHEB_AFTER_ZERO, CHEB_NEXT };
 void launch_cheb_init(bool fp64, void* x, const void* b, const void* dinv, double c2, int64_t n, cudaStream_t s);
 void launch_cheb_step(bool fp64, int step, bool last, void* x, void* d, const void* b, const void* Ax, const void* dinv,
                       double c1, double c2, int64_t n, cudaStream_t s);

@@ -1598,6 +1598,11 @@ size_t cell_smem_bytes(int k, bool fp64, int tc, int max_local, bool mapped) {
 
 void launch_vmult(const CellLaunch& L, bool fp64, const void* src, void* dst, int add, cudaStream_t s) {
   if (L.n_tiles == 0) return;
+  if (cells_ok(L)) {  // a level of few cells
+    launch_cell_vectors(L, fp64, src, s);
+    launch_cell_sum(L, fp64, dst, add != 0, s);
+    return;
+  }
   if (fp64) {
     CellArgs<double> A = make_args<double>(L);
     A.src = static_cast<const double*>(src);
@@ -1624,6 +1629,7 @@ void launch_vmult(const CellLaunch& L, bool fp64, const void* src, void* dst, in
 }
 
 bool vmult_tiles_ok(const CellLaunch& L, bool fp64) {
+  if (cells_ok(L)) return false;
   if (L.use_lanes && lanes_ok(L)) return true;
   return L.tc <= CHUNK && !L.geom && (fp64 || (L.use_lines && L.threads == BLOCK));
 }

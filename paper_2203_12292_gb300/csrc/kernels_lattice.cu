@@ -221,7 +221,6 @@ struct RestrictSmem {
 
 template <int K, typename T>
 __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
-  pdl_begin();
   using L = Lat<K>;
   using SM = RestrictSmem<K, T>;
   constexpr int N = L::N, N2 = L::N2, N3 = L::N3, M = L::M, M2 = L::M2, M3 = L::M3;
@@ -254,6 +253,7 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
 #pragma unroll
     for (int i = 0; i < L::EPL; ++i) en[i] = ep[w * L::ES + lane + 32 * i];
   cp_async_wait_all();
+  pdl_wait();
   __syncthreads();
   const T* __restrict__ src = A.src;
   const T* __restrict__ rhs = A.rhs;
@@ -404,9 +404,9 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
   for (int i = threadIdx.x; i < ti.n_foreign; i += NT) A.halo[hp[i]] = ys[ti.n_owned + i];
 }
 
-// one direction of C on the coarse values of a warp's lattice (node (a, b, c)
-// at a + M b + M^2 c)
-template <int K, int D, typename T>
+// one direction of C (TRANS: C^T) on the coarse values of a warp's lattice
+// (node (a, b, c) at a + M b + M^2 c)
+template <int K, int D, bool TRANS, typename T>
 __device__ __forceinline__ void lattice_hang(T* lat, uint16_t m, int lane) {
   using L = Lat<K>;
   if (lane >= L::N2) return;
@@ -417,7 +417,7 @@ __device__ __forceinline__ void lattice_hang(T* lat, uint16_t m, int lane) {
   T x[L::N];
 #pragma unroll
   for (int a = 0; a < L::N; ++a) x[a] = p[a * S];
-  interp_line<K, false>(x, (m >> D) & 1);
+  interp_line<K, TRANS>(x, (m >> D) & 1);
 #pragma unroll
   for (int a = 0; a < L::N; ++a) p[a * S] = x[a];
 }
@@ -430,7 +430,6 @@ constexpr size_t prolong_smem() {
 
 template <int K, typename T>
 __global__ void __launch_bounds__(WPB * 32) prolong_lattice(LatArgs<T> A) {
-  pdl_begin();
   using L = Lat<K>;
   constexpr int N = L::N, N3 = L::N3, M = L::M, M2 = L::M2;
   constexpr int NT = WPB * 32;
@@ -452,6 +451,7 @@ __global__ void __launch_bounds__(WPB * 32) prolong_lattice(LatArgs<T> A) {
     m = A.mask_c[c];
   }
   cp_async_wait_all();
+  pdl_wait();
   __syncthreads();
   if (c >= A.n_coarse) return;
   {  // G^(c)
@@ -474,11 +474,11 @@ __global__ void __launch_bounds__(WPB * 32) prolong_lattice(LatArgs<T> A) {
   }
   __syncwarp();
   if (m & MASK_HANG) {  // C^(c) (uniform over the warp)
-    lattice_hang<K, 0>(lat, m, lane);
+    lattice_hang<K, 0, false>(lat, m, lane);
     __syncwarp();
-    lattice_hang<K, 1>(lat, m, lane);
+    lattice_hang<K, 1, false>(lat, m, lane);
     __syncwarp();
-    lattice_hang<K, 2>(lat, m, lane);
+    lattice_hang<K, 2, false>(lat, m, lane);
     __syncwarp();
   }
   if (ent[L::ES - 1] > 0) {
@@ -528,6 +528,108 @@ __global__ void __launch_bounds__(WPB * 32) prolong_lattice(LatArgs<T> A) {
       const int32_t g = ent[p & 127];
       if (n < N3 && g >= 0) atomicAdd(A.dst + g + (int)((p >> 7) & 31), lat[p >> 12]);
     }
+  }
+}
+
+// restriction onto a level of few cells: the coarse cell's result to its cell
+// vector (kernels_small.cu adds them up)
+template <int K, typename T>
+__global__ void __launch_bounds__(WPB * 32) restrict_cells(LatArgs<T> A) {
+  using L = Lat<K>;
+  constexpr int N = L::N, N3 = L::N3, M = L::M, M2 = L::M2;
+  constexpr int NT = WPB * 32;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  T* lat = reinterpret_cast<T*>(smem) + w * L::LS;
+  uint32_t* s_pt = reinterpret_cast<uint32_t*>(smem + (size_t)WPB * L::LS * sizeof(T));
+  uint32_t* s_nd = s_pt + L::NI * 32;
+  int32_t* ent = reinterpret_cast<int32_t*>(s_nd + L::NJ * 32) + w * (L::ES + 32);
+  const int c = blockIdx.x * WPB + w;
+  for (int i = threadIdx.x; i < L::NI * 32; i += NT) cp_async(s_pt + i, &g_lat.pt[K][i]);
+  for (int i = threadIdx.x; i < L::NJ * 32; i += NT) cp_async(s_nd + i, &g_lat.nd[K][i]);
+  uint16_t m = 0;
+  if (c < A.n_coarse) {
+#pragma unroll
+    for (int i = 0; i < L::EPL; ++i) cp_async(ent + lane + 32 * i, A.ent + (size_t)c * L::ES + lane + 32 * i);
+    m = A.mask_c[c];
+  }
+  cp_async_wait_all();
+  pdl_wait();
+  __syncthreads();
+  if (c >= A.n_coarse) return;
+  const T* __restrict__ src = A.src;
+  const T* __restrict__ rhs = A.rhs;
+  if (ent[L::ES - 1] > 0) {
+    T v[L::NI];
+#pragma unroll
+    for (int i = 0; i < L::NI; ++i) {
+      const uint32_t p = s_pt[lane + 32 * i];
+      const int32_t g = ent[p & 127];
+      v[i] = T(0);
+      if (g >= 0) {
+        const int gi = g + (int)((p >> 7) & 31);
+        v[i] = rhs ? rhs[gi] - src[gi] : src[gi];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < L::NI; ++i) lat[s_pt[lane + 32 * i] >> 12] = v[i];
+    __syncwarp();
+#pragma unroll 1
+    for (int q = lane; q < M2; q += 32) {  // z-lines
+      T x[M];
+#pragma unroll
+      for (int i = 0; i < M; ++i) x[i] = lat[q + M2 * i];
+      line_restrict<K>(x);
+#pragma unroll
+      for (int i = 0; i < N; ++i) lat[q + M2 * i] = x[i];
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int q = lane; q < M * N; q += 32) {  // y-lines (x, c)
+      T* p = lat + q % M + M2 * (q / M);
+      T x[M];
+#pragma unroll
+      for (int i = 0; i < M; ++i) x[i] = p[M * i];
+      line_restrict<K>(x);
+#pragma unroll
+      for (int i = 0; i < N; ++i) p[M * i] = x[i];
+    }
+    __syncwarp();
+    if (lane < N * N) {  // x-lines (b, c)
+      T* p = lat + M * (lane % N) + M2 * (lane / N);
+      T x[M];
+#pragma unroll
+      for (int i = 0; i < M; ++i) x[i] = p[i];
+      line_restrict<K>(x);
+#pragma unroll
+      for (int i = 0; i < N; ++i) p[i] = x[i];
+    }
+  } else {  // identity category (no fine cells: no owned slots, zeros)
+#pragma unroll
+    for (int i = 0; i < L::NJ; ++i) {
+      const uint32_t p = s_nd[lane + 32 * i];
+      const int32_t g = ent[p & 127];
+      T v = T(0);
+      if (g >= 0) {
+        const int gi = g + (int)((p >> 7) & 31);
+        v = rhs ? rhs[gi] - src[gi] : src[gi];
+      }
+      lat[p >> 12] = v;
+    }
+  }
+  __syncwarp();
+  if (m & MASK_HANG) {  // C^(c)T
+    lattice_hang<K, 2, true>(lat, m, lane);
+    __syncwarp();
+    lattice_hang<K, 1, true>(lat, m, lane);
+    __syncwarp();
+    lattice_hang<K, 0, true>(lat, m, lane);
+    __syncwarp();
+  }
+#pragma unroll
+  for (int i = 0; i < L::NJ; ++i) {
+    const int n = lane + 32 * i;
+    if (n < N3) A.dst[(size_t)c * N3 + n] = lat[s_nd[n] >> 12];
   }
 }
 
@@ -663,6 +765,25 @@ void run_restrict(const TransferLaunch& L, const T* src, T* dst, const T* rhs, b
   launch_halo_add(L.coarse, sizeof(T) == 8, dst, s);
 }
 
+template <int K, typename T>
+void run_restrict_cells(const TransferLaunch& L, const T* src, const T* rhs, cudaStream_t s) {
+  LatArgs<T> A = lat_args(L, src, static_cast<T*>(L.coarse.cell_vec));
+  A.rhs = rhs;
+  smem_allow(restrict_cells<K, T>, prolong_smem<K, T>());
+  launch_pdl(restrict_cells<K, T>, (L.n_coarse + WPB - 1) / WPB, WPB * 32, prolong_smem<K, T>(), s, A);
+  note_launches(1);
+}
+
+template <typename T>
+void restrict_cells_any(const TransferLaunch& L, const T* src, const T* rhs, cudaStream_t s) {
+  switch (L.kf) {
+    case 1: run_restrict_cells<1>(L, src, rhs, s); break;
+    case 2: run_restrict_cells<2>(L, src, rhs, s); break;
+    case 3: run_restrict_cells<3>(L, src, rhs, s); break;
+    case 4: run_restrict_cells<4>(L, src, rhs, s); break;
+  }
+}
+
 template <typename T>
 void prolong_any(const TransferLaunch& L, const T* src, T* dst, cudaStream_t s) {
   switch (L.kf) {
@@ -723,6 +844,13 @@ void launch_prolong_lattice(const TransferLaunch& L, bool fp64, const void* coar
     prolong_any(L, static_cast<const double*>(coarse), static_cast<double*>(fine), s);
   else
     prolong_any(L, static_cast<const float*>(coarse), static_cast<float*>(fine), s);
+}
+
+void launch_restrict_cells(const TransferLaunch& L, bool fp64, const void* fine, const void* rhs, cudaStream_t s) {
+  if (fp64)
+    restrict_cells_any(L, static_cast<const double*>(fine), static_cast<const double*>(rhs), s);
+  else
+    restrict_cells_any(L, static_cast<const float*>(fine), static_cast<const float*>(rhs), s);
 }
 
 void launch_restrict_lattice(const TransferLaunch& L, bool fp64, const void* fine, const void* rhs, void* coarse,

@@ -97,6 +97,57 @@ __device__ __forceinline__ df df_dot(const df* x, const float* ch, const float* 
   return df_norm(S, L);
 }
 
+// even-odd forward transform with B (nodal -> modes in mode order) and its
+// backward transform, in double-float, rows as df_dot
+template <int K>
+__device__ __forceinline__ void df_eo_fwd_fast(df* u) {
+  constexpr int N = K + 1, NH = N / 2, NE = (N + 1) / 2;
+  const float(&Bh)[NMAX][NMAX] = c_tf[K].Be;
+  const float(&Bl)[NMAX][NMAX] = c_tflo[K].Be;
+  df e[NE], o[NH > 0 ? NH : 1];
+#pragma unroll
+  for (int j = 0; j < NH; ++j) {
+    e[j] = df_add(u[j], u[N - 1 - j]);
+    o[j] = df_sub(u[j], u[N - 1 - j]);
+  }
+  if (N % 2) e[NH] = u[NH];
+#pragma unroll
+  for (int r = 0; r < NE; ++r) u[r] = df_dot<NE>(e, Bh[r], Bl[r]);
+#pragma unroll
+  for (int r = 0; r < NH; ++r) u[NE + r] = df_dot<NH>(o, Bh[NE + r], Bl[NE + r]);
+}
+
+template <int K>
+__device__ __forceinline__ void df_eo_bwd_fast(df* u) {
+  constexpr int N = K + 1, NH = N / 2, NE = (N + 1) / 2;
+  df E[NE], O[NH > 0 ? NH : 1];
+  float ch[NMAX], cl[NMAX];
+#pragma unroll
+  for (int j = 0; j < NE; ++j) {
+#pragma unroll
+    for (int r = 0; r < NE; ++r) {
+      ch[r] = c_tf[K].Be[r][j];
+      cl[r] = c_tflo[K].Be[r][j];
+    }
+    E[j] = df_dot<NE>(u, ch, cl);
+  }
+#pragma unroll
+  for (int j = 0; j < NH; ++j) {
+#pragma unroll
+    for (int r = 0; r < NH; ++r) {
+      ch[r] = c_tf[K].Be[NE + r][j];
+      cl[r] = c_tflo[K].Be[NE + r][j];
+    }
+    O[j] = df_dot<NH>(u + NE, ch, cl);
+  }
+#pragma unroll
+  for (int j = 0; j < NH; ++j) {
+    u[j] = df_add(E[j], O[j]);
+    u[N - 1 - j] = df_sub(E[j], O[j]);
+  }
+  if (N % 2) u[NH] = E[NH];
+}
+
 // I_p (TRANS: transposed) on one df line, by the mirror identity of interp_line_reg
 template <int K, bool TRANS>
 __device__ __forceinline__ void interp_line_df(df* v, int p) {
