@@ -424,81 +424,29 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 8 : 1) vmult_lanes(Lane
 // wider than its FP64 pipe.  Values are converted once on entry to and once
 // on exit from the tile; the cell buffer and the accumulator hold df pairs.
 // ---------------------------------------------------------------------------
-template <int K, int D, bool TRANS, bool SWEEP = false>
-__device__ __forceinline__ void hang_pass_df(df* cb, uint16_t m, uint32_t hlD, int w, int lane) {
-  constexpr int N = K + 1, N2 = N * N;
-  constexpr int S = (D == 0 ? 1 : (D == 1 ? N : N2)) * 32;
-  const int p = (m >> D) & 1;
-#pragma unroll 1
-  for (int i = 0; i < N; ++i) {
-    const int u = i, v = w;  // line (u, v): the other two coordinates
-    const bool hl = (hlD >> (u + N * v)) & 1u;
-    if (!SWEEP && !hl) continue;
-    const int base = D == 0 ? N * u + N2 * v : (D == 1 ? u + N2 * v : u + N * v);
-    df* ptr = cb + base * 32 + lane;
-    df x[N];
-#pragma unroll
-    for (int a = 0; a < N; ++a) x[a] = ptr[a * S];
-    if (SWEEP && TRANS) df_eo_bwd_fast<K>(x);
-    if (hl) interp_line_df<K, TRANS>(x, p);
-    if (SWEEP && !TRANS) df_eo_fwd_fast<K>(x);
-#pragma unroll
-    for (int a = 0; a < N; ++a) ptr[a * S] = x[a];
-  }
-}
-
-template <int K, bool FWD>
-__device__ __forceinline__ void sweep_y_df(df* cb, int w, int lane) {
-  constexpr int N = K + 1, N2 = N * N;
-#pragma unroll 1
-  for (int i = 0; i < N; ++i) {
-    df* p = cb + (i + N2 * w) * 32 + lane;
-    df v[N];
-#pragma unroll
-    for (int b = 0; b < N; ++b) v[b] = p[b * N * 32];
-    if (FWD)
-      df_eo_fwd_fast<K>(v);
-    else
-      df_eo_bwd_fast<K>(v);
-#pragma unroll
-    for (int b = 0; b < N; ++b) p[b * N * 32] = v[b];
-  }
-}
-
-// forward sweep, h (lam_a + lam_b + lam_c) in mode order, backward sweep on the
-// lines along direction D (2: z-lines (a, b) = (i, w); 0: x-lines (b, c) = (i, w))
-template <int K, int D>
-__device__ __forceinline__ void sweep_scale_df(df* cb, int w, int lane, df h) {
-  constexpr int N = K + 1, N2 = N * N;
-  constexpr int S = (D == 0 ? 1 : N2) * 32;
-#pragma unroll 1
-  for (int i = 0; i < N; ++i) {
-    df* p = cb + (D == 0 ? N * (i + N * w) : i + N * w) * 32 + lane;
-    df v[N];
-#pragma unroll
-    for (int c = 0; c < N; ++c) v[c] = p[c * S];
-    df_eo_fwd_fast<K>(v);
-#pragma unroll
-    for (int c = 0; c < N; ++c) {
-      // mode index of the node: along D the line index c, the others (i, w)
-      const int idx = D == 0 ? c + N * i + N2 * w : i + N * w + N2 * c;
-      v[c] = df_mul(v[c], df_mul(df{c_tf[K].lam3[idx], c_tflo[K].lam3[idx]}, h));
-    }
-    df_eo_bwd_fast<K>(v);
-#pragma unroll
-    for (int c = 0; c < N; ++c) p[c * S] = v[c];
-  }
-}
+// The passes over the 1D lines as one loop, so that each transform is one piece
+// of code: written out pass by pass, the kernel's instructions did not fit the
+// instruction caches (the largest stall was "no instruction", 57 % issue
+// active).  A pass takes the lines along direction D through, in this order,
+// C_e, the forward transform, the scaling, the backward transform, C_e^T.
+enum : uint8_t { DF_C = 4, DF_FWD = 8, DF_SCALE = 16, DF_BWD = 32, DF_CT = 64 };  // bits 0-1: D
+__constant__ uint8_t c_df_pass[2][9] = {
+    // tiles without hanging cells: x, y forward, z, y, x backward
+    {0 | DF_FWD, 1 | DF_FWD, 2 | DF_FWD | DF_SCALE | DF_BWD, 1 | DF_BWD, 0 | DF_BWD, 0, 0, 0, 0},
+    // with hanging cells: C_x, C_y, C_z and the sweeps in the order z, y, x, and back
+    {0 | DF_C, 1 | DF_C, 2 | DF_C | DF_FWD, 1 | DF_FWD, 0 | DF_FWD | DF_SCALE | DF_BWD, 1 | DF_BWD, 2 | DF_BWD | DF_CT,
+     1 | DF_CT, 0 | DF_CT}};
 
 template <int K>
-__global__ void __launch_bounds__((K + 1) * 32) vmult_lanes_df(LaneArgsT<double> A) {
-  pdl_begin();
-  constexpr int N = K + 1, N3 = N * N * N, NT = N * 32;
+__global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(LaneArgsT<double> A) {
+  constexpr int N = K + 1, N2 = N * N, NT = N * 32;
   extern __shared__ __align__(16) unsigned char smem[];
   LaneTile* st = reinterpret_cast<LaneTile*>(smem);
   LaneHang* hg = reinterpret_cast<LaneHang*>(smem + sizeof(LaneTile));
+  // the cell buffer and the tile's DoF buffer (input, then accumulator) share one region, as in
+  // vmult_lanes: 6 instead of 4 blocks per SM at k = 4
   df* cb = reinterpret_cast<df*>(smem + sizeof(LaneTile) + sizeof(LaneHang));
-  double* xd0 = reinterpret_cast<double*>(cb + N3 * 32);  // 16-byte aligned
+  double* xd0 = reinterpret_cast<double*>(cb);  // 16-byte aligned
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   // block b's tile: records in launch order at [b] (no dependent load of the tile index) or tile0 + b
   const int bx = blockIdx.x, tl = A.tile0 + bx;
@@ -506,12 +454,6 @@ __global__ void __launch_bounds__((K + 1) * 32) vmult_lanes_df(LaneArgsT<double>
   const LaneHang* lhp = A.order ? A.lh_lo + bx : A.lh + tl;
   const TileInfo ti = A.order ? A.tiles_lo[bx] : A.tiles[tl];
   const int nloc = ti.n_owned + ti.n_foreign;
-  // tile DoF i at xd[i] (fp64 on arrival, then df in place; the zero region after it)
-  const double* so = A.src + ti.dof_begin;
-  const int sh = (int)((reinterpret_cast<uintptr_t>(so) >> 3) & 1);
-  double* xd = xd0 + sh;
-  df* xs = reinterpret_cast<df*>(xd);
-  const int h0 = min(sh, ti.n_owned), nv = (ti.n_owned - h0) >> 1;
   {
     const uint4* g = reinterpret_cast<const uint4*>(ltp);
     uint4* s = reinterpret_cast<uint4*>(st);
@@ -521,6 +463,15 @@ __global__ void __launch_bounds__((K + 1) * 32) vmult_lanes_df(LaneArgsT<double>
       uint4* shh = reinterpret_cast<uint4*>(hg);
       for (int i = threadIdx.x; i < (int)(sizeof(LaneHang) / 16); i += NT) cp_async16(shh + i, gh + i);
     }
+  }
+  pdl_wait();
+  // tile DoF i at xd[i] (fp64 on arrival, then df in place; the zero region after it)
+  const double* so = A.src + ti.dof_begin;
+  const int sh = (int)((reinterpret_cast<uintptr_t>(so) >> 3) & 1);
+  double* xd = xd0 + sh;
+  df* xs = reinterpret_cast<df*>(xd);
+  const int h0 = min(sh, ti.n_owned), nv = (ti.n_owned - h0) >> 1;
+  {
     if (threadIdx.x < h0) cp_async(xd + threadIdx.x, so + threadIdx.x);
 #pragma unroll 4
     for (int j = threadIdx.x; j < nv; j += NT) cp_async16(xd + h0 + 2 * j, so + h0 + 2 * j);
@@ -549,89 +500,97 @@ __global__ void __launch_bounds__((K + 1) * 32) vmult_lanes_df(LaneArgsT<double>
     h = df_from(A.coef ? hd * A.coef[c] : hd);
   }
   char* xb = reinterpret_cast<char*>(xs);
-  const int nxl = c_ll.nx[K][w];
   __syncthreads();
-
-  // G_e (+ C_x on hanging tiles, else the forward x sweep)
+  {  // G_e: the x-lines (b, c) = (i, w), all gathered before the cell buffer is written
+    df v[N][N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const uint32_t li = c_ll.line[K][i + N * w];
+      const int s0 = li & 0xff, o0 = (li >> 8) & 0xff, o1 = li >> 16;
+      const df* p0 = reinterpret_cast<const df*>(xb + 2 * (st->ls[s0][lane] + o0));
+      const df* p1 = reinterpret_cast<const df*>(xb + 2 * (st->ls[s0 + 1][lane] + o1));
+      const df* p2 = reinterpret_cast<const df*>(xb + 2 * (st->ls[s0 + 2][lane] + o0));
+      v[i][0] = *p0;
+#pragma unroll
+      for (int a = 1; a < K; ++a) v[i][a] = p1[a - 1];
+      v[i][K] = *p2;
+    }
+    __syncthreads();  // the DoF buffer is dead
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+      for (int a = 0; a < N; ++a) cb[(N * (i + N * w) + a) * 32 + lane] = v[i][a];
+  }
+  // the first pass takes the warp's own lines
+  const int npass = hang ? 9 : 5;
 #pragma unroll 1
-  for (int i = 0; i < nxl; ++i) {
-    const int r = c_ll.xw[K][w][i];
-    const uint32_t li = c_ll.line[K][r];
-    const int s0 = li & 0xff, o0 = (li >> 8) & 0xff, o1 = li >> 16;
-    const df* p0 = reinterpret_cast<const df*>(xb + 2 * (st->ls[s0][lane] + o0));
-    const df* p1 = reinterpret_cast<const df*>(xb + 2 * (st->ls[s0 + 1][lane] + o1));
-    const df* p2 = reinterpret_cast<const df*>(xb + 2 * (st->ls[s0 + 2][lane] + o0));
-    df v[N];
-    v[0] = *p0;
-#pragma unroll
-    for (int a = 1; a < K; ++a) v[a] = p1[a - 1];
-    v[K] = *p2;
-    if (!hang)
-      df_eo_fwd_fast<K>(v);
-    else if ((hg->hl[0][lane] >> r) & 1u)
-      interp_line_df<K, false>(v, m & 1);
-    df* p = cb + N * r * 32 + lane;
-#pragma unroll
-    for (int a = 0; a < N; ++a) p[a * 32] = v[a];
-  }
-  __syncthreads();
-  if (hang) {
-    hang_pass_df<K, 1, false>(cb, m, hg->hl[1][lane], w, lane);  // C_y
-    __syncthreads();
-    hang_pass_df<K, 2, false, true>(cb, m, hg->hl[2][lane], w, lane);  // C_z, forward z sweep
-    __syncthreads();
-  }
-  {  // the tile DoFs are dead: clear the accumulator
-    float4* z4 = reinterpret_cast<float4*>(xd0);
-    for (int i = threadIdx.x; i < (sh + nloc + 1) / 2; i += NT) z4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  sweep_y_df<K, true>(cb, w, lane);
-  __syncthreads();
-  if (!hang)
-    sweep_scale_df<K, 2>(cb, w, lane, h);
-  else
-    sweep_scale_df<K, 0>(cb, w, lane, h);
-  __syncthreads();
-  sweep_y_df<K, false>(cb, w, lane);
-  __syncthreads();
-  if (hang) {
-    hang_pass_df<K, 2, true, true>(cb, m, hg->hl[2][lane], w, lane);  // backward z sweep, C_z^T
-    __syncthreads();
-    hang_pass_df<K, 1, true>(cb, m, hg->hl[1][lane], w, lane);  // C_y^T
-    __syncthreads();
-  }
-  // backward x sweep (tiles without hanging cells) or C_x^T, then G_e^T on the warp's class of x-lines
-  const uint32_t hs = hang ? hg->hs[lane] : 0u;
-  const int zb = nloc * 4;
+  for (int ps = 0; ps < npass; ++ps) {
+    const int f = c_df_pass[hang][ps], D = f & 3;
+    const int S = D == 0 ? 1 : (D == 1 ? N : N2);
+    const int b0 = D == 0 ? N2 * w : (D == 1 ? N2 * w : N * w), bs = D == 0 ? N : 1;  // line i at b0 + bs i
+    const uint32_t hl = (f & (DF_C | DF_CT)) ? hg->hl[D][lane] >> (N * w) : 0u;
+    const int p = (m >> D) & 1;
 #pragma unroll 1
-  for (int i = 0; i < nxl; ++i) {
-    const int r = c_ll.xw[K][w][i];
-    const df* p = cb + N * r * 32 + lane;
-    df v[N];
+    for (int i = 0; i < N; ++i) {
+      const bool on = (hl >> i) & 1u;
+      // a pass of C_e or C_e^T alone touches the hanging lines only
+      if (!(f & (DF_FWD | DF_BWD)) && !on) continue;
+      const int q = b0 + bs * i;
+      df* ptr = cb + q * 32 + lane;
+      df v[N];
 #pragma unroll
-    for (int a = 0; a < N; ++a) v[a] = p[a * 32];
-    if (!hang)
-      df_eo_bwd_fast<K>(v);
-    else if ((hg->hl[0][lane] >> r) & 1u)
-      interp_line_df<K, true>(v, m & 1);
-    const uint32_t li = c_ll.line[K][r];
-    const int s0 = li & 0xff, o0 = (li >> 8) & 0xff, o1 = li >> 16;
-    const int b0 = st->ls[s0][lane], b1 = st->ls[s0 + 1][lane], b2 = st->ls[s0 + 2][lane];
-    df* q0 = reinterpret_cast<df*>(xb + 2 * (b0 + o0));
-    df* q1 = reinterpret_cast<df*>(xb + 2 * (b1 + o1));
-    df* q2 = reinterpret_cast<df*>(xb + 2 * (b2 + o0));
-    if (!hang) {
-      *q0 = df_add(*q0, v[0]);
+      for (int a = 0; a < N; ++a) v[a] = ptr[a * S * 32];
+      if ((f & DF_C) && on) interp_line_df<K, false>(v, p);
+      if (f & DF_FWD) df_eo_fwd_fast<K>(v);
+      if (f & DF_SCALE) {  // h (lam_a + lam_b + lam_c) in mode order
 #pragma unroll
-      for (int a = 1; a < K; ++a) q1[a - 1] = df_add(q1[a - 1], v[a]);
-      *q2 = df_add(*q2, v[K]);
-    } else {
-      const bool g0 = __any_sync(0xffffffffu, (hs >> s0) & 1u), g1 = __any_sync(0xffffffffu, (hs >> (s0 + 1)) & 1u),
-                 g2 = __any_sync(0xffffffffu, (hs >> (s0 + 2)) & 1u);
-      add_ordered_df(q0, v[0], b0 != zb, lane, g0);
+        for (int c = 0; c < N; ++c)
+          v[c] = df_mul(v[c], df_mul(df{c_tf[K].lam3[q + c * S], c_tflo[K].lam3[q + c * S]}, h));
+      }
+      if (f & DF_BWD) df_eo_bwd_fast<K>(v);
+      if ((f & DF_CT) && on) interp_line_df<K, true>(v, p);
 #pragma unroll
-      for (int a = 1; a < K; ++a) add_ordered_df(q1 + a - 1, v[a], b1 != zb, lane, g1);
-      add_ordered_df(q2, v[K], b2 != zb, lane, g2);
+      for (int a = 0; a < N; ++a) ptr[a * S * 32] = v[a];
+    }
+    __syncthreads();
+  }
+  // G_e^T on the warp's class of x-lines: all lines read before the accumulator (the same
+  // region) is cleared
+  {
+    constexpr int NXW = K <= 2 ? 4 : N;  // x-lines per warp at most
+    const int nxl = c_ll.nx[K][w];
+    df v[NXW][N];
+#pragma unroll
+    for (int i = 0; i < NXW; ++i)
+      if (i < nxl) {
+        const df* p = cb + N * c_ll.xw[K][w][i] * 32 + lane;
+#pragma unroll
+        for (int a = 0; a < N; ++a) v[i][a] = p[a * 32];
+      }
+    __syncthreads();  // the cell buffer is dead
+    {
+      float4* z4 = reinterpret_cast<float4*>(xd0);
+      for (int i = threadIdx.x; i < (sh + nloc + 1) / 2; i += NT) z4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    const uint32_t hs = hang ? hg->hs[lane] : 0u;
+    const int zb = nloc * 4;
+#pragma unroll
+    for (int i = 0; i < NXW; ++i) {
+      if (i >= nxl) break;
+      const uint32_t li = c_ll.line[K][c_ll.xw[K][w][i]];
+      const int s0 = li & 0xff, o0 = (li >> 8) & 0xff, o1 = li >> 16;
+      const int b0 = st->ls[s0][lane], b1 = st->ls[s0 + 1][lane], b2 = st->ls[s0 + 2][lane];
+      df* q0 = reinterpret_cast<df*>(xb + 2 * (b0 + o0));
+      df* q1 = reinterpret_cast<df*>(xb + 2 * (b1 + o1));
+      df* q2 = reinterpret_cast<df*>(xb + 2 * (b2 + o0));
+      const bool g0 = hang && __any_sync(0xffffffffu, (hs >> s0) & 1u),
+                 g1 = hang && __any_sync(0xffffffffu, (hs >> (s0 + 1)) & 1u),
+                 g2 = hang && __any_sync(0xffffffffu, (hs >> (s0 + 2)) & 1u);
+      add_ordered_df(q0, v[i][0], b0 != zb, lane, g0);
+#pragma unroll
+      for (int a = 1; a < K; ++a) add_ordered_df(q1 + a - 1, v[i][a], b1 != zb, lane, g1);
+      add_ordered_df(q2, v[i][K], b2 != zb, lane, g2);
     }
   }
   __syncthreads();
@@ -656,7 +615,9 @@ size_t lanes_smem(int max_local) {
 template <int K>
 size_t lanes_df_smem(int max_local) {
   constexpr int N3 = (K + 1) * (K + 1) * (K + 1);
-  return sizeof(LaneTile) + sizeof(LaneHang) + ((size_t)N3 * 32 + (size_t)max_local + LANE_ZERO + 4) * sizeof(double);
+  // one region for the cell buffer and the tile DoFs, as in lanes_smem
+  return sizeof(LaneTile) + sizeof(LaneHang) +
+         std::max((size_t)N3 * 32, (size_t)max_local + LANE_ZERO + 4) * sizeof(double);
 }
 
 template <int K>

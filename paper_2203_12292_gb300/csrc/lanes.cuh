@@ -171,11 +171,8 @@ __device__ __forceinline__ void interp_line_df(df* v, int p) {
   for (int a = 0; a < N; ++a) v[a] = df_sel(p, y[K - a], y[a]);
 }
 
-__device__ __forceinline__ void add_ordered_df(df* x, df v, bool real, int lane, bool hang_any) {
-  if (!hang_any) {
-    *x = df_add(*x, v);
-    return;
-  }
+// the same in double-float
+static __device__ __noinline__ void add_ordered_df_slow(df* x, df v, bool real, int lane) {
   const unsigned key = real ? (unsigned)__cvta_generic_to_shared(x) : ~(unsigned)lane;
   const unsigned peers = __match_any_sync(0xffffffffu, key);
   const int rank = __popc(peers & ((1u << lane) - 1u));
@@ -184,6 +181,13 @@ __device__ __forceinline__ void add_ordered_df(df* x, df v, bool real, int lane,
     if (real && rank == q) *x = df_add(*x, v);
     __syncwarp();
   }
+}
+
+__device__ __forceinline__ void add_ordered_df(df* x, df v, bool real, int lane, bool hang_any) {
+  if (!hang_any)
+    *x = df_add(*x, v);
+  else
+    add_ordered_df_slow(x, v, real, lane);
 }
 
 // host: entity slot and offset of local node (a, b, c) of a degree-k cell
