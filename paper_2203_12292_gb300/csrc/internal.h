@@ -55,12 +55,16 @@ struct LaneTile {
 static_assert(sizeof(LaneTile) % 64 == 0, "LaneTile is copied in 16-byte pieces");
 // per tile, for the tiles with hanging cells: per lane the lines of its cell
 // on a hanging face or edge, one set per direction D (bit u + (k+1) v for the
-// line through the other two coordinates (u, v), in increasing axis order),
-// and the 27-bit set of its slots on a hanging face or edge
+// line through the other two coordinates (u, v), in increasing axis order), and
+// per slot the lane's rank, in lane order, among the lanes whose slot starts at
+// the same DoF (siblings behind one coarse face or edge) and the largest number
+// of such lanes
 struct LaneHang {
   uint32_t hl[3][32];
-  uint32_t hs[32];
+  uint8_t rank[NSLOT][32];
+  uint8_t most[32];
 };
+static_assert(sizeof(LaneHang) % 16 == 0, "LaneHang is copied in 16-byte pieces");
 
 struct TileInfo {
   int32_t cell_begin;

@@ -35,8 +35,8 @@
 //     (b, c) are grouped into classes by (b or "boundary", c or "boundary");
 //     each class is given to one warp, so two warps never add to the same
 //     DoF.  Within one instruction two lanes add to the same DoF only through
-//     hanging slots (siblings behind one coarse face or edge), added one lane
-//     after another in lane order.  These tiles apply C_e and C_e^T (Sec. 3.2,
+//     hanging slots (siblings behind one coarse face or edge); they take turns
+//     in lane order, with ranks from the set-up (LaneHang).  These tiles apply C_e and C_e^T (Sec. 3.2,
 //     direction by direction) between separate passes.
 // The sums are therefore reproducible bit for bit.
 #include <algorithm>
@@ -73,11 +73,17 @@ struct LaneArgsT {
 };
 using LaneArgs = LaneArgsT<float>;
 
-// one direction D of C_e (TRANS: C_e^T) on the lines of warp w: line
-// q = i + N w has the other coordinates (u, v) = (q % N, q / N) in increasing
-// axis order; lane j interpolates when the line lies on a hanging face or edge
-// of its cell.  SWEEP (D = 2 only): the z sweep follows (forward after C_z) or
-// precedes (backward before C_z^T) the interpolation on the same lines.
+// base node of line q = u + N v along D
+template <int K, int D>
+__device__ __forceinline__ int line_base(int q) {
+  constexpr int N = K + 1, N2 = N * N;
+  return D == 0 ? N * q : (D == 1 ? q % N + N2 * (q / N) : q);
+}
+
+// one direction D of C_e (TRANS: C_e^T) on the lines of warp w; lane j
+// interpolates when the line lies on a hanging face or edge of its cell.  SWEEP
+// (D = 2 only): the z sweep follows (forward after C_z) or precedes (backward
+// before C_z^T) the interpolation on the same lines.
 template <int K, int D, bool TRANS, bool SWEEP = false>
 __device__ __forceinline__ void hang_pass(float* cb, uint16_t m, uint32_t hlD, int w, int lane) {
   constexpr int N = K + 1, N2 = N * N;
@@ -86,11 +92,10 @@ __device__ __forceinline__ void hang_pass(float* cb, uint16_t m, uint32_t hlD, i
   const int p = (m >> D) & 1;
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    const int u = i, v = w;  // line (u, v): the other two coordinates
-    const bool hl = (hlD >> (u + N * v)) & 1u;
+    const int q = c_ll.bl[K][w][i];
+    const bool hl = (hlD >> q) & 1u;
     if (!SWEEP && !hl) continue;
-    const int base = D == 0 ? N * u + N2 * v : (D == 1 ? u + N2 * v : u + N * v);
-    float* ptr = cb + base * 32 + lane;
+    float* ptr = cb + line_base<K, D>(q) * 32 + lane;
     float x[N];
 #pragma unroll
     for (int a = 0; a < N; ++a) x[a] = ptr[a * S];
@@ -151,7 +156,7 @@ __device__ __forceinline__ void sweep_y(float* cb, int w, int lane) {
 template <int K>
 __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 8 : 1) vmult_lanes(LaneArgs A) {
   pdl_begin();
-  constexpr int N = K + 1, N2 = N * N, N3 = N2 * N, NT = N * 32;
+  constexpr int N = K + 1, N2 = N * N, NT = N * 32;
   extern __shared__ __align__(16) unsigned char smem[];
   LaneTile* st = reinterpret_cast<LaneTile*>(smem);
   LaneHang* hg = reinterpret_cast<LaneHang*>(smem + sizeof(LaneTile));
@@ -304,29 +309,27 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 8 : 1) vmult_lanes(Lane
     }
     if (w == 0) named_bar_arrive(1, 64);
   } else {
-    // G_e and C_x on the warp's x-lines, all gathered before the cell buffer is written
-    constexpr int NXW = K <= 2 ? 4 : N;  // x-lines per warp at most
+    // G_e and C_x on the warp's lines, all gathered before the cell buffer is written
+    constexpr int NXW = K <= 2 ? 4 : N;  // x-lines per warp at most (its class in the scatter)
     float v[NXW][N];
 #pragma unroll
-    for (int i = 0; i < NXW; ++i)
-      if (i < nxl) {
-        const int r = c_ll.xw[K][w][i];
-        float *p0, *p1, *p2;
-        xline_ptrs<K>(st, xb, r, lane, p0, p1, p2);
-        v[i][0] = *p0;
+    for (int i = 0; i < N; ++i) {
+      const int r = c_ll.bl[K][w][i];
+      float *p0, *p1, *p2;
+      xline_ptrs<K>(st, xb, r, lane, p0, p1, p2);
+      v[i][0] = *p0;
 #pragma unroll
-        for (int a = 1; a < K; ++a) v[i][a] = p1[a - 1];
-        v[i][K] = *p2;
-        if ((hg->hl[0][lane] >> r) & 1u) interp_line_reg<K, false>(v[i], m & 1);
-      }
+      for (int a = 1; a < K; ++a) v[i][a] = p1[a - 1];
+      v[i][K] = *p2;
+      if ((hg->hl[0][lane] >> r) & 1u) interp_line_reg<K, false>(v[i], m & 1);
+    }
     __syncthreads();  // the DoF buffer is dead
 #pragma unroll
-    for (int i = 0; i < NXW; ++i)
-      if (i < nxl) {
-        float* p = cb + N * c_ll.xw[K][w][i] * 32 + lane;
+    for (int i = 0; i < N; ++i) {
+      float* p = cb + N * c_ll.bl[K][w][i] * 32 + lane;
 #pragma unroll
-        for (int a = 0; a < N; ++a) p[a * 32] = v[i][a];
-      }
+      for (int a = 0; a < N; ++a) p[a * 32] = v[i][a];
+    }
     __syncthreads();
     hang_pass<K, 1, false>(cb, m, hg->hl[1][lane], w, lane);  // C_y
     __syncthreads();
@@ -371,25 +374,17 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 8 : 1) vmult_lanes(Lane
     __syncthreads();  // the cell buffer is dead
     clear_acc(xs0, sh + nloc, NT);
     __syncthreads();
-    const uint32_t hs = hg->hs[lane];
-    const int zb = nloc * 4;  // byte offset of the zero region
 #pragma unroll
     for (int i = 0; i < NXW; ++i) {
       if (i >= nxl) break;
       const int r = c_ll.xw[K][w][i];
       if ((hg->hl[0][lane] >> r) & 1u) interp_line_reg<K, true>(v[i], m & 1);
-      const uint32_t li = c_ll.line[K][r];
-      const int s0 = li & 0xff, o0 = (li >> 8) & 0xff, o1 = li >> 16;
-      const int b0 = st->ls[s0][lane], b1 = st->ls[s0 + 1][lane], b2 = st->ls[s0 + 2][lane];
-      float* p0 = reinterpret_cast<float*>(xb + b0 + o0);
-      float* p1 = reinterpret_cast<float*>(xb + b1 + o1);
-      float* p2 = reinterpret_cast<float*>(xb + b2 + o0);
-      const bool h0 = __any_sync(0xffffffffu, (hs >> s0) & 1u), h1 = __any_sync(0xffffffffu, (hs >> (s0 + 1)) & 1u),
-                 h2 = __any_sync(0xffffffffu, (hs >> (s0 + 2)) & 1u);
-      add_ordered(p0, v[i][0], b0 != zb, lane, h0);
-#pragma unroll
-      for (int a = 1; a < K; ++a) add_ordered(p1 + a - 1, v[i][a], b1 != zb, lane, h1);
-      add_ordered(p2, v[i][K], b2 != zb, lane, h2);
+      const int s0 = c_ll.line[K][r] & 0xff;
+      float *p0, *p1, *p2;
+      xline_ptrs<K>(st, xb, r, lane, p0, p1, p2);
+      add_turns<1>(p0, v[i], hg->rank[s0][lane], hg->most[s0]);
+      if constexpr (K > 1) add_turns<K - 1>(p1, v[i] + 1, hg->rank[s0 + 1][lane], hg->most[s0 + 1]);
+      add_turns<1>(p2, v[i] + K, hg->rank[s0 + 2][lane], hg->most[s0 + 2]);
     }
   }
   __syncthreads();
@@ -501,11 +496,11 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(L
   }
   char* xb = reinterpret_cast<char*>(xs);
   __syncthreads();
-  {  // G_e: the x-lines (b, c) = (i, w), all gathered before the cell buffer is written
+  {  // G_e: the warp's x-lines, all gathered before the cell buffer is written
     df v[N][N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      const uint32_t li = c_ll.line[K][i + N * w];
+      const uint32_t li = c_ll.line[K][c_ll.bl[K][w][i]];
       const int s0 = li & 0xff, o0 = (li >> 8) & 0xff, o1 = li >> 16;
       const df* p0 = reinterpret_cast<const df*>(xb + 2 * (st->ls[s0][lane] + o0));
       const df* p1 = reinterpret_cast<const df*>(xb + 2 * (st->ls[s0 + 1][lane] + o1));
@@ -519,7 +514,7 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(L
 #pragma unroll
     for (int i = 0; i < N; ++i)
 #pragma unroll
-      for (int a = 0; a < N; ++a) cb[(N * (i + N * w) + a) * 32 + lane] = v[i][a];
+      for (int a = 0; a < N; ++a) cb[(N * c_ll.bl[K][w][i] + a) * 32 + lane] = v[i][a];
   }
   // the first pass takes the warp's own lines
   const int npass = hang ? 9 : 5;
@@ -527,15 +522,15 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(L
   for (int ps = 0; ps < npass; ++ps) {
     const int f = c_df_pass[hang][ps], D = f & 3;
     const int S = D == 0 ? 1 : (D == 1 ? N : N2);
-    const int b0 = D == 0 ? N2 * w : (D == 1 ? N2 * w : N * w), bs = D == 0 ? N : 1;  // line i at b0 + bs i
-    const uint32_t hl = (f & (DF_C | DF_CT)) ? hg->hl[D][lane] >> (N * w) : 0u;
+    const uint32_t hl = (f & (DF_C | DF_CT)) ? hg->hl[D][lane] : 0u;
     const int p = (m >> D) & 1;
 #pragma unroll 1
     for (int i = 0; i < N; ++i) {
-      const bool on = (hl >> i) & 1u;
+      const int r = c_ll.bl[K][w][i];
+      const bool on = (hl >> r) & 1u;
       // a pass of C_e or C_e^T alone touches the hanging lines only
       if (!(f & (DF_FWD | DF_BWD)) && !on) continue;
-      const int q = b0 + bs * i;
+      const int q = D == 0 ? N * r : (D == 1 ? r % N + N2 * (r / N) : r);
       df* ptr = cb + q * 32 + lane;
       df v[N];
 #pragma unroll
@@ -573,24 +568,18 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(L
       for (int i = threadIdx.x; i < (sh + nloc + 1) / 2; i += NT) z4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
-    const uint32_t hs = hang ? hg->hs[lane] : 0u;
-    const int zb = nloc * 4;
 #pragma unroll
     for (int i = 0; i < NXW; ++i) {
       if (i >= nxl) break;
       const uint32_t li = c_ll.line[K][c_ll.xw[K][w][i]];
       const int s0 = li & 0xff, o0 = (li >> 8) & 0xff, o1 = li >> 16;
-      const int b0 = st->ls[s0][lane], b1 = st->ls[s0 + 1][lane], b2 = st->ls[s0 + 2][lane];
-      df* q0 = reinterpret_cast<df*>(xb + 2 * (b0 + o0));
-      df* q1 = reinterpret_cast<df*>(xb + 2 * (b1 + o1));
-      df* q2 = reinterpret_cast<df*>(xb + 2 * (b2 + o0));
-      const bool g0 = hang && __any_sync(0xffffffffu, (hs >> s0) & 1u),
-                 g1 = hang && __any_sync(0xffffffffu, (hs >> (s0 + 1)) & 1u),
-                 g2 = hang && __any_sync(0xffffffffu, (hs >> (s0 + 2)) & 1u);
-      add_ordered_df(q0, v[i][0], b0 != zb, lane, g0);
-#pragma unroll
-      for (int a = 1; a < K; ++a) add_ordered_df(q1 + a - 1, v[i][a], b1 != zb, lane, g1);
-      add_ordered_df(q2, v[i][K], b2 != zb, lane, g2);
+      df* q0 = reinterpret_cast<df*>(xb + 2 * (st->ls[s0][lane] + o0));
+      df* q1 = reinterpret_cast<df*>(xb + 2 * (st->ls[s0 + 1][lane] + o1));
+      df* q2 = reinterpret_cast<df*>(xb + 2 * (st->ls[s0 + 2][lane] + o0));
+      add_turns<1>(q0, v[i], hang ? hg->rank[s0][lane] : 0, hang ? hg->most[s0] : 1);
+      if constexpr (K > 1)
+        add_turns<K - 1>(q1, v[i] + 1, hang ? hg->rank[s0 + 1][lane] : 0, hang ? hg->most[s0 + 1] : 1);
+      add_turns<1>(q2, v[i] + K, hang ? hg->rank[s0 + 2][lane] : 0, hang ? hg->most[s0 + 2] : 1);
     }
   }
   __syncthreads();

@@ -175,26 +175,6 @@ __device__ __forceinline__ void interp_line(T* v, int p) {
   for (int a = 0; a < N; ++a) v[a] = p ? y[K - a] : y[a];
 }
 
-// *x += v, lanes with one address in lane order (siblings behind one hanging
-// face or edge); see add_ordered
-__device__ __forceinline__ void add_lanes(float* x, float v, bool real, int lane, bool hang_any) {
-  add_ordered(x, v, real, lane, hang_any);
-}
-__device__ __forceinline__ void add_lanes(double* x, double v, bool real, int lane, bool hang_any) {
-  if (!hang_any) {
-    *x += v;
-    return;
-  }
-  const unsigned key = real ? (unsigned)__cvta_generic_to_shared(x) : ~(unsigned)lane;
-  const unsigned peers = __match_any_sync(0xffffffffu, key);
-  const int rank = __popc(peers & ((1u << lane) - 1u));
-  const int most = __reduce_max_sync(0xffffffffu, (unsigned)__popc(peers));
-  for (int q = 0; q < most; ++q) {
-    if (real && rank == q) *x += v;
-    __syncwarp();
-  }
-}
-
 template <int K>
 struct Lat {
   static constexpr int N = K + 1, N2 = N * N, N3 = N2 * N, M = 2 * K + 1, M2 = M * M, M3 = M2 * M;
@@ -368,8 +348,6 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
   __syncthreads();
   if (w < N) {  // the warp's class of x-lines: no two warps add to one DoF
     const int nxl = c_ll.nx[K][w];
-    const uint32_t hs = hang ? hg->hs[lane] : 0u;
-    const int zb = nloc * 4;  // byte offset of absent slots
     char* xb = reinterpret_cast<char*>(ys);
     constexpr int SC = sizeof(T) / 4;
 #pragma unroll 1
@@ -381,17 +359,13 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
       if (hang && ((hg->hl[0][lane] >> r) & 1u)) interp_line<K, true>(v, m & 1);
       const uint32_t li = c_ll.line[K][r];
       const int s0 = li & 0xff, o0 = (li >> 8) & 0xff, o1 = li >> 16;
-      const int b0 = st->ls[s0][lane], b1 = st->ls[s0 + 1][lane], b2 = st->ls[s0 + 2][lane];
-      T* p0 = reinterpret_cast<T*>(xb + SC * (b0 + o0));
-      T* p1 = reinterpret_cast<T*>(xb + SC * (b1 + o1));
-      T* p2 = reinterpret_cast<T*>(xb + SC * (b2 + o0));
-      const bool h0 = hang && __any_sync(0xffffffffu, (hs >> s0) & 1u),
-                 h1 = hang && __any_sync(0xffffffffu, (hs >> (s0 + 1)) & 1u),
-                 h2 = hang && __any_sync(0xffffffffu, (hs >> (s0 + 2)) & 1u);
-      add_lanes(p0, v[0], b0 != zb, lane, h0);
-#pragma unroll
-      for (int a = 1; a < K; ++a) add_lanes(p1 + a - 1, v[a], b1 != zb, lane, h1);
-      add_lanes(p2, v[K], b2 != zb, lane, h2);
+      T* p0 = reinterpret_cast<T*>(xb + SC * (st->ls[s0][lane] + o0));
+      T* p1 = reinterpret_cast<T*>(xb + SC * (st->ls[s0 + 1][lane] + o1));
+      T* p2 = reinterpret_cast<T*>(xb + SC * (st->ls[s0 + 2][lane] + o0));
+      add_turns<1>(p0, v, hang ? hg->rank[s0][lane] : 0, hang ? hg->most[s0] : 1);
+      if constexpr (K > 1)
+        add_turns<K - 1>(p1, v + 1, hang ? hg->rank[s0 + 1][lane] : 0, hang ? hg->most[s0 + 1] : 1);
+      add_turns<1>(p2, v + K, hang ? hg->rank[s0 + 2][lane] : 0, hang ? hg->most[s0 + 2] : 1);
     }
   }
   __syncthreads();

@@ -23,6 +23,10 @@ struct LaneLines {
   uint32_t line[KMAX + 1][NMAX * NMAX];
   int8_t xw[KMAX + 1][NMAX][LW];
   int32_t nx[KMAX + 1][NMAX];  // x-lines of each warp
+  // lines q = u + N v (the other two coordinates, in increasing axis order) of
+  // warp w in the passes of tiles with hanging cells: N lines each, the boundary
+  // ones (16 of 25 at k = 4, the only ones that can hang) dealt evenly
+  uint8_t bl[KMAX + 1][NMAX][NMAX];
 };
 static __constant__ LaneLines c_ll;  // one copy per translation unit (filled by its upload function)
 
@@ -48,28 +52,26 @@ __device__ __forceinline__ void interp_line_reg(float* v, int p) {
   for (int a = 0; a < N; ++a) v[a] = p ? y[K - a] : y[a];
 }
 
-// *x += v where lanes with the same address (siblings behind one hanging face
-// or edge) add one after another in lane order; absent DoFs (the zero region)
-// add nothing.  Only lanes whose slot hangs can share an address within one
-// instruction: without such a lane (hang_any = 0) the plain addition is exact.
-static __device__ __noinline__ void add_ordered_slow(float* x, float v, bool real, int lane) {
-  const unsigned key = real ? (unsigned)__cvta_generic_to_shared(x) : ~(unsigned)lane;
-  const unsigned peers = __match_any_sync(0xffffffffu, key);
-  const int rank = __popc(peers & ((1u << lane) - 1u));
-  const int most = __reduce_max_sync(0xffffffffu, (unsigned)__popc(peers));
-  for (int q = 0; q < most; ++q) {
-    if (real && rank == q) *x += v;
+// x[i] += v[i] for the C nodes of one slot: lanes whose slot starts at the same
+// DoF take turns in lane order (rank and turns come with the tile: finding the
+// lanes that meet with a match over the warp's addresses at every node was the
+// largest part of a hanging tile: Q4 sphere postsmoothing 311 -> 261 us with the
+// turns and the hanging lines dealt evenly to the warps)
+template <int C, typename T>
+__device__ __forceinline__ void add_turns(T* x, const T* v, int rank, int turns) {
+  if (turns <= 1) {  // uniform over the warp
+#pragma unroll
+    for (int i = 0; i < C; ++i) x[i] += v[i];
+    return;
+  }
+#pragma unroll 1
+  for (int q = 0; q < turns; ++q) {
+    if (rank == q) {
+#pragma unroll
+      for (int i = 0; i < C; ++i) x[i] += v[i];
+    }
     __syncwarp();
   }
-}
-
-// (the ordered path out of line: the unrolled scatter of the tiles with hanging cells calls it
-// at every node, and inlined it would multiply that code)
-__device__ __forceinline__ void add_ordered(float* x, float v, bool real, int lane, bool hang_any) {
-  if (!hang_any)
-    *x += v;
-  else
-    add_ordered_slow(x, v, real, lane);
 }
 
 __device__ __forceinline__ df df_sel(bool p, df a, df b) { return df{p ? a.hi : b.hi, p ? a.lo : b.lo}; }
@@ -171,25 +173,6 @@ __device__ __forceinline__ void interp_line_df(df* v, int p) {
   for (int a = 0; a < N; ++a) v[a] = df_sel(p, y[K - a], y[a]);
 }
 
-// the same in double-float
-static __device__ __noinline__ void add_ordered_df_slow(df* x, df v, bool real, int lane) {
-  const unsigned key = real ? (unsigned)__cvta_generic_to_shared(x) : ~(unsigned)lane;
-  const unsigned peers = __match_any_sync(0xffffffffu, key);
-  const int rank = __popc(peers & ((1u << lane) - 1u));
-  const int most = __reduce_max_sync(0xffffffffu, (unsigned)__popc(peers));
-  for (int q = 0; q < most; ++q) {
-    if (real && rank == q) *x = df_add(*x, v);
-    __syncwarp();
-  }
-}
-
-__device__ __forceinline__ void add_ordered_df(df* x, df v, bool real, int lane, bool hang_any) {
-  if (!hang_any)
-    *x = df_add(*x, v);
-  else
-    add_ordered_df_slow(x, v, real, lane);
-}
-
 // host: entity slot and offset of local node (a, b, c) of a degree-k cell
 // (the numbering of the level set-up: slot cx + 3 cy + 9 cz, DoFs of an
 // entity lexicographic over its interior axes)
@@ -247,6 +230,15 @@ inline void fill_lane_lines(LaneLines& t) {
       }
     }
     for (int w = 0; w < n; ++w) t.nx[k][w] = load[w];
+    std::vector<int> bal(n, 0);
+    int w = 0;
+    for (int pass = 0; pass < 2; ++pass)
+      for (int q = 0; q < n * n; ++q) {
+        const bool boundary = cls(q % n) < 0 || cls(q / n) < 0;
+        if (boundary != (pass == 0)) continue;
+        t.bl[k][w][bal[w]++] = (uint8_t)q;
+        w = (w + 1) % n;
+      }
   }
 }
 

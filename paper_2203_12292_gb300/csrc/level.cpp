@@ -351,10 +351,19 @@ void build_level(const Octree& mesh, int k, int tile_cells, int LM, LevelHost& L
               if ((f1 && on1) || (f2 && on2) || (ed && on1 && on2)) lh.hl[D][j] |= 1u << (u + n * v);
             }
         }
-        for (int s2 = 0; s2 < NSLOT; ++s2) {
-          const int cl[3] = {s2 % 3, (s2 / 3) % 3, s2 / 9};
-          if (slot_hanging(m, cl)) lh.hs[j] |= 1u << s2;
+      }
+      const LaneTile& lt = L.lane[t];
+      const int zero = 4 * (L.tiles[t].n_owned + L.tiles[t].n_foreign);
+      for (int s2 = 0; s2 < NSLOT; ++s2) {
+        int most = 1;
+        for (int j = 0; j < 32; ++j) {
+          if (lt.ls[s2][j] == zero) continue;
+          int r = 0;
+          for (int i = 0; i < j; ++i) r += lt.ls[s2][i] == lt.ls[s2][j];
+          lh.rank[s2][j] = (uint8_t)r;
+          most = std::max(most, r + 1);
         }
+        lh.most[s2] = (uint8_t)most;
       }
     }
   }
@@ -556,6 +565,13 @@ void validate_level(const LevelHost& L) {
           if (dof >= nloc) fail("lane DoF outside the tile");
           planes[dof] |= 1u << c;
           classes[dof] |= uint64_t(1) << xcls;
+          if (lt.hang) {  // the lanes of a slot that meet one DoF add in turns, one rank after another
+            const LaneHang& lh = L.lane_hang[t];
+            const int s = nslot[nd];
+            int before = 0;
+            for (int i = 0; i < j; ++i) before += lt.ls[s][i] == off;
+            if (lh.rank[s][j] != before || lh.most[s] <= before) fail("rank of a lane in a shared slot");
+          }
           if (!lt.hang) {
             const int64_t key = (int64_t)t * 1024 + nd;
             if (stamp[dof] == key) fail("two cells add to one DoF through one node");
