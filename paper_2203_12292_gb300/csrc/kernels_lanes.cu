@@ -12,9 +12,9 @@
 //   * the entity starts of the tile are stored transposed (slot s of cell j
 //     at s * 32 + j), read conflict-free.
 // The sweeps apply the fast-diagonalisation form of the Cartesian cell matrix
-// h (K x M x M + M x K x M + M x M x K) = h B^T(x3) diag(lam_a+lam_b+lam_c) B(x3)
-// with the even-odd split of B (rows of B are symmetric or antisymmetric
-// under x -> 1 - x).
+// h (K x M x M + M x K x M + M x M x K) in two directions, with the even-odd
+// split of B (rows of B are symmetric or antisymmetric under x -> 1 - x), and
+// K + (lam + lam') M in the innermost one (zline.cuh).
 //
 // Accumulation without atomics and in a fixed order.  Two local nodes of
 // different cells can be the same DoF only if, along every axis, their
@@ -44,6 +44,7 @@
 #include "device.cuh"
 #include "kernels.h"
 #include "lanes.cuh"
+#include "zline.cuh"
 
 namespace gcmg {
 
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 8 : 1) vmult_lanes(Lane
   // is cleared after the cell buffer's last read (8 instead of 7 blocks per SM at k = 4)
   float* cb = reinterpret_cast<float*>(smem + sizeof(LaneTile) + sizeof(LaneHang));
   float* xs0 = cb;  // 16-byte aligned
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, w = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);  // w: uniform
   // block b's tile: records in launch order at [b] (no dependent load of the tile index) or tile0 + b
   const int bx = blockIdx.x, tl = A.tile0 + bx;
   const LaneTile* ltp = A.order ? A.lt_lo + bx : A.lt + tl;
@@ -258,23 +259,16 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 8 : 1) vmult_lanes(Lane
       for (int n = 0; n < N2; ++n) p[n * 32] = u[n];
     }
     __syncthreads();
-    // z: forward sweep, h (lam_a + lam_b + lam_c) in mode order, backward sweep (lines (a, b) = (i, w))
-    {
-      const float hb = h * tb.lame[w];
+    // z: h (K + (lam_a + lam_b) M) on the lines of modes (a, b) = (i, w)
 #pragma unroll
-      for (int i = 0; i < N; ++i) {
-        float* p = cb + (i + N * w) * 32 + lane;
-        float v[N];
+    for (int i = 0; i < N; ++i) {
+      float* p = cb + (i + N * w) * 32 + lane;
+      float v[N];
 #pragma unroll
-        for (int c = 0; c < N; ++c) v[c] = p[c * N2 * 32];
-        eo_forward<N, 0, 1>(v, tb.Be);
-        const float hab = fmaf(h, tb.lame[i], hb);
+      for (int c = 0; c < N; ++c) v[c] = p[c * N2 * 32];
+      zline<K>(v, c_zl.h[K - 1][i + N * w]);
 #pragma unroll
-        for (int c = 0; c < N; ++c) v[c] *= fmaf(h, tb.lame[c], hab);
-        eo_backward<N, 0, 1>(v, tb.Be);
-#pragma unroll
-        for (int c = 0; c < N; ++c) p[c * N2 * 32] = v[c];
-      }
+      for (int c = 0; c < N; ++c) p[c * N2 * 32] = h * v[c];
     }
     __syncthreads();
     {
@@ -337,23 +331,16 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 8 : 1) vmult_lanes(Lane
     __syncthreads();
     sweep_y<K, true>(cb, w, lane);
     __syncthreads();
-    // x: forward sweep, h (lam_a + lam_b + lam_c) in mode order, backward sweep (lines (b, c) = (i, w))
-    {
-      const float hc = h * tb.lame[w];
+    // x: h (K + (lam_b + lam_c) M) on the lines of modes (b, c) = (i, w)
 #pragma unroll
-      for (int i = 0; i < N; ++i) {
-        float* p = cb + N * (i + N * w) * 32 + lane;
-        float v[N];
+    for (int i = 0; i < N; ++i) {
+      float* p = cb + N * (i + N * w) * 32 + lane;
+      float x[N];
 #pragma unroll
-        for (int a = 0; a < N; ++a) v[a] = p[a * 32];
-        eo_forward<N, 0, 1>(v, tb.Be);
-        const float hbc = fmaf(h, tb.lame[i], hc);
+      for (int a = 0; a < N; ++a) x[a] = p[a * 32];
+      zline<K>(x, c_zl.h[K - 1][i + N * w]);
 #pragma unroll
-        for (int a = 0; a < N; ++a) v[a] *= fmaf(h, tb.lame[a], hbc);
-        eo_backward<N, 0, 1>(v, tb.Be);
-#pragma unroll
-        for (int a = 0; a < N; ++a) p[a * 32] = v[a];
-      }
+      for (int a = 0; a < N; ++a) p[a * 32] = h * x[a];
     }
     __syncthreads();
     sweep_y<K, false>(cb, w, lane);
@@ -423,13 +410,14 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 8 : 1) vmult_lanes(Lane
 // of code: written out pass by pass, the kernel's instructions did not fit the
 // instruction caches (the largest stall was "no instruction", 57 % issue
 // active).  A pass takes the lines along direction D through, in this order,
-// C_e, the forward transform, the scaling, the backward transform, C_e^T.
-enum : uint8_t { DF_C = 4, DF_FWD = 8, DF_SCALE = 16, DF_BWD = 32, DF_CT = 64 };  // bits 0-1: D
+// C_e, the forward transform, the innermost direction's matrix (zline), the
+// backward transform, C_e^T.
+enum : uint8_t { DF_C = 4, DF_FWD = 8, DF_Z = 16, DF_BWD = 32, DF_CT = 64 };  // bits 0-1: D
 __constant__ uint8_t c_df_pass[2][9] = {
     // tiles without hanging cells: x, y forward, z, y, x backward
-    {0 | DF_FWD, 1 | DF_FWD, 2 | DF_FWD | DF_SCALE | DF_BWD, 1 | DF_BWD, 0 | DF_BWD, 0, 0, 0, 0},
+    {0 | DF_FWD, 1 | DF_FWD, 2 | DF_Z, 1 | DF_BWD, 0 | DF_BWD, 0, 0, 0, 0},
     // with hanging cells: C_x, C_y, C_z and the sweeps in the order z, y, x, and back
-    {0 | DF_C, 1 | DF_C, 2 | DF_C | DF_FWD, 1 | DF_FWD, 0 | DF_FWD | DF_SCALE | DF_BWD, 1 | DF_BWD, 2 | DF_BWD | DF_CT,
+    {0 | DF_C, 1 | DF_C, 2 | DF_C | DF_FWD, 1 | DF_FWD, 0 | DF_Z, 1 | DF_BWD, 2 | DF_BWD | DF_CT,
      1 | DF_CT, 0 | DF_CT}};
 
 template <int K>
@@ -442,7 +430,7 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(L
   // vmult_lanes: 6 instead of 4 blocks per SM at k = 4
   df* cb = reinterpret_cast<df*>(smem + sizeof(LaneTile) + sizeof(LaneHang));
   double* xd0 = reinterpret_cast<double*>(cb);  // 16-byte aligned
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, w = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);  // w: uniform
   // block b's tile: records in launch order at [b] (no dependent load of the tile index) or tile0 + b
   const int bx = blockIdx.x, tl = A.tile0 + bx;
   const LaneTile* ltp = A.order ? A.lt_lo + bx : A.lt + tl;
@@ -529,7 +517,7 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(L
       const int r = c_ll.bl[K][w][i];
       const bool on = (hl >> r) & 1u;
       // a pass of C_e or C_e^T alone touches the hanging lines only
-      if (!(f & (DF_FWD | DF_BWD)) && !on) continue;
+      if (!(f & (DF_FWD | DF_Z | DF_BWD)) && !on) continue;
       const int q = D == 0 ? N * r : (D == 1 ? r % N + N2 * (r / N) : r);
       df* ptr = cb + q * 32 + lane;
       df v[N];
@@ -537,10 +525,10 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(L
       for (int a = 0; a < N; ++a) v[a] = ptr[a * S * 32];
       if ((f & DF_C) && on) interp_line_df<K, false>(v, p);
       if (f & DF_FWD) df_eo_fwd_fast<K>(v);
-      if (f & DF_SCALE) {  // h (lam_a + lam_b + lam_c) in mode order
+      if (f & DF_Z) {  // h (K + (lam + lam') M) on the line of modes r
+        zline<K>(v, c_zl.h[K - 1][r], c_zl.l[K - 1][r]);
 #pragma unroll
-        for (int c = 0; c < N; ++c)
-          v[c] = df_mul(v[c], df_mul(df{c_tf[K].lam3[q + c * S], c_tflo[K].lam3[q + c * S]}, h));
+        for (int c = 0; c < N; ++c) v[c] = df_mul(v[c], h);
       }
       if (f & DF_BWD) df_eo_bwd_fast<K>(v);
       if ((f & DF_CT) && on) interp_line_df<K, true>(v, p);
@@ -636,6 +624,7 @@ void upload_tables_lanes() {
   static LaneLines t;
   fill_lane_lines(t);
   cudaMemcpyToSymbol(c_ll, &t, sizeof(t));
+  upload_zlines();
 }
 
 bool lanes_ok(const CellLaunch& L) { return L.lane_tiles && L.tc <= 32 && !L.geom && L.k >= 1 && L.k <= KMAX; }

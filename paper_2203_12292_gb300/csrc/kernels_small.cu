@@ -19,6 +19,7 @@
 #include "device.cuh"
 #include "kernels.h"
 #include "lanes.cuh"
+#include "zline.cuh"
 
 namespace gcmg {
 
@@ -28,44 +29,8 @@ namespace {
 
 constexpr int SWPB = 4;  // warps per block
 
-// arithmetic of the cell pipeline: fp32, or double-float on fp64 vectors
-template <typename T>
-struct Arith;
-template <>
-struct Arith<float> {
-  using V = float;
-  static __device__ __forceinline__ V in(float x) { return x; }
-  static __device__ __forceinline__ float out(V x) { return x; }
-};
-template <>
-struct Arith<double> {
-  using V = df;
-  static __device__ __forceinline__ V in(double x) { return df_from(x); }
-  static __device__ __forceinline__ double out(V x) { return df_to(x); }
-};
-
-template <int K, bool FWD>
-__device__ __forceinline__ void eo_line(float* v) {
-  if (FWD)
-    eo_forward<K + 1, 0, 1>(v, tab<float>(K).Be);
-  else
-    eo_backward<K + 1, 0, 1>(v, tab<float>(K).Be);
-}
-template <int K, bool FWD>
-__device__ __forceinline__ void eo_line(df* v) {
-  if (FWD)
-    df_eo_fwd_fast<K>(v);
-  else
-    df_eo_bwd_fast<K>(v);
-}
-template <int K, bool TRANS>
-__device__ __forceinline__ void hang_line(float* v, int p) {
-  interp_line_reg<K, TRANS>(v, p);
-}
-template <int K, bool TRANS>
-__device__ __forceinline__ void hang_line(df* v, int p) {
-  interp_line_df<K, TRANS>(v, p);
-}
+// the z-line coefficients again: a lane reads its own line's, which constant memory would serialise
+__device__ ZLines g_zl;
 
 template <typename T>
 struct CellVecArgs {
@@ -141,15 +106,20 @@ __global__ void __launch_bounds__(SWPB * 32) cell_vectors(CellVecArgs<T> A) {
   const int q = lane / N2, r = lane - q * N2;     // the lane's cell and line
   const bool on = q < nc;
   uint16_t m = 0;
-  V sc[N];                                        // h (lam_a + lam_b + lam_c) on the z-line (a, b) = r
+  constexpr int NC = (N / 2) * (N / 2) + ((N + 1) / 2) * ((N + 1) / 2);
+  float zh[NC], zl[sizeof(T) == 8 ? NC : 1];      // K + (lam_a + lam_b) M on the z-line (a, b) = r
+  V h = V(0);
   if (on) {
     const CellMeta& cm = A.meta[c0 + q];
     m = cm.mask;
-    double h = ldexp(A.dom, -(int)cm.level);
-    if (A.coef) h *= A.coef[c0 + q];
-    const double lab = c_td[K].lame[r % N] + c_td[K].lame[r / N];
+    double hd = ldexp(A.dom, -(int)cm.level);
+    if (A.coef) hd *= A.coef[c0 + q];
+    h = V(hd);
 #pragma unroll
-    for (int c = 0; c < N; ++c) sc[c] = V(h * (lab + c_td[K].lame[c]));
+    for (int i = 0; i < NC; ++i) {
+      zh[i] = g_zl.h[K - 1][r][i];
+      if (sizeof(T) == 8) zl[i] = g_zl.l[K - 1][r][i];
+    }
   }
   const bool hang = __any_sync(0xffffffffu, (m & MASK_HANG) != 0);
   pdl_wait();
@@ -174,10 +144,12 @@ __global__ void __launch_bounds__(SWPB * 32) cell_vectors(CellVecArgs<T> A) {
     V x[N];
 #pragma unroll
     for (int c = 0; c < N; ++c) x[c] = cl[r + N2 * c];
-    eo_line<K, true>(x);
+    if constexpr (sizeof(T) == 8)
+      zline<K>(x, zh, zl);
+    else
+      zline<K>(x, zh);
 #pragma unroll
-    for (int c = 0; c < N; ++c) x[c] = x[c] * sc[c];
-    eo_line<K, false>(x);
+    for (int c = 0; c < N; ++c) x[c] = x[c] * h;
 #pragma unroll
     for (int c = 0; c < N; ++c) cl[r + N2 * c] = x[c];
   }
@@ -349,6 +321,10 @@ void upload_tables_small() {
   static LaneLines ll;
   fill_lane_lines(ll);
   cudaMemcpyToSymbol(c_ll, &ll, sizeof(ll));
+  upload_zlines();
+  static ZLines z;
+  cudaMemcpyFromSymbol(&z, c_zl, sizeof(z));
+  cudaMemcpyToSymbol(g_zl, &z, sizeof(z));
 }
 
 // recorded launch lists (the persistent batch) keep the tile kernels

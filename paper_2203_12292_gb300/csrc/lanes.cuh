@@ -173,6 +173,45 @@ __device__ __forceinline__ void interp_line_df(df* v, int p) {
   for (int a = 0; a < N; ++a) v[a] = df_sel(p, y[K - a], y[a]);
 }
 
+// arithmetic of the cell pipeline: fp32, or double-float on fp64 vectors
+template <typename T>
+struct Arith;
+template <>
+struct Arith<float> {
+  using V = float;
+  static __device__ __forceinline__ V in(float x) { return x; }
+  static __device__ __forceinline__ float out(V x) { return x; }
+};
+template <>
+struct Arith<double> {
+  using V = df;
+  static __device__ __forceinline__ V in(double x) { return df_from(x); }
+  static __device__ __forceinline__ double out(V x) { return df_to(x); }
+};
+
+template <int K, bool FWD>
+__device__ __forceinline__ void eo_line(float* v) {
+  if (FWD)
+    eo_forward<K + 1, 0, 1>(v, tab<float>(K).Be);
+  else
+    eo_backward<K + 1, 0, 1>(v, tab<float>(K).Be);
+}
+template <int K, bool FWD>
+__device__ __forceinline__ void eo_line(df* v) {
+  if (FWD)
+    df_eo_fwd_fast<K>(v);
+  else
+    df_eo_bwd_fast<K>(v);
+}
+template <int K, bool TRANS>
+__device__ __forceinline__ void hang_line(float* v, int p) {
+  interp_line_reg<K, TRANS>(v, p);
+}
+template <int K, bool TRANS>
+__device__ __forceinline__ void hang_line(df* v, int p) {
+  interp_line_df<K, TRANS>(v, p);
+}
+
 // host: entity slot and offset of local node (a, b, c) of a degree-k cell
 // (the numbering of the level set-up: slot cx + 3 cy + 9 cz, DoFs of an
 // entity lexicographic over its interior axes)
