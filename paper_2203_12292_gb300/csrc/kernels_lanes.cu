@@ -580,6 +580,173 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(L
   for (int i = threadIdx.x; i < ti.n_foreign; i += NT) A.halo[hp[i]] = df_to(xs[ti.n_owned + i]);
 }
 
+// ---------------------------------------------------------------------------
+// degree 1: one warp per tile, the lane's cell (8 values) in registers.  The
+// sweeps need neither a cell buffer nor a barrier, and a tile is one chain of its
+// metadata, its DoFs and about 300 instructions: four tiles per block, each on
+// its own, hide one another's latencies, and only the vertex rows of the lane
+// record are copied (512 of 1,856 B).  Octant mesh, 269,998 cells: fp32 19.9 ->
+// 14.4 us, fp64 45 -> 34 us.  At k = 2 (27 values, 64 or 96 registers) the same
+// kernel was slower than vmult_lanes: 34,903 cells 14 -> 21 us in fp32, 31 -> 44 us
+// in fp64.
+// ---------------------------------------------------------------------------
+constexpr int RWPB = 4;  // tiles (warps) per block
+
+template <int K>
+__device__ __forceinline__ void reg_z(float* v, int q) {
+  zline<K>(v, c_zl.h[K - 1][q]);
+}
+template <int K>
+__device__ __forceinline__ void reg_z(df* v, int q) {
+  zline<K>(v, c_zl.h[K - 1][q], c_zl.l[K - 1][q]);
+}
+
+template <int K, int D, bool FWD, typename V>
+__device__ __forceinline__ void reg_sweep(V* u) {
+  constexpr int N = K + 1, S = line_stride<N, D>();
+#pragma unroll
+  for (int q = 0; q < N * N; ++q) {
+    const int base = line_base<K, D>(q);
+    V v[N];
+#pragma unroll
+    for (int a = 0; a < N; ++a) v[a] = u[base + a * S];
+    eo_line<K, FWD>(v);
+#pragma unroll
+    for (int a = 0; a < N; ++a) u[base + a * S] = v[a];
+  }
+}
+
+template <int K, int D, bool TRANS, typename V>
+__device__ __forceinline__ void reg_hang(V* u, uint16_t m, uint32_t hl) {
+  constexpr int N = K + 1, S = line_stride<N, D>();
+  const int p = (m >> D) & 1;
+#pragma unroll
+  for (int q = 0; q < N * N; ++q) {
+    const int x = q % N, y = q / N;
+    if (x > 0 && x < K && y > 0 && y < K) continue;  // inside the cell
+    if (!((hl >> q) & 1u)) continue;
+    const int base = line_base<K, D>(q);
+    V v[N];
+#pragma unroll
+    for (int a = 0; a < N; ++a) v[a] = u[base + a * S];
+    hang_line<K, TRANS>(v, p);
+#pragma unroll
+    for (int a = 0; a < N; ++a) u[base + a * S] = v[a];
+  }
+}
+
+// rows of the lane record in shared memory: the 8 vertex slots
+constexpr int REG_ROWS = 8;
+__device__ __forceinline__ int vertex_slot(int r) { return 2 * (r & 1) + 6 * ((r >> 1) & 1) + 18 * (r >> 2); }
+template <typename V>
+size_t reg_smem(int max_local) {
+  return RWPB * ((size_t)REG_ROWS * 64 + ((((size_t)max_local + LANE_ZERO) * sizeof(V) + 15) & ~(size_t)15));
+}
+
+template <typename T>
+__global__ void __launch_bounds__(RWPB * 32) vmult_q1(LaneArgsT<T> A, int n_tiles, int warp_bytes) {
+  using AR = Arith<T>;
+  using V = typename AR::V;
+  constexpr int K = 1, N = 2, N2 = 4, N3 = 8, NR = REG_ROWS;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int bx = blockIdx.x * RWPB + w, tl = A.tile0 + bx;
+  if (bx >= n_tiles) return;
+  uint16_t(*ls)[32] = reinterpret_cast<uint16_t(*)[32]>(smem + (size_t)w * warp_bytes);
+  V* xs = reinterpret_cast<V*>(smem + (size_t)w * warp_bytes + NR * 64);
+  T* xt = reinterpret_cast<T*>(xs);  // the values as they arrive; converted in place
+  const LaneTile* lt = A.order ? A.lt_lo + bx : A.lt + tl;
+  const LaneHang* lh = A.order ? A.lh_lo + bx : A.lh + tl;
+  const TileInfo ti = A.order ? A.tiles_lo[bx] : A.tiles[tl];
+  const int nloc = ti.n_owned + ti.n_foreign;
+  for (int i = lane; i < NR * 4; i += 32)
+    cp_async16(reinterpret_cast<unsigned char*>(ls) + 16 * i,
+               reinterpret_cast<const unsigned char*>(lt->ls[vertex_slot(i >> 2)]) + 16 * (i & 3));
+  const uint16_t m = lt->mask[lane];
+  const bool hang = lt->hang != 0;
+  uint32_t hl[3] = {0u, 0u, 0u};
+  if (hang)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) hl[d] = lh->hl[d][lane];
+  const int32_t* fl = A.foreign + ti.foreign_begin;
+  constexpr int FU = 4;  // foreign indices loaded ahead of the predecessor's completion
+  int idx[FU];
+#pragma unroll
+  for (int u = 0; u < FU; ++u) idx[u] = lane + 32 * u < ti.n_foreign ? fl[lane + 32 * u] : -1;
+  double h = ldexp(A.dom, -(int)lt->level[lane]);
+  if (A.coef) h *= A.coef[ti.cell_begin + min(lane, ti.n_cells - 1)];
+  pdl_wait();
+  const T* so = A.src + ti.dof_begin;
+  for (int i = lane; i < ti.n_owned; i += 32) cp_async(xt + i, so + i);
+#pragma unroll
+  for (int u = 0; u < FU; ++u)
+    if (idx[u] >= 0) cp_async(xt + ti.n_owned + lane + 32 * u, A.src + idx[u]);
+  for (int i = lane + 32 * FU; i < ti.n_foreign; i += 32) cp_async(xt + ti.n_owned + i, A.src + fl[i]);
+  cp_async_wait_all();
+  __syncwarp();
+  if constexpr (sizeof(T) == 8)
+    for (int i = lane; i < nloc; i += 32) xs[i] = AR::in(xt[i]);  // one lane per element: in place
+  for (int i = lane; i < LANE_ZERO; i += 32) xs[nloc + i] = V(0);
+  __syncwarp();
+  // G_e
+  V u[N3];
+#pragma unroll
+  for (int n = 0; n < N3; ++n) u[n] = xs[ls[n][lane] >> 2];
+  __syncwarp();
+  for (int i = lane; i < nloc; i += 32) xs[i] = V(0);  // the accumulator
+  if (hang) {
+    reg_hang<K, 0, false>(u, m, hl[0]);
+    reg_hang<K, 1, false>(u, m, hl[1]);
+    reg_hang<K, 2, false>(u, m, hl[2]);
+  }
+  reg_sweep<K, 0, true>(u);
+  reg_sweep<K, 1, true>(u);
+  {  // z: h (K + (lam_a + lam_b) M)
+    const V hv = V(h);
+#pragma unroll
+    for (int q = 0; q < N2; ++q) {
+      V v[N];
+#pragma unroll
+      for (int a = 0; a < N; ++a) v[a] = u[q + a * N2];
+      reg_z<K>(v, q);
+#pragma unroll
+      for (int a = 0; a < N; ++a) u[q + a * N2] = v[a] * hv;
+    }
+  }
+  reg_sweep<K, 1, false>(u);
+  reg_sweep<K, 0, false>(u);
+  if (hang) {
+    reg_hang<K, 2, true>(u, m, hl[2]);
+    reg_hang<K, 1, true>(u, m, hl[1]);
+    reg_hang<K, 0, true>(u, m, hl[0]);
+  }
+  __syncwarp();
+  // G_e^T, node by node: the lanes of one node meet only behind hanging faces and edges (turns)
+#pragma unroll
+  for (int n = 0; n < N3; ++n) {
+    const int slot = vertex_slot(n);
+    add_turns<1>(xs + (ls[n][lane] >> 2), &u[n], hang ? lh->rank[slot][lane] : 0, hang ? lh->most[slot] : 1);
+    __syncwarp();
+  }
+  T* d = A.dst + ti.dof_begin;
+  for (int i = lane; i < ti.n_owned; i += 32) {
+    const T v = AR::out(xs[i]);
+    d[i] = A.add ? d[i] + v : v;
+  }
+  const int32_t* hp = A.halo_pos + ti.foreign_begin;
+  for (int i = lane; i < ti.n_foreign; i += 32) A.halo[hp[i]] = AR::out(xs[ti.n_owned + i]);
+}
+
+template <typename T>
+cudaError_t run_q1(const CellLaunch& L, const LaneArgsT<T>& A, int n_tiles, cudaStream_t s) {
+  const size_t sm = reg_smem<typename Arith<T>::V>(L.max_local);
+  cudaError_t e = smem_allow(vmult_q1<T>, sm);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(vmult_q1<T>, (n_tiles + RWPB - 1) / RWPB, RWPB * 32, sm, s, A, n_tiles, (int)(sm / RWPB));
+  note_launches(1);
+  return e;
+}
+
 template <int K>
 size_t lanes_smem(int max_local) {
   constexpr int N3 = (K + 1) * (K + 1) * (K + 1);
@@ -651,7 +818,7 @@ void launch_vmult_lanes_df(const CellLaunch& L, const double* src, double* dst, 
   A.add = add;
   A.tile0 = t0;
   switch (L.k) {
-    case 1: run_lanes_df<1>(L, A, t1 - t0, s); break;
+    case 1: run_q1(L, A, t1 - t0, s); break;
     case 2: run_lanes_df<2>(L, A, t1 - t0, s); break;
     case 3: run_lanes_df<3>(L, A, t1 - t0, s); break;
     case 4: run_lanes_df<4>(L, A, t1 - t0, s); break;
@@ -682,7 +849,7 @@ void launch_vmult_lanes(const CellLaunch& L, const void* src, void* dst, int add
   A.add = add;
   A.tile0 = t0;
   switch (L.k) {
-    case 1: run_lanes<1>(L, A, t1 - t0, s); break;
+    case 1: run_q1(L, A, t1 - t0, s); break;
     case 2: run_lanes<2>(L, A, t1 - t0, s); break;
     case 3: run_lanes<3>(L, A, t1 - t0, s); break;
     case 4: run_lanes<4>(L, A, t1 - t0, s); break;
