@@ -473,7 +473,7 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(L
   if (threadIdx.x < LANE_ZERO) xs[nloc + threadIdx.x] = df{0.f, 0.f};
   cp_async_wait_all();
   __syncthreads();
-  for (int i = threadIdx.x; i < nloc; i += NT) xs[i] = df_from(xd[i]);  // one thread per element: in place
+  for (int i = threadIdx.x; i < nloc; i += NT) xs[i] = df_from_bits(xd[i]);  // one thread per element: in place
   const uint16_t m = st->mask[lane];
   const bool hang = st->hang != 0;
   df h;
@@ -573,11 +573,11 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(L
   __syncthreads();
   double* d = A.dst + ti.dof_begin;
   if (A.add)
-    for (int i = threadIdx.x; i < ti.n_owned; i += NT) d[i] += df_to(xs[i]);
+    for (int i = threadIdx.x; i < ti.n_owned; i += NT) d[i] += df_to_bits(xs[i]);
   else
-    for (int i = threadIdx.x; i < ti.n_owned; i += NT) d[i] = df_to(xs[i]);
+    for (int i = threadIdx.x; i < ti.n_owned; i += NT) d[i] = df_to_bits(xs[i]);
   const int32_t* hp = A.halo_pos + ti.foreign_begin;
-  for (int i = threadIdx.x; i < ti.n_foreign; i += NT) A.halo[hp[i]] = df_to(xs[ti.n_owned + i]);
+  for (int i = threadIdx.x; i < ti.n_foreign; i += NT) A.halo[hp[i]] = df_to_bits(xs[ti.n_owned + i]);
 }
 
 // ---------------------------------------------------------------------------
