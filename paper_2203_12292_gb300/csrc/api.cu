@@ -751,9 +751,8 @@ void setup_handle(Handle& H, const std::vector<Octree>& gc_meshes, int lmax, con
     LevelHost& lh = L->host;
     L->tiles.upload(lh.tiles, H.stream);
     L->halo.alloc(lh.foreign.size() * sizeof(double));
-    L->halo_dofs.upload(lh.halo_dofs, H.stream);
-    L->halo_ptr.upload(lh.halo_ptr, H.stream);
-    L->halo_src.upload(lh.halo_src, H.stream);
+    L->halo_ents.upload(lh.halo_ents, H.stream);
+    L->halo_blocks.upload(lh.halo_blocks, H.stream);
     L->halo_pos.upload(lh.halo_pos, H.stream);
     L->meta.upload(lh.meta, H.stream);
     L->foreign.upload(lh.foreign, H.stream);
@@ -790,11 +789,10 @@ void setup_handle(Handle& H, const std::vector<Octree>& gc_meshes, int lmax, con
     c.tiles = L->tiles.as<TileInfo>();
     c.n_tiles = (int)lh.tiles.size();
     c.halo = L->halo.p;
-    c.halo_dofs = L->halo_dofs.as<int32_t>();
-    c.halo_ptr = L->halo_ptr.as<int32_t>();
-    c.halo_src = L->halo_src.as<int32_t>();
+    c.halo_ents = L->halo_ents.as<int32_t>();
+    c.halo_blocks = L->halo_blocks.as<HaloBlock>();
     c.halo_pos = L->halo_pos.as<int32_t>();
-    c.n_halo = (int)lh.halo_dofs.size();
+    c.n_halo = (int)lh.halo_blocks.size();
     c.meta = L->meta.as<CellMeta>();
     c.foreign = L->foreign.as<int32_t>();
     c.subptr = L->subptr.as<uint16_t>();
@@ -1047,7 +1045,7 @@ int gcmg_get_level_info(const gcmg_handle* h, int level, gcmg_level_info* info) 
     info->n_cells = (int64_t)L.host.cells.size();
     info->degree = L.host.k;
     info->n_tiles = (int)L.host.tiles.size();
-    info->n_halo = (int64_t)L.host.halo_dofs.size();
+    info->n_halo = L.host.n_halo_dofs;
     info->tile_cells = L.host.tile_cells;
     info->max_local = L.host.max_local;
     info->fp32 = L.fp32 ? 1 : 0;

@@ -19,7 +19,7 @@ struct LevelDev {
   DevBuf tiles, meta, foreign, subptr, perm, cell_ijk, gstart, own, mask, lane_tiles, lane_order, lane_hang, tiles_lo,
       lane_tiles_lo, lane_hang_lo;
   DevBuf sum_ptr, sum_pos, cell_vec;  // levels of few cells
-  DevBuf halo, halo_dofs, halo_ptr, halo_src, halo_pos;
+  DevBuf halo, halo_ents, halo_blocks, halo_pos;
   DevBuf diag64, dinv64, dinv32;
   DevBuf x, b, d, t;        // V-cycle vectors in level precision
   DevBuf w64a, w64b, w64c;  // fp64 work vectors (set-up, fp64 smoothing through the API)

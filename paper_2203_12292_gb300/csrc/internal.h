@@ -66,6 +66,16 @@ struct LaneHang {
 };
 static_assert(sizeof(LaneHang) % 16 == 0, "LaneHang is copied in 16-byte pieces");
 
+// one block of the halo pass: n DoFs of the entities halo_ents[ent0 ..], all
+// with nd DoFs and c contributing tiles each; DoF i of the block has its c slots
+// at slot0 + i c
+constexpr int HALO_BLOCK_DOFS = 512;
+struct HaloBlock {
+  int32_t ent0, n, nd, c, slot0;
+  int32_t inv;  // 2^16 / nd rounded up: i / nd = i inv >> 16 for i < HALO_BLOCK_DOFS
+  int32_t pad[2];
+};
+
 struct TileInfo {
   int32_t cell_begin;
   int32_t n_cells;
@@ -146,10 +156,12 @@ struct LevelHost {
   std::vector<int32_t> foreign;    // foreign DoF global indices, per tile contiguous
   std::vector<uint16_t> subptr;    // per tile: n_sub+1 offsets into the tile's permuted cell list
   std::vector<uint8_t> perm;       // per cell (tile order): local cell index in sub-colour order
-  std::vector<int32_t> halo_dofs;  // DoFs that receive contributions from other tiles (increasing)
-  std::vector<int32_t> halo_ptr;   // per halo DoF: range into halo_src
-  std::vector<int32_t> halo_src;   // foreign-slot indices (positions in `foreign`)
-  std::vector<int32_t> halo_pos;   // per foreign slot: its position in the DoF-ordered halo buffer
+  // DoFs that receive contributions from other tiles, by entity: sections of equal
+  // (DoFs per entity, contributing tiles), increasing inside a section
+  std::vector<int32_t> halo_ents;  // first DoF of every entity
+  std::vector<HaloBlock> halo_blocks;
+  int64_t n_halo_dofs = 0;
+  std::vector<int32_t> halo_pos;   // per foreign slot: its position in the halo buffer
   int max_local = 0;               // max tile-local DoF count
   std::vector<LaneTile> lane;      // per tile (tiles of at most 32 cells): lane-per-cell metadata
   std::vector<int32_t> lane_order; // tiles with hanging cells, then the others (launch order)

@@ -23,13 +23,12 @@ struct CellLaunch {
   const uint16_t* subptr;
   const uint8_t* perm;
   const int32_t* cell_ijk;  // per cell i, j, k (right-hand side only)
-  // halo: one slot per (tile, foreign DoF); per halo DoF the slots to add
+  // halo: one slot per (tile, foreign DoF), in the order of the halo pass
   void* halo;  // n_foreign_total values of the launch precision
-  const int32_t* halo_dofs;
-  const int32_t* halo_ptr;
-  const int32_t* halo_src;
-  const int32_t* halo_pos;  // per foreign slot: position in the DoF-ordered halo buffer
-  int n_halo;
+  const int32_t* halo_ents;       // first DoF of every halo entity
+  const HaloBlock* halo_blocks;
+  const int32_t* halo_pos;  // per foreign slot: position in the halo buffer
+  int n_halo;                     // blocks of the halo pass
   int k;
   int tc;
   int max_local;

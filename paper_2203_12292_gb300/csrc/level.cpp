@@ -201,6 +201,7 @@ void build_level(const Octree& mesh, int k, int tile_cells, int LM, LevelHost& L
   L.max_local = 0;
   L.max_sub = 0;
   std::vector<int32_t> lstart_of(ne, -1);
+  std::vector<int32_t> fent, fpos;  // every foreign entity of every tile: entity, first foreign slot
   for (int t = 0; t < nt; ++t) {
     const int c0 = t * tile_cells, c1 = std::min(nc, c0 + tile_cells);
     TileInfo& T = L.tiles[t];
@@ -249,6 +250,8 @@ void build_level(const Octree& mesh, int k, int tile_cells, int LM, LevelHost& L
     for (int32_t e : fgn) {
       lstart_of[e] = local_next;
       local_next += endofs[e];
+      fent.push_back(e);
+      fpos.push_back((int32_t)L.foreign.size());
       for (int q = 0; q < endofs[e]; ++q) L.foreign.push_back(estart[e] + q);
     }
     T.n_foreign = local_next - T.n_owned;
@@ -370,30 +373,52 @@ void build_level(const Octree& mesh, int k, int tile_cells, int LM, LevelHost& L
   L.n_free = next;
   for (int e = 0; e < ne; ++e)
     if (estart[e] < 0) throw std::runtime_error("entity without an owner tile");
-  // halo: the foreign slots of every DoF, grouped by DoF in slot order
+  // Halo.  The tiles that contribute to a DoF contribute to its whole entity, so
+  // the pass that adds the slots needs one word per entity (about 6 DoFs at k =
+  // 4) instead of a DoF index and a slot offset per DoF: entities sorted into
+  // sections of equal (DoFs, contributing tiles), the slots of a DoF next to each
+  // other in tile order.  The blocks of all sections run through the level together
+  // (sorted by their first DoF), so a sector that two of them touch is still in L2.
   {
-    const int64_t nf = (int64_t)L.foreign.size();
-    std::vector<int32_t> order(nf);
-    for (int64_t i = 0; i < nf; ++i) order[i] = (int32_t)i;
-    std::stable_sort(order.begin(), order.end(),
-                     [&](int32_t a2, int32_t b2) { return L.foreign[a2] < L.foreign[b2]; });
-    L.halo_dofs.clear();
-    L.halo_ptr.assign(1, 0);
-    L.halo_src.assign(nf, 0);
-    for (int64_t i = 0; i < nf; ++i) {
-      const int32_t g = L.foreign[order[i]];
-      if (L.halo_dofs.empty() || L.halo_dofs.back() != g) {
-        if (!L.halo_dofs.empty()) L.halo_ptr.push_back((int32_t)i);
-        L.halo_dofs.push_back(g);
-      }
-      L.halo_src[i] = order[i];
+    std::vector<int32_t> cnt(ne, 0), base(ne, 0), seen(ne, 0), ents;
+    int cmax = 0;
+    for (int32_t e : fent) {
+      if (cnt[e]++ == 0) ents.push_back(e);
+      cmax = std::max(cmax, (int)cnt[e]);
     }
-    L.halo_ptr.push_back((int32_t)nf);
-    if (L.halo_dofs.empty()) L.halo_ptr.assign(1, 0);
-    // tiles write each foreign contribution straight to its DoF-ordered position, so that
-    // the halo pass reads every DoF's slots contiguously
-    L.halo_pos.assign(nf, 0);
-    for (int64_t e = 0; e < nf; ++e) L.halo_pos[L.halo_src[e]] = (int32_t)e;
+    std::sort(ents.begin(), ents.end(), [&](int32_t x, int32_t y) { return estart[x] < estart[y]; });
+    L.halo_ents.clear();
+    L.halo_blocks.clear();
+    L.n_halo_dofs = 0;
+    int ndmax = 1;
+    for (int32_t e : ents) ndmax = std::max(ndmax, (int)endofs[e]);
+    std::vector<std::vector<int32_t>> sec((size_t)(ndmax + 1) * (cmax + 1));  // by DoFs and tiles
+    for (int32_t e : ents) sec[(size_t)endofs[e] * (cmax + 1) + cnt[e]].push_back(e);
+    int32_t slot = 0;
+    for (int nd = ndmax; nd >= 1; --nd)
+      for (int c = 1; c <= cmax; ++c) {
+        const auto& v = sec[(size_t)nd * (cmax + 1) + c];
+        const int per = std::max(1, HALO_BLOCK_DOFS / nd);
+        for (size_t i = 0; i < v.size(); i += per) {
+          const int m = (int)std::min<size_t>(per, v.size() - i);
+          L.halo_blocks.push_back(HaloBlock{(int32_t)L.halo_ents.size(), m * nd, nd, c, slot, (65536 + nd - 1) / nd, {0, 0}});
+          for (int j = 0; j < m; ++j) {
+            base[v[i + j]] = slot;
+            slot += nd * c;
+            L.halo_ents.push_back(estart[v[i + j]]);
+          }
+          L.n_halo_dofs += (int64_t)m * nd;
+        }
+      }
+    std::sort(L.halo_blocks.begin(), L.halo_blocks.end(), [&](const HaloBlock& x, const HaloBlock& y) {
+      return L.halo_ents[x.ent0] < L.halo_ents[y.ent0];
+    });
+    L.halo_pos.assign(L.foreign.size(), 0);
+    for (size_t i = 0; i < fent.size(); ++i) {
+      const int32_t e = fent[i];
+      const int s = seen[e]++;
+      for (int q = 0; q < endofs[e]; ++q) L.halo_pos[fpos[i] + q] = base[e] + q * cnt[e] + s;
+    }
   }
   // global starts and transfer ownership (first non-hanging reference wins)
   L.gstart.assign((size_t)nc * NSLOT, -1);
@@ -500,20 +525,32 @@ void validate_level(const LevelHost& L) {
         }
       }
   }
-  // halo: every foreign slot appears exactly once, grouped under its DoF
+  // halo: every foreign slot has a position of its own, and the blocks of the halo
+  // pass find the slots of every DoF, in slot (tile) order
   const int64_t nf = (int64_t)L.foreign.size();
-  std::vector<char> hit(nf, 0);
-  const int64_t nh = (int64_t)L.halo_dofs.size();
-  if ((int64_t)L.halo_ptr.size() != nh + 1 || L.halo_ptr[0] != 0 || L.halo_ptr[nh] != nf) fail("halo offsets");
-  for (int64_t u = 0; u < nh; ++u) {
-    if (u > 0 && L.halo_dofs[u] <= L.halo_dofs[u - 1]) fail("halo DoFs not increasing");
-    for (int32_t e = L.halo_ptr[u]; e < L.halo_ptr[u + 1]; ++e) {
-      const int32_t src = L.halo_src[e];
-      if (src < 0 || src >= nf || hit[src]) fail("halo slot used twice or out of range");
-      hit[src] = 1;
-      if (L.foreign[src] != L.halo_dofs[u]) fail("halo slot under the wrong DoF");
-    }
+  std::vector<int32_t> at(nf, -1);
+  for (int64_t f = 0; f < nf; ++f) {
+    const int32_t p = L.halo_pos[f];
+    if (p < 0 || p >= nf || at[p] >= 0) fail("halo position used twice or out of range");
+    at[p] = (int32_t)f;
   }
+  int64_t covered = 0, n_halo = 0;
+  for (const HaloBlock& h : L.halo_blocks) {
+    if (h.n < 1 || h.n > HALO_BLOCK_DOFS || h.nd < 1 || h.n % h.nd || h.c < 1) fail("halo block");
+    if (h.ent0 < 0 || h.ent0 + h.n / h.nd > (int64_t)L.halo_ents.size()) fail("halo block beyond the entities");
+    for (int i = 0; i < h.n; ++i) {
+      if (((i * h.inv) >> 16) != i / h.nd) fail("halo division");
+      const int32_t g = L.halo_ents[h.ent0 + i / h.nd] + i % h.nd;
+      for (int e = 0; e < h.c; ++e) {
+        const int64_t p = (int64_t)h.slot0 + (int64_t)i * h.c + e;
+        if (p < 0 || p >= nf || L.foreign[at[p]] != g) fail("halo slot under the wrong DoF");
+        if (e > 0 && at[p] <= at[p - 1]) fail("halo slots of a DoF out of order");
+      }
+      covered += h.c;
+    }
+    n_halo += h.n;
+  }
+  if (covered != nf || n_halo != L.n_halo_dofs) fail("halo slots not covered");
   // the lane kernels' order of accumulation (tiles of at most 32 cells).  Node (a, b, c) of the
   // cell in lane j adds to tile-local DoF ls[slot][j] / 4 + offset (absent slots: the zero region).
   //  * tiles without hanging cells (fp32 kernel, warp c holds plane c): the planes whose nodes
