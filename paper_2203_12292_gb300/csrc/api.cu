@@ -514,6 +514,13 @@ void vcycle_ls_body(Handle& H) {
   }
 }
 
+// the captured graphs belong to the levels' present operators, smoothers and timers
+void reset_graphs(Handle& H) {
+  H.g_core.reset();
+  H.g_a.reset();
+  H.g_cg.reset();
+}
+
 // the V-cycle on the level vectors (b -> x of the finest level)
 void vcycle_core(Handle& H) {
   const int top = H.top_mg;
@@ -673,8 +680,7 @@ void setup_numerics(Handle& H) {
     ck_launches("eigenvalue estimate");
   }
   setup_dense(H);
-  H.g_core.reset();
-  H.g_a.reset();
+  reset_graphs(H);
 }
 
 // per DoF the positions of its entries in the cell vectors (node n of cell c at
@@ -899,7 +905,8 @@ void setup_handle(Handle& H, const std::vector<Octree>& gc_meshes, int lmax, con
     }
     ck(cudaStreamSynchronize(H.stream), "upload");  // the host vectors are freed on return
   }
-  H.scratch.alloc(DOT_BLOCKS * sizeof(double));
+  H.scratch.alloc(DOT_SCRATCH_BYTES);
+  ck(cudaMemsetAsync(H.scratch.p, 0, DOT_SCRATCH_BYTES, H.stream), "memset");
   H.scal.alloc(16 * sizeof(double));
   ck(cudaMemsetAsync(H.scal.p, 0, 16 * sizeof(double), H.stream), "memset");
   setup_numerics(H);
@@ -909,6 +916,7 @@ void setup_handle(Handle& H, const std::vector<Octree>& gc_meshes, int lmax, con
   H.cg_q.alloc(nf * sizeof(double));
   H.cg_z.alloc(nf * sizeof(double));
   H.cg_x.alloc(nf * sizeof(double));
+  H.cg_out.alloc(4 * sizeof(double));
   ck(cudaStreamSynchronize(H.stream), "setup");
   ck_launches("setup");
 }
@@ -1078,8 +1086,7 @@ int gcmg_set_profiling(gcmg_handle* h, int on) {
     Profiler& P = h->h.prof;
     prof_flush(h->h);
     P.on = on != 0;
-    h->h.g_core.reset();
-    h->h.g_a.reset();
+    reset_graphs(h->h);
     P.nlev = (int)h->h.lev.size();
     P.ms.assign((size_t)P.nlev * NSTAGE, 0.0);
     P.cnt.assign((size_t)P.nlev * NSTAGE, 0);
@@ -1348,7 +1355,7 @@ int gcmg_set_lambda(gcmg_handle* h, int level, double lam) {
     check_level(h->h, level);
     h->h.lev[level]->lam = lam;
     if (level <= h->h.dense_top) h->h.dense_ok = false;  // that interval is not the matrix's: level by level from now on
-    h->h.g_core.reset();
+    reset_graphs(h->h);
   });
 }
 
@@ -1434,6 +1441,25 @@ int gcmg_cg_solve(gcmg_handle* h, const double* b, double* x, double rtol, int m
     double* S = H.scal.as<double>();
     cudaStream_t s = H.stream;
     gcmg_solve_stats st{0, 0.0, 0.0, GCMG_OK};
+    const bool flexible = any_learned(H);
+    if (H.use_graphs && !H.prof.on && !flexible) {  // the whole loop as one graph launch
+      if (!H.g_cg.exec) cg_capture(H);
+      launch_cg_limits(S, maxit, rtol, s);
+      ck(cudaMemcpyAsync(r, b, n * sizeof(double), cudaMemcpyDeviceToDevice, s), "copy");
+      ck(cudaGraphLaunch(H.g_cg.exec, s), "graph launch");
+      ck(cudaMemcpyAsync(x, xi, n * sizeof(double), cudaMemcpyDeviceToDevice, s), "copy");
+      double out[4];
+      ck(cudaMemcpyAsync(out, H.cg_out.p, sizeof(out), cudaMemcpyDeviceToHost, s), "scalars");
+      ck(cudaStreamSynchronize(s), "cg");
+      const int its = (int)out[0];
+      note_launches((int)(H.g_cg.kernels + its * H.cg_body_kernels));
+      const double nb = std::sqrt(out[2]);
+      st = gcmg_solve_stats{its, nb, nb == 0.0 ? 0.0 : std::sqrt(out[1]) / nb, (int)out[3]};
+      status = st.status;
+      ck_launches("cg");
+      if (stats) *stats = st;
+      return;
+    }
     launch_zero(true, xi, n, s);
     ck(cudaMemcpyAsync(r, b, n * sizeof(double), cudaMemcpyDeviceToDevice, s), "copy");
     const double nb = std::sqrt(dot_host(H, r, r, n));
@@ -1455,10 +1481,9 @@ int gcmg_cg_solve(gcmg_handle* h, const double* b, double* x, double rtol, int m
       vmult(H, top, true, p, q, GCMG_STAGE_CG_VMULT);
       const int pr = prof_begin(H, top, GCMG_STAGE_CG_VECTOR);
       launch_dot(p, q, n, H.scratch.as<double>(), S, 0, DOT_ALPHA, H.stream);
-      launch_cg_update_xr(xi, r, p, q, S, n, H.scratch.as<double>(), S, H.stream, r32);
+      launch_cg_update_xr(xi, r, p, q, S, n, H.scratch.as<double>(), H.stream, r32);
       prof_end(H, pr);
     };
-    const bool flexible = any_learned(H);
     const bool fused = r32 && !flexible;
     vcycle(H, r, z);
     launch_dot(r, z, n, H.scratch.as<double>(), S, 0, DOT_STORE, s);  // rz
@@ -1638,7 +1663,7 @@ int gcmg_set_smoother(gcmg_handle* h, int level, int kind, const gcmg_mlp* net) 
       if (!H.lscratch.p) H.lscratch.alloc((2 * DOT_BLOCKS + 2) * sizeof(double));
     }
     L.smoother = kind;
-    H.g_core.reset();
+    reset_graphs(H);
   });
 }
 
@@ -1769,8 +1794,7 @@ int gcmg_set_graphs(gcmg_handle* h, int on) {
   return guarded([&] {
     if (!h) throw Error(GCMG_ERR_ARG, "null handle");
     h->h.use_graphs = on != 0;
-    h->h.g_core.reset();
-    h->h.g_a.reset();
+    reset_graphs(h->h);
   });
 }
 

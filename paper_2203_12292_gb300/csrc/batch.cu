@@ -57,6 +57,7 @@ struct gcmg_batch {
   int key_maxit = -1;
   gcmg::DevBuf stats;  // per problem: iterations, rr, |b|^2, status
   std::vector<long long> pro_kernels, body_kernels;
+  std::vector<char> first_in_prologue;  // flexible CG: the first iteration's kernels are the prologue's
   ~gcmg_batch() {
     if (exec) cudaGraphExecDestroy(exec);
     if (cap) cudaStreamDestroy(cap);
@@ -151,7 +152,7 @@ void vcycle_kernels(Handle& H, const double* b, double* x) {
 void op_half(Handle& H, const CgVecs& v) {
   vmult(H, (int)H.lev.size() - 1, true, v.p, v.q, GCMG_STAGE_CG_VMULT);
   launch_dot(v.p, v.q, v.n, v.scratch, v.S, 0, DOT_ALPHA, H.stream);
-  launch_cg_update_xr(v.x, v.r, v.p, v.q, v.S, v.n, v.scratch, v.S, H.stream);
+  launch_cg_update_xr(v.x, v.r, v.p, v.q, v.S, v.n, v.scratch, H.stream);
 }
 
 void cg_prologue(Handle& H, const double* b, double rtol2, int maxit, cudaGraphConditionalHandle hc) {
@@ -200,6 +201,100 @@ long long record(Handle& H, cudaStream_t cs, F&& body) {
   return k;
 }
 
+// the V-cycle's own vectors in CG: r is written into its right-hand side by the
+// update of r, and z is read where the V-cycle leaves it (no copies or casts in
+// the loop; the same values)
+struct CgIo {
+  void* rb;
+  bool rb64;
+  const void* z;
+  bool z64;
+};
+CgIo cg_io(Handle& H) {
+  LevelDev& F = *H.lev.back();
+  if (H.ls) return CgIo{F.w64a.p, true, F.w64b.p, true};
+  return CgIo{F.b.p, !F.fp32, F.x.p, !F.fp32};
+}
+
+// before the loop: x = p = 0, r = b (b null: r holds it), |b|^2
+void cg_graph_prologue(Handle& H, const double* b, cudaGraphConditionalHandle hc) {
+  const CgVecs v = vecs(H);
+  const CgIo io = cg_io(H);
+  launch_zero(true, v.x, v.n, H.stream);
+  launch_zero(true, v.p, v.n, H.stream);
+  if (b) launch_copy(b, v.r, v.n, H.stream);
+  if (io.rb64)
+    launch_copy(v.r, static_cast<double*>(io.rb), v.n, H.stream);
+  else
+    launch_cast(false, v.r, io.rb, v.n, H.stream);
+  launch_dot(v.r, v.r, v.n, v.scratch, v.S, 7, DOT_STORE, H.stream);
+  launch_cg_start(hc, v.S, H.stream);
+}
+
+// one iteration; the update of x and r ends it and sets the loop's condition
+void cg_graph_body(Handle& H, cudaGraphConditionalHandle hc) {
+  const CgVecs v = vecs(H);
+  const CgIo io = cg_io(H);
+  if (H.ls)
+    vcycle_ls_body(H);
+  else
+    vcycle_level(H, H.top_mg);
+  if (io.z64) {
+    const double* z = static_cast<const double*>(io.z);
+    launch_dot(v.r, z, v.n, v.scratch, v.S, 0, DOT_BETA_FIRST, H.stream);
+    launch_cg_update_p(v.p, z, v.S, v.n, H.stream);
+  } else {
+    const float* z = static_cast<const float*>(io.z);
+    launch_dot(v.r, z, v.n, v.scratch, v.S, 0, DOT_BETA_FIRST, H.stream);
+    launch_cg_update_p(v.p, z, v.S, v.n, H.stream);
+  }
+  vmult(H, (int)H.lev.size() - 1, true, v.p, v.q, GCMG_STAGE_CG_VMULT);
+  launch_dot(v.p, v.q, v.n, v.scratch, v.S, 0, DOT_ALPHA, H.stream);
+  launch_cg_update_xr_loop(v.x, v.r, v.p, v.q, v.S, v.n, v.scratch, H.stream, io.rb, io.rb64, hc);
+}
+
+// one CG as part of the graph G, captured on stream cs: before the loop, a WHILE
+// node whose body is one iteration, after the loop; kernels outside and per
+// iteration
+template <typename PRO, typename BODY, typename EPI>
+void add_loop(Handle& H, cudaGraph_t G, cudaStream_t cs, PRO&& pro, BODY&& body, EPI&& epi, long long& outside,
+              long long& inside) {
+  cudaGraphConditionalHandle hc = 0;
+  cudaGraph_t g_out = nullptr;
+  ck(cudaStreamBeginCaptureToGraph(cs, G, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed), "capture");
+  ck(cudaGraphConditionalHandleCreate(&hc, G, 0, 0), "conditional handle");
+  outside = record(H, cs, [&] { pro(hc); });
+  cudaStreamCaptureStatus st;
+  const cudaGraphNode_t* deps = nullptr;
+  const cudaGraphEdgeData* edges = nullptr;
+  size_t nd = 0;
+  ck(cudaStreamGetCaptureInfo(cs, &st, nullptr, nullptr, &deps, &edges, &nd), "capture info");
+  cudaGraphNodeParams prm = {};
+  prm.type = cudaGraphNodeTypeConditional;
+  prm.conditional.handle = hc;
+  prm.conditional.type = cudaGraphCondTypeWhile;
+  prm.conditional.size = 1;
+  cudaGraphNode_t wn;
+  ck(cudaGraphAddNode(&wn, G, deps, edges, nd, &prm), "while node");
+  cudaGraph_t body_graph = prm.conditional.phGraph_out[0];
+  ck(cudaStreamUpdateCaptureDependencies(cs, &wn, nullptr, 1, cudaStreamSetCaptureDependencies), "capture dependencies");
+  outside += record(H, cs, epi);
+  ck(cudaStreamEndCapture(cs, &g_out), "end capture");
+  ck(cudaStreamBeginCaptureToGraph(cs, body_graph, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed), "capture");
+  inside = record(H, cs, [&] { body(hc); });
+  ck(cudaStreamEndCapture(cs, &g_out), "end capture");
+}
+
+// an unfinished capture of cs is ended and G destroyed
+void drop_capture(cudaStream_t cs, cudaGraph_t G) {
+  cudaStreamCaptureStatus st;
+  if (cudaStreamIsCapturing(cs, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone) {
+    cudaGraph_t g = nullptr;
+    cudaStreamEndCapture(cs, &g);
+  }
+  cudaGraphDestroy(G);
+}
+
 void build_graph(gcmg_batch& B, const double* const* b, double* const* x, double rtol, int maxit) {
   if (B.exec) cudaGraphExecDestroy(B.exec);
   B.exec = nullptr;
@@ -210,59 +305,48 @@ void build_graph(gcmg_batch& B, const double* const* b, double* const* x, double
   ck(cudaGraphCreate(&G, 0), "graph create");
   B.pro_kernels.assign(np, 0);
   B.body_kernels.assign(np, 0);
+  B.first_in_prologue.assign(np, 0);
   double* stats = B.stats.as<double>();
   try {
     for (int i = 0; i < np; ++i) {
       Handle& H = B.probs[i]->h;
       const CgVecs v = vecs(H);
-      cudaGraph_t body = nullptr;
-      cudaGraphConditionalHandle hc = 0;
-      ck(cudaStreamBeginCaptureToGraph(cs, G, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed), "capture");
       if (v.n == 0) {
+        cudaGraph_t g_out = nullptr;
+        ck(cudaStreamBeginCaptureToGraph(cs, G, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed), "capture");
         B.pro_kernels[i] = record(H, cs, [&] {
           launch_scalar_set(v.S, 7, 0.0, cs);
           launch_scalar_set(v.S, 8, 0.0, cs);
           launch_cg_stats(v.S, rtol2, stats + 4 * i, cs);
         });
-      } else {
-        ck(cudaGraphConditionalHandleCreate(&hc, G, 0, 0), "conditional handle");
-        B.pro_kernels[i] = record(H, cs, [&] { cg_prologue(H, b[i], rtol2, maxit, hc); });
-        // the WHILE node after the prologue, then the epilogue after it
-        cudaStreamCaptureStatus st;
-        const cudaGraphNode_t* deps = nullptr;
-        const cudaGraphEdgeData* edges = nullptr;
-        size_t nd = 0;
-        ck(cudaStreamGetCaptureInfo(cs, &st, nullptr, nullptr, &deps, &edges, &nd), "capture info");
-        cudaGraphNodeParams prm = {};
-        prm.type = cudaGraphNodeTypeConditional;
-        prm.conditional.handle = hc;
-        prm.conditional.type = cudaGraphCondTypeWhile;
-        prm.conditional.size = 1;
-        cudaGraphNode_t wn;
-        ck(cudaGraphAddNode(&wn, G, deps, edges, nd, &prm), "while node");
-        body = prm.conditional.phGraph_out[0];
-        ck(cudaStreamUpdateCaptureDependencies(cs, &wn, nullptr, 1, cudaStreamSetCaptureDependencies),
-           "capture dependencies");
-        B.pro_kernels[i] += record(H, cs, [&] {
-          launch_copy(v.x, x[i], v.n, cs);
-          launch_cg_stats(v.S, rtol2, stats + 4 * i, cs);
-        });
-      }
-      cudaGraph_t g_out = nullptr;
-      ck(cudaStreamEndCapture(cs, &g_out), "end capture");
-      if (body) {
-        ck(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed), "capture");
-        B.body_kernels[i] = record(H, cs, [&] { cg_body(H, rtol2, maxit, hc); });
         ck(cudaStreamEndCapture(cs, &g_out), "end capture");
+      } else if (any_learned(H)) {  // flexible CG: its first iteration runs before the loop
+        B.first_in_prologue[i] = 1;
+        add_loop(
+            H, G, cs, [&](cudaGraphConditionalHandle hc) { cg_prologue(H, b[i], rtol2, maxit, hc); },
+            [&](cudaGraphConditionalHandle hc) { cg_body(H, rtol2, maxit, hc); },
+            [&] {
+              launch_copy(v.x, x[i], v.n, cs);
+              launch_cg_stats(v.S, rtol2, stats + 4 * i, cs);
+            },
+            B.pro_kernels[i], B.body_kernels[i]);
+      } else {
+        add_loop(
+            H, G, cs,
+            [&](cudaGraphConditionalHandle hc) {
+              launch_cg_limits(v.S, maxit, rtol, cs);
+              cg_graph_prologue(H, b[i], hc);
+            },
+            [&](cudaGraphConditionalHandle hc) { cg_graph_body(H, hc); },
+            [&] {
+              launch_copy(v.x, x[i], v.n, cs);
+              launch_cg_result(v.S, stats + 4 * i, cs);
+            },
+            B.pro_kernels[i], B.body_kernels[i]);
       }
     }
   } catch (...) {
-    cudaStreamCaptureStatus st;
-    if (cudaStreamIsCapturing(cs, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone) {
-      cudaGraph_t g = nullptr;
-      cudaStreamEndCapture(cs, &g);
-    }
-    cudaGraphDestroy(G);
+    drop_capture(cs, G);
     throw;
   }
   const cudaError_t e = cudaGraphInstantiate(&B.exec, G, 0);
@@ -406,6 +490,27 @@ double time_vmult(Handle& H, bool fp64, int reps) {
 }
 
 }  // namespace
+
+void cg_capture(Handle& H) {
+  H.g_cg.reset();
+  if (!H.cap_stream) ck(cudaStreamCreateWithFlags(&H.cap_stream, cudaStreamNonBlocking), "stream");
+  cudaGraph_t G = nullptr;
+  ck(cudaGraphCreate(&G, 0), "graph create");
+  const CgVecs v = vecs(H);
+  try {
+    add_loop(
+        H, G, H.cap_stream, [&](cudaGraphConditionalHandle hc) { cg_graph_prologue(H, nullptr, hc); },
+        [&](cudaGraphConditionalHandle hc) { cg_graph_body(H, hc); },
+        [&] { launch_cg_result(v.S, H.cg_out.as<double>(), H.stream); }, H.g_cg.kernels, H.cg_body_kernels);
+  } catch (...) {
+    drop_capture(H.cap_stream, G);
+    throw;
+  }
+  const cudaError_t e = cudaGraphInstantiate(&H.g_cg.exec, G, 0);
+  cudaGraphDestroy(G);
+  ck(e, "graph instantiate");
+}
+
 }  // namespace gcmg
 
 using namespace gcmg;
@@ -554,7 +659,7 @@ int gcmg_batch_cg_solve(gcmg_batch* b, const double* const* rhs, double* const* 
     long long kernels = 0;
     for (int i = 0; i < np; ++i) {
       const int it = (int)h[4 * i];
-      kernels += b->pro_kernels[i] + (it > 1 ? (long long)(it - 1) * b->body_kernels[i] : 0);
+      kernels += b->pro_kernels[i] + (long long)std::max(0, it - b->first_in_prologue[i]) * b->body_kernels[i];
       if (stats) {
         const double nb2 = h[4 * i + 2];
         stats[i] = gcmg_solve_stats{it, std::sqrt(nb2), nb2 > 0 ? std::sqrt(h[4 * i + 1] / nb2) : 0.0,

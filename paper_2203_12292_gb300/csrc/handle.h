@@ -105,6 +105,8 @@ struct Handle {
   bool use_graphs = true;
   GraphRec* capturing = nullptr;
   GraphRec g_core, g_a;
+  GraphRec g_cg;                // a whole CG solve; kernels: outside its loop
+  long long cg_body_kernels = 0;  // per iteration
   Profiler prof;
   gcmg_config cfg{};
   std::vector<std::unique_ptr<LevelDev>> lev;
@@ -113,7 +115,7 @@ struct Handle {
   DevBuf Ainv;
   int n0 = 0;
   DevBuf scratch, scal, modes;
-  DevBuf cg_r, cg_p, cg_q, cg_z, cg_x;
+  DevBuf cg_r, cg_p, cg_q, cg_z, cg_x, cg_out;
   DevBuf lscratch;     // inner products of the learned step's Galerkin step length
   // host-buffer operator: the input copy in DoF order on its own stream, overlapped with the tiles
   cudaStream_t copy_stream = nullptr;
@@ -126,6 +128,7 @@ struct Handle {
   ~Handle() {
     g_core.reset();
     g_a.reset();
+    g_cg.reset();
     if (cap_stream) cudaStreamDestroy(cap_stream);
     for (cudaEvent_t e : pipe_ev) cudaEventDestroy(e);
     for (cudaEvent_t e : many_ev)
@@ -150,6 +153,11 @@ void vmult(Handle& H, int l, bool fp64, const void* src, void* dst, int stage = 
 // pending: the level's right-hand side is still in its cell vectors (a restricted residual)
 void vcycle_level(Handle& H, int l, bool pending = false);
 bool any_learned(const Handle& H);
+void reset_graphs(Handle& H);
+void vcycle_ls_body(Handle& H);
+// g_cg: CG of the handle as one graph (batch.cu); limits and right-hand side
+// (cg_r) are set before a launch
+void cg_capture(Handle& H);
 
 }  // namespace gcmg
 

@@ -219,9 +219,10 @@ void launch_xpby(double* p, const double* z, double beta, int64_t n, cudaStream_
 void launch_coarse_solve(bool fp64, const double* Ainv, int n, const void* b, void* x, cudaStream_t s);
 
 // deterministic fp64 dot products: partial sums into `scratch` (DOT_BLOCKS
-// doubles), then one block combines them in fixed order
+// doubles and a counter, zero between launches), combined in fixed order
 constexpr int DOT_BLOCKS = 304;
-enum DotOp { DOT_STORE = 0, DOT_ALPHA = 1, DOT_BETA = 2, DOT_BETA_FLEX = 3 };
+constexpr size_t DOT_SCRATCH_BYTES = (DOT_BLOCKS + 1) * sizeof(double);
+enum DotOp { DOT_STORE = 0, DOT_ALPHA = 1, DOT_BETA = 2, DOT_BETA_FLEX = 3, DOT_BETA_FIRST = 4 };
 void launch_dot(const double* x, const double* y, int64_t n, double* scratch, double* scal, int slot, int op,
                 cudaStream_t s);
 // the same with y in fp32 (widened exactly: equal to the sums over an fp64 copy of y)
@@ -233,9 +234,19 @@ int64_t dot_noalloc_max_n();
 cudaError_t launch_dot_noalloc(const double* x, const double* y, int64_t n, double* result, cudaStream_t s);
 // CG updates with device scalars: scal[0] = rz, [1] = pq, [2] = rr, [3] = alpha, [4] = beta, [5] = rz_new,
 // [6] = r_{k+1}.z_k of flexible CG
-// r32 != null: r is also written rounded to fp32 (the fp32 V-cycle's right-hand side)
-void launch_cg_update_xr(double* x, double* r, const double* p, const double* q, const double* scal, int64_t n,
-                         double* scratch, double* scal_out, cudaStream_t s, float* r32 = nullptr);
+// rb != null: r is also written into the V-cycle's right-hand side (fp64 or rounded to fp32)
+void launch_cg_update_xr(double* x, double* r, const double* p, const double* q, double* scal, int64_t n,
+                         double* scratch, cudaStream_t s, void* rb = nullptr, bool rb64 = false);
+// CG as a loop inside a graph: further scalars.  cg_limits sets the limits of the
+// next solve, cg_start begins it (|b|^2 in scal[7]), the update of x and r ends
+// an iteration (it sets the WHILE node's condition h), cg_result writes
+// (iterations, rr, |b|^2, status)
+constexpr int CG_ITERATIONS = 8, CG_MAXIT = 9, CG_RTOL = 10, CG_RR = 12;
+void launch_cg_limits(double* scal, int maxit, double rtol, cudaStream_t s);
+void launch_cg_start(cudaGraphConditionalHandle h, double* scal, cudaStream_t s);
+void launch_cg_update_xr_loop(double* x, double* r, const double* p, const double* q, double* scal, int64_t n,
+                              double* scratch, cudaStream_t s, void* rb, bool rb64, cudaGraphConditionalHandle h);
+void launch_cg_result(const double* scal, double* out, cudaStream_t s);
 void launch_cg_update_p(double* p, const double* z, const double* scal, int64_t n, cudaStream_t s);
 void launch_cg_update_p(double* p, const float* z, const double* scal, int64_t n, cudaStream_t s);
 // CG inside a graph: scal[7] = |b|^2, scal[8] = iterations; the check kernel

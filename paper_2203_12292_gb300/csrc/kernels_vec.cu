@@ -202,40 +202,10 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return sh[0];
 }
 
-// reductions of the CG vectors: DOT_BLOCKS blocks of RB threads (two per SM,
-// full occupancy), every thread keeps RU partial sums so that RU loads per
-// array are in flight
+// reductions of the CG vectors: blocks of RB threads (two per SM, full
+// occupancy), every thread keeps RU partial sums so that RU loads per array are
+// in flight (two elements per load measured slower: mixed Q4 solve 22.2 -> 22.5 ms)
 constexpr int RB = 1024, RU = 4;
-
-__device__ __forceinline__ double block_sum_rb(double v, double* sh) {
-  sh[threadIdx.x] = v;
-  __syncthreads();
-  for (int s = RB / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-    __syncthreads();
-  }
-  return sh[0];
-}
-
-// each block sums a fixed contiguous chunk in a fixed order: the result does
-// not depend on scheduling (y in fp32: the fp32 V-cycle's output, widened
-// exactly, so the sums equal those over its fp64 copy)
-template <typename TY>
-__global__ void __launch_bounds__(RB, 2) dot_partial(const double* x, const TY* y, int64_t n, double* part) {
-  pdl_begin();
-  __shared__ double sh[RB];
-  const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-  const int64_t i0 = blockIdx.x * chunk, i1 = min(n, i0 + chunk);
-  double s[RU] = {};
-  int64_t i = i0 + threadIdx.x;
-  for (; i + (RU - 1) * RB < i1; i += RU * RB) {
-#pragma unroll
-    for (int u = 0; u < RU; ++u) s[u] += x[i + u * RB] * (double)y[i + u * RB];
-  }
-  for (; i < i1; i += RB) s[0] += x[i] * (double)y[i];
-  const double v = block_sum_rb((s[0] + s[1]) + (s[2] + s[3]), sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = v;
-}
 
 __global__ void __launch_bounds__(BLOCK) dot_final(const double* part, int np, double* scal, int slot, int op) {
   pdl_begin();
@@ -261,54 +231,8 @@ __global__ void __launch_bounds__(BLOCK) dot_final(const double* part, int np, d
   }
 }
 
-// x += alpha p, r -= alpha q, partial sums of r.r: DOT_BLOCKS blocks of XB
-// threads, XU elements per thread in flight; CAST: r also rounded to fp32
-// into r32 (the fp32 V-cycle's right-hand side)
+// the update of x and r: blocks of XB threads, XU elements per thread in flight
 constexpr int XB = 512, XU = 4;
-
-template <bool CAST>
-__global__ void __launch_bounds__(XB, 2) cg_xr_kernel(double* x, double* r, const double* p, const double* q,
-                                                      const double* scal, int64_t n, double* part, float* r32) {
-  pdl_begin();
-  __shared__ double sh[XB];
-  const double alpha = scal[3];
-  const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-  const int64_t i0 = blockIdx.x * chunk, i1 = min(n, i0 + chunk);
-  double s[XU] = {};
-  int64_t i = i0 + threadIdx.x;
-  for (; i + (XU - 1) * XB < i1; i += XU * XB) {
-    double xv[XU], rv[XU], pv[XU], qv[XU];
-#pragma unroll
-    for (int u = 0; u < XU; ++u) {
-      xv[u] = x[i + u * XB];
-      rv[u] = r[i + u * XB];
-      pv[u] = p[i + u * XB];
-      qv[u] = q[i + u * XB];
-    }
-#pragma unroll
-    for (int u = 0; u < XU; ++u) {
-      x[i + u * XB] = xv[u] + alpha * pv[u];
-      const double ri = rv[u] - alpha * qv[u];
-      r[i + u * XB] = ri;
-      if (CAST) r32[i + u * XB] = (float)ri;
-      s[u] += ri * ri;
-    }
-  }
-  for (; i < i1; i += XB) {
-    x[i] += alpha * p[i];
-    const double ri = r[i] - alpha * q[i];
-    r[i] = ri;
-    if (CAST) r32[i] = (float)ri;
-    s[0] += ri * ri;
-  }
-  sh[threadIdx.x] = (s[0] + s[1]) + (s[2] + s[3]);
-  __syncthreads();
-  for (int h = XB / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) sh[threadIdx.x] += sh[threadIdx.x + h];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
-}
 
 template <typename TZ>
 __global__ void cg_p_kernel(double* p, const TZ* z, const double* scal, int64_t n) {
@@ -563,40 +487,253 @@ void launch_coarse_solve(bool fp64, const double* Ainv, int n, const void* b, vo
     { launch_pdl(coarse_kernel<float>, 1, BLOCK, 0, s, Ainv, n, (const float*)b, (float*)x); note_launches(1); }
 }
 
+// ---------------------------------------------------------------------------
+// The reductions of CG in one launch: the block that finishes last adds the
+// partial sums, in block order, and forms the scalars.  One block per
+// REDUCE_MIN elements up to DOT_BLOCKS (a vector that small is one block: no
+// counter, no second pass); the blocks' chunks are fixed, so repeated calls give
+// the same bits.  The recorded launches of the persistent batch keep the kernels
+// above (256 threads, partial sums and their addition as two operations).
+// Q2 octant solve (6,407 DoFs), with the loop as one graph: 1.06 -> 0.83 ms; batch of
+// 16 problems 8.98 -> 7.26 ms.
+// ---------------------------------------------------------------------------
+namespace {
+
+constexpr int64_t REDUCE_MIN = 8192;
+int reduce_blocks(int64_t n) {
+  return (int)std::min<int64_t>(DOT_BLOCKS, std::max<int64_t>(1, (n + REDUCE_MIN - 1) / REDUCE_MIN));
+}
+
+// sum over a block of NT threads in a fixed order, in thread 0
+template <int NT>
+__device__ __forceinline__ double block_sum_fixed(double v, double* sh) {
+#pragma unroll
+  for (int h = 16; h > 0; h >>= 1) v += __shfl_down_sync(0xffffffffu, v, h);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    v = threadIdx.x < NT / 32 ? sh[threadIdx.x] : 0.0;
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) v += __shfl_down_sync(0xffffffffu, v, h);
+  }
+  return v;
+}
+
+// v: the thread's part; fin(total) runs once, in one thread.  part: DOT_BLOCKS
+// partial sums, then the counter of finished blocks (zero between launches)
+template <int NT, typename F>
+__device__ __forceinline__ void reduce_finish(double v, double* part, F&& fin) {
+  __shared__ double sh[32];
+  __shared__ bool last;
+  v = block_sum_fixed<NT>(v, sh);
+  if (gridDim.x > 1) {
+    if (threadIdx.x == 0) {
+      unsigned* done = reinterpret_cast<unsigned*>(part + DOT_BLOCKS);
+      part[blockIdx.x] = v;
+      __threadfence();
+      last = atomicAdd(done, 1u) == gridDim.x - 1;
+      if (last) *done = 0u;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    v = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += NT) v += __ldcg(part + i);
+    v = block_sum_fixed<NT>(v, sh);
+  }
+  if (threadIdx.x == 0) fin(v);
+}
+
+__device__ __forceinline__ void dot_scalars(double s, double* scal, int slot, int op) {
+  if (op == DOT_STORE) {
+    scal[slot] = s;
+  } else if (op == DOT_ALPHA) {  // pq, alpha = rz / pq (0 when pq = 0: zero right-hand side)
+    scal[1] = s;
+    scal[3] = s != 0.0 ? scal[0] / s : 0.0;
+  } else {  // rz_new, beta, rz <- rz_new
+    scal[5] = s;
+    if (op == DOT_BETA)
+      scal[4] = s / scal[0];
+    else if (op == DOT_BETA_FLEX)  // beta = (rz_new - r_{k+1}.z_k) / rz
+      scal[4] = (s - scal[6]) / scal[0];
+    else  // DOT_BETA_FIRST: 0 in the first iteration (p = z)
+      scal[4] = scal[CG_ITERATIONS] == 0.0 ? 0.0 : s / scal[0];
+    scal[0] = s;
+  }
+}
+
+template <typename TY>
+__global__ void __launch_bounds__(RB, 2) dot_kernel(const double* x, const TY* y, int64_t n, double* part, double* scal,
+                                                    int slot, int op) {
+  pdl_begin();
+  const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
+  const int64_t i0 = blockIdx.x * chunk, i1 = min(n, i0 + chunk);
+  double s[RU] = {};
+  int64_t i = i0 + threadIdx.x;
+  for (; i + (RU - 1) * RB < i1; i += RU * RB) {
+#pragma unroll
+    for (int u = 0; u < RU; ++u) s[u] += x[i + u * RB] * (double)y[i + u * RB];
+  }
+  for (; i < i1; i += RB) s[0] += x[i] * (double)y[i];
+  reduce_finish<RB>((s[0] + s[1]) + (s[2] + s[3]), part,
+                    [&](double v) { dot_scalars(v, scal, slot, op); });
+}
+
+// x += alpha p, r -= alpha q, r.r into scal[2]; rb (may be null): r also into the
+// V-cycle's right-hand side.  loop: the iteration's end inside a graph: the
+// iteration is counted and the WHILE node's condition set (see cg_start_kernel)
+template <typename TB>
+__global__ void __launch_bounds__(XB, 2) cg_xr_dot(double* x, double* r, const double* p, const double* q, double* scal,
+                                                   int64_t n, double* part, TB* rb, int loop,
+                                                   cudaGraphConditionalHandle h) {
+  pdl_begin();
+  const double alpha = scal[3];
+  const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
+  const int64_t i0 = blockIdx.x * chunk, i1 = min(n, i0 + chunk);
+  double s[XU] = {};
+  int64_t i = i0 + threadIdx.x;
+  for (; i + (XU - 1) * XB < i1; i += XU * XB) {
+    double xv[XU], rv[XU], pv[XU], qv[XU];
+#pragma unroll
+    for (int u = 0; u < XU; ++u) {
+      xv[u] = x[i + u * XB];
+      rv[u] = r[i + u * XB];
+      pv[u] = p[i + u * XB];
+      qv[u] = q[i + u * XB];
+    }
+#pragma unroll
+    for (int u = 0; u < XU; ++u) {
+      x[i + u * XB] = xv[u] + alpha * pv[u];
+      const double ri = rv[u] - alpha * qv[u];
+      r[i + u * XB] = ri;
+      if (rb) rb[i + u * XB] = (TB)ri;
+      s[u] += ri * ri;
+    }
+  }
+  for (; i < i1; i += XB) {
+    x[i] += alpha * p[i];
+    const double ri = r[i] - alpha * q[i];
+    r[i] = ri;
+    if (rb) rb[i] = (TB)ri;
+    s[0] += ri * ri;
+  }
+  reduce_finish<XB>((s[0] + s[1]) + (s[2] + s[3]), part, [&](double rr) {
+    scal[2] = rr;
+    if (!loop) return;
+    const double it = scal[CG_ITERATIONS] + 1.0;
+    scal[CG_ITERATIONS] = it;
+    const bool good = scal[1] > 0.0 && rr == rr;  // else breakdown: (p, Ap) <= 0 or a NaN
+    if (good) scal[CG_RR] = rr;
+    const bool done = sqrt(rr) <= scal[CG_RTOL] * sqrt(scal[7]);
+    cudaGraphSetConditional(h, good && !done && it < scal[CG_MAXIT] ? 1u : 0u);
+  });
+}
+
+// |b|^2 in scal[7]: the loop runs unless b = 0 or maxit = 0
+__global__ void cg_start_kernel(cudaGraphConditionalHandle h, double* scal) {
+  pdl_begin();
+  scal[CG_ITERATIONS] = 0.0;
+  scal[CG_RR] = scal[7];
+  scal[0] = 0.0;
+  scal[1] = 1.0;
+  scal[2] = scal[7];
+  cudaGraphSetConditional(h, scal[7] != 0.0 && scal[CG_MAXIT] > 0.0 ? 1u : 0u);
+}
+
+__global__ void cg_limits_kernel(double* scal, double maxit, double rtol) {
+  pdl_begin();
+  scal[CG_MAXIT] = maxit;
+  scal[CG_RTOL] = rtol;
+}
+
+// iterations, r.r of the last sound iteration, |b|^2, status
+__global__ void cg_result_kernel(const double* scal, double* out) {
+  pdl_begin();
+  const double rr = scal[2], nb2 = scal[7];
+  double status = GCMG_ERR_NOT_CONVERGED;
+  if (nb2 == 0.0)
+    status = GCMG_OK;
+  else if (!(scal[1] > 0.0) || rr != rr)
+    status = GCMG_ERR_BREAKDOWN;
+  else if (scal[CG_ITERATIONS] > 0.0 && sqrt(rr) <= scal[CG_RTOL] * sqrt(nb2))
+    status = GCMG_OK;
+  out[0] = scal[CG_ITERATIONS];
+  out[1] = scal[CG_RR];
+  out[2] = nb2;
+  out[3] = status;
+}
+
+template <typename TY>
+void dot_any(const double* x, const TY* y, int64_t n, double* scratch, double* scal, int slot, int op, cudaStream_t s) {
+  if (dwl_recording()) {
+    launch_pdl(dot_partial_b<TY>, DOT_BLOCKS, BLOCK, 0, s, x, y, n, scratch);
+    note_launches(1);
+    launch_pdl(dot_final, 1, BLOCK, 0, s, scratch, DOT_BLOCKS, scal, slot, op);
+  } else {
+    launch_pdl(dot_kernel<TY>, reduce_blocks(n), RB, 0, s, x, y, n, scratch, scal, slot, op);
+  }
+  note_launches(1);
+}
+
+template <typename TB>
+void cg_xr_any(double* x, double* r, const double* p, const double* q, double* scal, int64_t n, double* scratch, TB* rb,
+               int loop, cudaGraphConditionalHandle h, cudaStream_t s) {
+  launch_pdl(cg_xr_dot<TB>, reduce_blocks(n), XB, 0, s, x, r, p, q, scal, n, scratch, rb, loop, h);
+  note_launches(1);
+}
+
+}  // namespace
+
 void launch_dot(const double* x, const double* y, int64_t n, double* scratch, double* scal, int slot, int op,
                 cudaStream_t s) {
-  if (dwl_recording())
-    launch_pdl(dot_partial_b<double>, DOT_BLOCKS, BLOCK, 0, s, x, y, n, scratch);
-  else
-    launch_pdl(dot_partial<double>, DOT_BLOCKS, RB, 0, s, x, y, n, scratch);
-  note_launches(1);
-  { launch_pdl(dot_final, 1, BLOCK, 0, s, scratch, DOT_BLOCKS, scal, slot, op); note_launches(1); }
+  dot_any(x, y, n, scratch, scal, slot, op, s);
 }
 
 void launch_dot(const double* x, const float* y, int64_t n, double* scratch, double* scal, int slot, int op,
                 cudaStream_t s) {
-  if (dwl_recording())
-    launch_pdl(dot_partial_b<float>, DOT_BLOCKS, BLOCK, 0, s, x, y, n, scratch);
-  else
-    launch_pdl(dot_partial<float>, DOT_BLOCKS, RB, 0, s, x, y, n, scratch);
-  note_launches(1);
-  { launch_pdl(dot_final, 1, BLOCK, 0, s, scratch, DOT_BLOCKS, scal, slot, op); note_launches(1); }
+  dot_any(x, y, n, scratch, scal, slot, op, s);
 }
 
-void launch_cg_update_xr(double* x, double* r, const double* p, const double* q, const double* scal, int64_t n,
-                         double* scratch, double* scal_out, cudaStream_t s, float* r32) {
+void launch_cg_update_xr(double* x, double* r, const double* p, const double* q, double* scal, int64_t n,
+                         double* scratch, cudaStream_t s, void* rb, bool rb64) {
   if (dwl_recording()) {
+    float* r32 = rb64 ? nullptr : static_cast<float*>(rb);
     if (r32)
-      launch_pdl(cg_xr_b<true>, DOT_BLOCKS, BLOCK, 0, s, x, r, p, q, scal, n, scratch, r32);
+      launch_pdl(cg_xr_b<true>, DOT_BLOCKS, BLOCK, 0, s, x, r, p, q, (const double*)scal, n, scratch, r32);
     else
-      launch_pdl(cg_xr_b<false>, DOT_BLOCKS, BLOCK, 0, s, x, r, p, q, scal, n, scratch, r32);
-  } else if (r32) {
-    launch_pdl(cg_xr_kernel<true>, DOT_BLOCKS, XB, 0, s, x, r, p, q, scal, n, scratch, r32);
-  } else {
-    launch_pdl(cg_xr_kernel<false>, DOT_BLOCKS, XB, 0, s, x, r, p, q, scal, n, scratch, r32);
+      launch_pdl(cg_xr_b<false>, DOT_BLOCKS, BLOCK, 0, s, x, r, p, q, (const double*)scal, n, scratch, r32);
+    note_launches(1);
+    launch_pdl(dot_final, 1, BLOCK, 0, s, scratch, DOT_BLOCKS, scal, 2, DOT_STORE);
+    note_launches(1);
+    return;
   }
+  if (rb64)
+    cg_xr_any(x, r, p, q, scal, n, scratch, static_cast<double*>(rb), 0, cudaGraphConditionalHandle{}, s);
+  else
+    cg_xr_any(x, r, p, q, scal, n, scratch, static_cast<float*>(rb), 0, cudaGraphConditionalHandle{}, s);
+}
+
+void launch_cg_update_xr_loop(double* x, double* r, const double* p, const double* q, double* scal, int64_t n,
+                              double* scratch, cudaStream_t s, void* rb, bool rb64, cudaGraphConditionalHandle h) {
+  if (rb64)
+    cg_xr_any(x, r, p, q, scal, n, scratch, static_cast<double*>(rb), 1, h, s);
+  else
+    cg_xr_any(x, r, p, q, scal, n, scratch, static_cast<float*>(rb), 1, h, s);
+}
+
+void launch_cg_start(cudaGraphConditionalHandle h, double* scal, cudaStream_t s) {
+  launch_pdl(cg_start_kernel, 1, 1, 0, s, h, scal);
   note_launches(1);
-  { launch_pdl(dot_final, 1, BLOCK, 0, s, scratch, DOT_BLOCKS, scal_out, 2, DOT_STORE); note_launches(1); }
+}
+
+void launch_cg_limits(double* scal, int maxit, double rtol, cudaStream_t s) {
+  launch_pdl(cg_limits_kernel, 1, 1, 0, s, scal, (double)maxit, rtol);
+  note_launches(1);
+}
+
+void launch_cg_result(const double* scal, double* out, cudaStream_t s) {
+  launch_pdl(cg_result_kernel, 1, 1, 0, s, scal, out);
+  note_launches(1);
 }
 
 // ---------------------------------------------------------------------------
