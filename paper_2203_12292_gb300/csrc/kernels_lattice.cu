@@ -1,4 +1,4 @@
-// Geometric level transfer (Sec. 3.5, Eqs. 5-7) with one warp per coarse cell.
+// Level transfer (Sec. 3.5, Eqs. 5-7) with one warp per coarse cell.
 //
 // The eight children of a refined coarse cell carry a lattice of (2k+1)^3
 // support points on 5 x 5 x 5 geometric entities (per axis: low vertex, low
@@ -25,6 +25,9 @@
 // Finest Q4 transfer of the octant mesh (18.7 M fine DoFs), fp32:
 // restriction 188 -> 67 us, prolongation 135 -> 44 us (3.7 TB/s of the bytes
 // it needs, 54 % of the copy rate; the entity table adds 19 MB).
+//   The p transfer (one mesh, degree k to floor(k / 2)) is the same with the cell's
+// own nodes as the lattice and its owned slots as the entities: Q4 sphere, fine
+// level, restriction with its halo pass 111 -> 57 us, prolongation 61 -> 43 us.
 #include <algorithm>
 #include <cstring>
 
@@ -50,6 +53,10 @@ __host__ __device__ constexpr int lat_words(int k) { return k == 1 ? 32 : 128; }
 struct LatTables {
   uint32_t pt[KMAX + 1][PT_MAX];  // lattice points: entity | offset << 7 | position << 12
   uint32_t nd[KMAX + 1][ND_MAX];  // cell nodes: slot | offset << 7 | lattice position of the coarse node << 12
+  // p transfer from degree k: the cell's fine nodes entity by entity, its coarse
+  // nodes, positions in the (k+1)^3 lattice
+  uint32_t pf[KMAX + 1][ND_MAX];
+  uint32_t pc[KMAX + 1][32];
 };
 __device__ LatTables g_lat;
 
@@ -75,6 +82,8 @@ __device__ __forceinline__ const LatSweeps<double>& sweeps<double>() {
 template <typename T>
 struct LatArgs {
   const int32_t* ent;  // per coarse cell lat_words(k) words
+  const int32_t* gstart_f;  // p: fine slots and owned slots per cell
+  const uint32_t* own_f;
   const int32_t* gstart_c;
   const uint16_t* mask_c;
   int n_coarse;
@@ -175,20 +184,69 @@ __device__ __forceinline__ void interp_line(T* v, int p) {
   for (int a = 0; a < N; ++a) v[a] = p ? y[K - a] : y[a];
 }
 
-template <int K>
+// lattice of one coarse cell of degree K: the children's (KF = 0, h transfer) or
+// the same cell's nodes of degree KF (p transfer)
+template <int K, int KF = 0>
 struct Lat {
-  static constexpr int N = K + 1, N2 = N * N, N3 = N2 * N, M = 2 * K + 1, M2 = M * M, M3 = M2 * M;
-  static constexpr int ES = lat_words(K), EPL = ES / 32;
+  static constexpr int N = K + 1, N2 = N * N, N3 = N2 * N;
+  static constexpr int M = KF ? KF + 1 : 2 * K + 1, M2 = M * M, M3 = M2 * M;
+  static constexpr int ES = KF ? 32 : lat_words(K), EPL = ES / 32;
   static constexpr int NI = (M3 + 31) / 32, NJ = (N3 + 31) / 32;
   static constexpr int LS = (M3 + 2) & ~1;  // lattice of a warp; position M3 takes the padding points
+  static __device__ __forceinline__ const uint32_t* points() { return KF ? g_lat.pf[KF] : g_lat.pt[K]; }
+  static __device__ __forceinline__ const uint32_t* nodes() { return KF ? g_lat.pc[KF] : g_lat.nd[K]; }
+  // lane's entity words of coarse cell c (p: the cell's owned slots)
+  template <typename T>
+  static __device__ __forceinline__ void words(const LatArgs<T>& A, int c, int lane, int32_t* en) {
+    if constexpr (KF == 0) {
+#pragma unroll
+      for (int i = 0; i < EPL; ++i) en[i] = A.ent[(size_t)c * ES + lane + 32 * i];
+    } else {
+      en[0] = -1;
+      if (lane < NSLOT && ((A.own_f[c] >> lane) & 1u)) en[0] = A.gstart_f[(size_t)c * NSLOT + lane];
+    }
+  }
+  // one line down (M -> N values) and up
+  template <typename T>
+  static __device__ __forceinline__ void down(T* v) {
+    if constexpr (KF == 0) {
+      line_restrict<K>(v);
+    } else {
+      T o[N];
+#pragma unroll
+      for (int a = 0; a < N; ++a) {
+        o[a] = tab<T>(KF).Pp[0][a] * v[0];
+#pragma unroll
+        for (int i = 1; i < M; ++i) o[a] += tab<T>(KF).Pp[i][a] * v[i];
+      }
+#pragma unroll
+      for (int a = 0; a < N; ++a) v[a] = o[a];
+    }
+  }
+  template <typename T>
+  static __device__ __forceinline__ void up(T* v) {
+    if constexpr (KF == 0) {
+      line_prolong<K>(v);
+    } else {
+      T o[M];
+#pragma unroll
+      for (int i = 0; i < M; ++i) {
+        o[i] = tab<T>(KF).Pp[i][0] * v[0];
+#pragma unroll
+        for (int a = 1; a < N; ++a) o[i] += tab<T>(KF).Pp[i][a] * v[a];
+      }
+#pragma unroll
+      for (int i = 0; i < M; ++i) v[i] = o[i];
+    }
+  }
 };
 
 // shared memory: lane records, point tables, entity starts, then the cell
 // buffer, then the warps' lattices; the tile's accumulator takes the lattices'
 // place once every cell of the tile has been reduced
-template <int K, typename T>
+template <int K, typename T, int KF>
 struct RestrictSmem {
-  using L = Lat<K>;
+  using L = Lat<K, KF>;
   static constexpr size_t pt = sizeof(LaneTile) + sizeof(LaneHang);
   static constexpr size_t nd = pt + (size_t)L::NI * 32 * 4;
   static constexpr size_t ent = nd + (size_t)L::NJ * 32 * 4;
@@ -199,11 +257,11 @@ struct RestrictSmem {
   }
 };
 
-template <int K, typename T>
+template <int K, typename T, int KF>
 __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
-  using L = Lat<K>;
-  using SM = RestrictSmem<K, T>;
-  constexpr int N = L::N, N2 = L::N2, N3 = L::N3, M = L::M, M2 = L::M2, M3 = L::M3;
+  using L = Lat<K, KF>;
+  using SM = RestrictSmem<K, T, KF>;
+  constexpr int N = L::N, N2 = L::N2, N3 = L::N3, M = L::M, M2 = L::M2;
   constexpr int NT = WPB * 32;
   extern __shared__ __align__(16) unsigned char smem[];
   LaneTile* st = reinterpret_cast<LaneTile*>(smem);
@@ -224,14 +282,11 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
     const uint4* gh = reinterpret_cast<const uint4*>(A.lh + blockIdx.x);
     uint4* sh = reinterpret_cast<uint4*>(hg);
     for (int i = threadIdx.x; i < (int)(sizeof(LaneHang) / 16); i += NT) cp_async16(sh + i, gh + i);
-    for (int i = threadIdx.x; i < L::NI * 32; i += NT) cp_async(s_pt + i, &g_lat.pt[K][i]);
-    for (int i = threadIdx.x; i < L::NJ * 32; i += NT) cp_async(s_nd + i, &g_lat.nd[K][i]);
+    for (int i = threadIdx.x; i < L::NI * 32; i += NT) cp_async(s_pt + i, L::points() + i);
+    for (int i = threadIdx.x; i < L::NJ * 32; i += NT) cp_async(s_nd + i, L::nodes() + i);
   }
   int32_t en[L::EPL];  // the next cell's entity words
-  const int32_t* ep = A.ent + (size_t)ti.cell_begin * L::ES;
-  if (w < nc)
-#pragma unroll
-    for (int i = 0; i < L::EPL; ++i) en[i] = ep[w * L::ES + lane + 32 * i];
+  if (w < nc) L::words(A, ti.cell_begin + w, lane, en);
   cp_async_wait_all();
   pdl_wait();
   __syncthreads();
@@ -240,11 +295,9 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
   for (int j = w; j < nc; j += WPB) {
 #pragma unroll
     for (int i = 0; i < L::EPL; ++i) ent[lane + 32 * i] = en[i];
-    if (j + WPB < nc)
-#pragma unroll
-      for (int i = 0; i < L::EPL; ++i) en[i] = ep[(j + WPB) * L::ES + lane + 32 * i];
+    if (j + WPB < nc) L::words(A, ti.cell_begin + j + WPB, lane, en);
     __syncwarp();
-    if (ent[L::ES - 1] > 0) {
+    if (KF || ent[L::ES - 1] > 0) {
       // the owned fine values, UB points in flight per lane
       constexpr int UB = sizeof(T) == 4 ? 12 : 8;
 #pragma unroll
@@ -273,7 +326,7 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
         T v[M];
 #pragma unroll
         for (int i = 0; i < M; ++i) v[i] = lat[q + M2 * i];
-        line_restrict<K>(v);
+        L::down(v);
 #pragma unroll
         for (int i = 0; i < N; ++i) lat[q + M2 * i] = v[i];
       }
@@ -284,7 +337,7 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
         T v[M];
 #pragma unroll
         for (int i = 0; i < M; ++i) v[i] = p[M * i];
-        line_restrict<K>(v);
+        L::down(v);
 #pragma unroll
         for (int i = 0; i < N; ++i) p[M * i] = v[i];
       }
@@ -294,7 +347,7 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
         T v[M];
 #pragma unroll
         for (int i = 0; i < M; ++i) v[i] = p[i];
-        line_restrict<K>(v);
+        L::down(v);
 #pragma unroll
         for (int i = 0; i < N; ++i) cb[(N * lane + i) * CBS + j] = v[i];
       }
@@ -380,9 +433,9 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
 
 // one direction of C (TRANS: C^T) on the coarse values of a warp's lattice
 // (node (a, b, c) at a + M b + M^2 c)
-template <int K, int D, bool TRANS, typename T>
+template <int K, int KF, int D, bool TRANS, typename T>
 __device__ __forceinline__ void lattice_hang(T* lat, uint16_t m, int lane) {
-  using L = Lat<K>;
+  using L = Lat<K, KF>;
   if (lane >= L::N2) return;
   const int u = lane % L::N, v = lane / L::N;
   if (!line_hangs<K, D>(m, u, v)) return;
@@ -396,15 +449,15 @@ __device__ __forceinline__ void lattice_hang(T* lat, uint16_t m, int lane) {
   for (int a = 0; a < L::N; ++a) p[a * S] = x[a];
 }
 
-template <int K, typename T>
+template <int K, typename T, int KF>
 constexpr size_t prolong_smem() {
-  return ((size_t)(Lat<K>::NI + Lat<K>::NJ) * 32 + (size_t)WPB * (Lat<K>::ES + 32)) * 4 +
-         (size_t)WPB * Lat<K>::LS * sizeof(T);
+  using L = Lat<K, KF>;
+  return ((size_t)(L::NI + L::NJ) * 32 + (size_t)WPB * (L::ES + 32)) * 4 + (size_t)WPB * L::LS * sizeof(T);
 }
 
-template <int K, typename T>
+template <int K, typename T, int KF>
 __global__ void __launch_bounds__(WPB * 32) prolong_lattice(LatArgs<T> A) {
-  using L = Lat<K>;
+  using L = Lat<K, KF>;
   constexpr int N = L::N, N3 = L::N3, M = L::M, M2 = L::M2;
   constexpr int NT = WPB * 32;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -415,12 +468,14 @@ __global__ void __launch_bounds__(WPB * 32) prolong_lattice(LatArgs<T> A) {
   int32_t* ent = reinterpret_cast<int32_t*>(s_nd + L::NJ * 32) + w * (L::ES + 32);
   int32_t* gsc = ent + L::ES;
   const int c = blockIdx.x * WPB + w;
-  for (int i = threadIdx.x; i < L::NI * 32; i += NT) cp_async(s_pt + i, &g_lat.pt[K][i]);
-  for (int i = threadIdx.x; i < L::NJ * 32; i += NT) cp_async(s_nd + i, &g_lat.nd[K][i]);
+  for (int i = threadIdx.x; i < L::NI * 32; i += NT) cp_async(s_pt + i, L::points() + i);
+  for (int i = threadIdx.x; i < L::NJ * 32; i += NT) cp_async(s_nd + i, L::nodes() + i);
   uint16_t m = 0;
   if (c < A.n_coarse) {
+    int32_t en[L::EPL];
+    L::words(A, c, lane, en);
 #pragma unroll
-    for (int i = 0; i < L::EPL; ++i) cp_async(ent + lane + 32 * i, A.ent + (size_t)c * L::ES + lane + 32 * i);
+    for (int i = 0; i < L::EPL; ++i) ent[lane + 32 * i] = en[i];
     if (lane < NSLOT) cp_async(gsc + lane, A.gstart_c + (size_t)c * NSLOT + lane);
     m = A.mask_c[c];
   }
@@ -448,20 +503,20 @@ __global__ void __launch_bounds__(WPB * 32) prolong_lattice(LatArgs<T> A) {
   }
   __syncwarp();
   if (m & MASK_HANG) {  // C^(c) (uniform over the warp)
-    lattice_hang<K, 0, false>(lat, m, lane);
+    lattice_hang<K, KF, 0, false>(lat, m, lane);
     __syncwarp();
-    lattice_hang<K, 1, false>(lat, m, lane);
+    lattice_hang<K, KF, 1, false>(lat, m, lane);
     __syncwarp();
-    lattice_hang<K, 2, false>(lat, m, lane);
+    lattice_hang<K, KF, 2, false>(lat, m, lane);
     __syncwarp();
   }
-  if (ent[L::ES - 1] > 0) {
+  if (KF || ent[L::ES - 1] > 0) {
     if (lane < N * N) {  // x-lines (b, c)
       T* p = lat + M * (lane % N) + M2 * (lane / N);
       T v[M];
 #pragma unroll
       for (int i = 0; i < N; ++i) v[i] = p[i];
-      line_prolong<K>(v);
+      L::up(v);
 #pragma unroll
       for (int i = 0; i < M; ++i) p[i] = v[i];
     }
@@ -472,7 +527,7 @@ __global__ void __launch_bounds__(WPB * 32) prolong_lattice(LatArgs<T> A) {
       T v[M];
 #pragma unroll
       for (int i = 0; i < N; ++i) v[i] = p[M * i];
-      line_prolong<K>(v);
+      L::up(v);
 #pragma unroll
       for (int i = 0; i < M; ++i) p[M * i] = v[i];
     }
@@ -482,7 +537,7 @@ __global__ void __launch_bounds__(WPB * 32) prolong_lattice(LatArgs<T> A) {
       T v[M];
 #pragma unroll
       for (int i = 0; i < N; ++i) v[i] = lat[q + M2 * i];
-      line_prolong<K>(v);
+      L::up(v);
 #pragma unroll
       for (int i = 0; i < M; ++i) lat[q + M2 * i] = v[i];
     }
@@ -507,9 +562,9 @@ __global__ void __launch_bounds__(WPB * 32) prolong_lattice(LatArgs<T> A) {
 
 // restriction onto a level of few cells: the coarse cell's result to its cell
 // vector (kernels_small.cu adds them up)
-template <int K, typename T>
+template <int K, typename T, int KF>
 __global__ void __launch_bounds__(WPB * 32) restrict_cells(LatArgs<T> A) {
-  using L = Lat<K>;
+  using L = Lat<K, KF>;
   constexpr int N = L::N, N3 = L::N3, M = L::M, M2 = L::M2;
   constexpr int NT = WPB * 32;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -519,12 +574,14 @@ __global__ void __launch_bounds__(WPB * 32) restrict_cells(LatArgs<T> A) {
   uint32_t* s_nd = s_pt + L::NI * 32;
   int32_t* ent = reinterpret_cast<int32_t*>(s_nd + L::NJ * 32) + w * (L::ES + 32);
   const int c = blockIdx.x * WPB + w;
-  for (int i = threadIdx.x; i < L::NI * 32; i += NT) cp_async(s_pt + i, &g_lat.pt[K][i]);
-  for (int i = threadIdx.x; i < L::NJ * 32; i += NT) cp_async(s_nd + i, &g_lat.nd[K][i]);
+  for (int i = threadIdx.x; i < L::NI * 32; i += NT) cp_async(s_pt + i, L::points() + i);
+  for (int i = threadIdx.x; i < L::NJ * 32; i += NT) cp_async(s_nd + i, L::nodes() + i);
   uint16_t m = 0;
   if (c < A.n_coarse) {
+    int32_t en[L::EPL];
+    L::words(A, c, lane, en);
 #pragma unroll
-    for (int i = 0; i < L::EPL; ++i) cp_async(ent + lane + 32 * i, A.ent + (size_t)c * L::ES + lane + 32 * i);
+    for (int i = 0; i < L::EPL; ++i) ent[lane + 32 * i] = en[i];
     m = A.mask_c[c];
   }
   cp_async_wait_all();
@@ -533,7 +590,7 @@ __global__ void __launch_bounds__(WPB * 32) restrict_cells(LatArgs<T> A) {
   if (c >= A.n_coarse) return;
   const T* __restrict__ src = A.src;
   const T* __restrict__ rhs = A.rhs;
-  if (ent[L::ES - 1] > 0) {
+  if (KF || ent[L::ES - 1] > 0) {
     T v[L::NI];
 #pragma unroll
     for (int i = 0; i < L::NI; ++i) {
@@ -553,7 +610,7 @@ __global__ void __launch_bounds__(WPB * 32) restrict_cells(LatArgs<T> A) {
       T x[M];
 #pragma unroll
       for (int i = 0; i < M; ++i) x[i] = lat[q + M2 * i];
-      line_restrict<K>(x);
+      L::down(x);
 #pragma unroll
       for (int i = 0; i < N; ++i) lat[q + M2 * i] = x[i];
     }
@@ -564,7 +621,7 @@ __global__ void __launch_bounds__(WPB * 32) restrict_cells(LatArgs<T> A) {
       T x[M];
 #pragma unroll
       for (int i = 0; i < M; ++i) x[i] = p[M * i];
-      line_restrict<K>(x);
+      L::down(x);
 #pragma unroll
       for (int i = 0; i < N; ++i) p[M * i] = x[i];
     }
@@ -574,7 +631,7 @@ __global__ void __launch_bounds__(WPB * 32) restrict_cells(LatArgs<T> A) {
       T x[M];
 #pragma unroll
       for (int i = 0; i < M; ++i) x[i] = p[i];
-      line_restrict<K>(x);
+      L::down(x);
 #pragma unroll
       for (int i = 0; i < N; ++i) p[i] = x[i];
     }
@@ -593,11 +650,11 @@ __global__ void __launch_bounds__(WPB * 32) restrict_cells(LatArgs<T> A) {
   }
   __syncwarp();
   if (m & MASK_HANG) {  // C^(c)T
-    lattice_hang<K, 2, true>(lat, m, lane);
+    lattice_hang<K, KF, 2, true>(lat, m, lane);
     __syncwarp();
-    lattice_hang<K, 1, true>(lat, m, lane);
+    lattice_hang<K, KF, 1, true>(lat, m, lane);
     __syncwarp();
-    lattice_hang<K, 0, true>(lat, m, lane);
+    lattice_hang<K, KF, 0, true>(lat, m, lane);
     __syncwarp();
   }
 #pragma unroll
@@ -680,6 +737,34 @@ void fill_lattice(LatTables& t) {
           t.nd[k][i++] = (uint32_t)slot | ((uint32_t)off << 7) | ((uint32_t)(a + m * (b + m * c)) << 12);
         }
     for (; i < ND_MAX; ++i) t.nd[k][i] = pad;
+    if (k < 2) continue;
+    // p: slots by dimension (interior, faces, edges, vertices); a word beyond the slots is -1
+    i = 0;
+    for (int d = 3; d >= 0; --d)
+      for (int s = 0; s < NSLOT; ++s) {
+        const int x[3] = {s % 3, (s / 3) % 3, s / 9};
+        if ((x[0] == 1) + (x[1] == 1) + (x[2] == 1) != d) continue;
+        int lo[3], hi[3], off = 0;
+        for (int e = 0; e < 3; ++e) {
+          lo[e] = x[e] == 0 ? 0 : (x[e] == 1 ? 1 : k);
+          hi[e] = x[e] == 1 ? k : lo[e] + 1;
+        }
+        for (int c = lo[2]; c < hi[2]; ++c)
+          for (int b = lo[1]; b < hi[1]; ++b)
+            for (int a = lo[0]; a < hi[0]; ++a)
+              t.pf[k][i++] = (uint32_t)s | ((uint32_t)off++ << 7) | ((uint32_t)(a + n * (b + n * c)) << 12);
+      }
+    for (; i < ND_MAX; ++i) t.pf[k][i] = (uint32_t)NSLOT | ((uint32_t)(n * n * n) << 12);
+    i = 0;
+    const int kc = k / 2;
+    for (int c = 0; c <= kc; ++c)
+      for (int b = 0; b <= kc; ++b)
+        for (int a = 0; a <= kc; ++a) {
+          int slot, off;
+          host_node_slot(kc, a, b, c, slot, off);
+          t.pc[k][i++] = (uint32_t)slot | ((uint32_t)off << 7) | ((uint32_t)(a + n * (b + n * c)) << 12);
+        }
+    for (; i < 32; ++i) t.pc[k][i] = (uint32_t)NSLOT | ((uint32_t)(n * n * n) << 12);
   }
 }
 
@@ -705,6 +790,8 @@ template <typename T>
 LatArgs<T> lat_args(const TransferLaunch& L, const T* src, T* dst) {
   LatArgs<T> A{};
   A.ent = L.lattice;
+  A.gstart_f = L.gstart_f;
+  A.own_f = L.own_f;
   A.gstart_c = L.gstart_c;
   A.mask_c = L.mask_c;
   A.n_coarse = L.n_coarse;
@@ -719,64 +806,66 @@ LatArgs<T> lat_args(const TransferLaunch& L, const T* src, T* dst) {
   return A;
 }
 
-template <int K, typename T>
+template <int K, typename T, int KF = 0>
 void run_prolong(const TransferLaunch& L, const T* src, T* dst, cudaStream_t s) {
   const LatArgs<T> A = lat_args(L, src, dst);
-  smem_allow(prolong_lattice<K, T>, prolong_smem<K, T>());
-  launch_pdl(prolong_lattice<K, T>, (L.n_coarse + WPB - 1) / WPB, WPB * 32, prolong_smem<K, T>(), s, A);
+  constexpr size_t sm = prolong_smem<K, T, KF>();
+  smem_allow(prolong_lattice<K, T, KF>, sm);
+  launch_pdl(prolong_lattice<K, T, KF>, (L.n_coarse + WPB - 1) / WPB, WPB * 32, sm, s, A);
   note_launches(1);
 }
 
-template <int K, typename T>
+template <int K, typename T, int KF = 0>
 void run_restrict(const TransferLaunch& L, const T* src, T* dst, const T* rhs, bool ow, cudaStream_t s) {
   LatArgs<T> A = lat_args(L, src, dst);
   A.rhs = rhs;
   A.overwrite = ow;
-  const size_t sm = RestrictSmem<K, T>::total(L.coarse.max_local);
-  smem_allow(restrict_lattice<K, T>, sm);
-  launch_pdl(restrict_lattice<K, T>, L.coarse.n_tiles, WPB * 32, sm, s, A);
+  const size_t sm = RestrictSmem<K, T, KF>::total(L.coarse.max_local);
+  smem_allow(restrict_lattice<K, T, KF>, sm);
+  launch_pdl(restrict_lattice<K, T, KF>, L.coarse.n_tiles, WPB * 32, sm, s, A);
   note_launches(1);
   launch_halo_add(L.coarse, sizeof(T) == 8, dst, s);
 }
 
-template <int K, typename T>
+template <int K, typename T, int KF = 0>
 void run_restrict_cells(const TransferLaunch& L, const T* src, const T* rhs, cudaStream_t s) {
   LatArgs<T> A = lat_args(L, src, static_cast<T*>(L.coarse.cell_vec));
   A.rhs = rhs;
-  smem_allow(restrict_cells<K, T>, prolong_smem<K, T>());
-  launch_pdl(restrict_cells<K, T>, (L.n_coarse + WPB - 1) / WPB, WPB * 32, prolong_smem<K, T>(), s, A);
+  constexpr size_t sm = prolong_smem<K, T, KF>();
+  smem_allow(restrict_cells<K, T, KF>, sm);
+  launch_pdl(restrict_cells<K, T, KF>, (L.n_coarse + WPB - 1) / WPB, WPB * 32, sm, s, A);
   note_launches(1);
 }
 
-template <typename T>
-void restrict_cells_any(const TransferLaunch& L, const T* src, const T* rhs, cudaStream_t s) {
-  switch (L.kf) {
-    case 1: run_restrict_cells<1>(L, src, rhs, s); break;
-    case 2: run_restrict_cells<2>(L, src, rhs, s); break;
-    case 3: run_restrict_cells<3>(L, src, rhs, s); break;
-    case 4: run_restrict_cells<4>(L, src, rhs, s); break;
-  }
-}
+// run F<coarse degree, T, fine degree of a p transfer> for the transfer L
+#define GCMG_BY_DEGREE(F, T, ...)                                 \
+  if (L.kind == 0) switch (L.kf) {                                \
+      case 1: F<1, T>(__VA_ARGS__); break;                        \
+      case 2: F<2, T>(__VA_ARGS__); break;                        \
+      case 3: F<3, T>(__VA_ARGS__); break;                        \
+      case 4: F<4, T>(__VA_ARGS__); break;                        \
+    }                                                             \
+  else switch (L.kf) {                                            \
+      case 2: F<1, T, 2>(__VA_ARGS__); break;                     \
+      case 3: F<1, T, 3>(__VA_ARGS__); break;                     \
+      case 4: F<2, T, 4>(__VA_ARGS__); break;                     \
+    }
 
 template <typename T>
 void prolong_any(const TransferLaunch& L, const T* src, T* dst, cudaStream_t s) {
-  switch (L.kf) {
-    case 1: run_prolong<1>(L, src, dst, s); break;
-    case 2: run_prolong<2>(L, src, dst, s); break;
-    case 3: run_prolong<3>(L, src, dst, s); break;
-    case 4: run_prolong<4>(L, src, dst, s); break;
-  }
+  GCMG_BY_DEGREE(run_prolong, T, L, src, dst, s)
 }
 
 template <typename T>
 void restrict_any(const TransferLaunch& L, const T* src, T* dst, const T* rhs, bool ow, cudaStream_t s) {
-  switch (L.kf) {
-    case 1: run_restrict<1>(L, src, dst, rhs, ow, s); break;
-    case 2: run_restrict<2>(L, src, dst, rhs, ow, s); break;
-    case 3: run_restrict<3>(L, src, dst, rhs, ow, s); break;
-    case 4: run_restrict<4>(L, src, dst, rhs, ow, s); break;
-  }
+  GCMG_BY_DEGREE(run_restrict, T, L, src, dst, rhs, ow, s)
 }
+
+template <typename T>
+void restrict_cells_any(const TransferLaunch& L, const T* src, const T* rhs, cudaStream_t s) {
+  GCMG_BY_DEGREE(run_restrict_cells, T, L, src, rhs, s)
+}
+#undef GCMG_BY_DEGREE
 
 }  // namespace
 
@@ -808,9 +897,9 @@ void launch_lattice_entities(const TransferLaunch& L, int32_t* ent, cudaStream_t
 // The restriction accumulates through the coarse level's lane records, which
 // exist for tiles of at most 32 cells, and reads its record per tile: larger
 // tiles keep restrict_h.
-bool lattice_prolong_ok(const TransferLaunch& L) { return L.kind == 0 && L.lattice; }
+bool lattice_prolong_ok(const TransferLaunch& L) { return L.kind == 1 || L.lattice; }
 bool lattice_restrict_ok(const TransferLaunch& L) {
-  return L.kind == 0 && L.lattice && L.coarse.lane_tiles && L.coarse.tc <= 32;
+  return lattice_prolong_ok(L) && L.coarse.lane_tiles && L.coarse.tc <= 32;
 }
 
 void launch_prolong_lattice(const TransferLaunch& L, bool fp64, const void* coarse, void* fine, cudaStream_t s) {
