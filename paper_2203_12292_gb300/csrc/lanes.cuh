@@ -81,9 +81,10 @@ __device__ __forceinline__ df df_sel(bool p, df a, df b) { return df{p ? a.hi : 
 // their exact rounding errors (fused multiply-add), the p_j are summed by
 // error-free two-sums, and the low-order terms (product errors, cross terms
 // x.hi cl and x.lo ch, two-sum errors) go into one fp32 sum; 12 T - 5
-// operations instead of 18 T - 11 for a chain of df_fma
+// operations instead of 18 T - 11 for a chain of df_fma.  df_dot_raw leaves the
+// normalisation out (3 of them; see df_add_raw)
 template <int T>
-__device__ __forceinline__ df df_dot(const df* x, const float* ch, const float* cl) {
+__device__ __forceinline__ df df_dot_raw(const df* x, const float* ch, const float* cl) {
   float S = __fmul_rn(x[0].hi, ch[0]);
   float L = __fmaf_rn(x[0].hi, cl[0], __fmaf_rn(x[0].lo, ch[0], __fmaf_rn(x[0].hi, ch[0], -S)));
 #pragma unroll
@@ -96,7 +97,12 @@ __device__ __forceinline__ df df_dot(const df* x, const float* ch, const float* 
     S = s;
     L = __fadd_rn(L, __fadd_rn(l, t));
   }
-  return df_norm(S, L);
+  return df{S, L};
+}
+template <int T>
+__device__ __forceinline__ df df_dot(const df* x, const float* ch, const float* cl) {
+  const df s = df_dot_raw<T>(x, ch, cl);
+  return df_norm(s.hi, s.lo);
 }
 
 // even-odd forward transform with B (nodal -> modes in mode order) and its
@@ -109,8 +115,8 @@ __device__ __forceinline__ void df_eo_fwd_fast(df* u) {
   df e[NE], o[NH > 0 ? NH : 1];
 #pragma unroll
   for (int j = 0; j < NH; ++j) {
-    e[j] = df_add(u[j], u[N - 1 - j]);
-    o[j] = df_sub(u[j], u[N - 1 - j]);
+    e[j] = df_add_raw(u[j], u[N - 1 - j]);
+    o[j] = df_sub_raw(u[j], u[N - 1 - j]);
   }
   if (N % 2) e[NH] = u[NH];
 #pragma unroll
@@ -131,7 +137,7 @@ __device__ __forceinline__ void df_eo_bwd_fast(df* u) {
       ch[r] = c_tf[K].Be[r][j];
       cl[r] = c_tflo[K].Be[r][j];
     }
-    E[j] = df_dot<NE>(u, ch, cl);
+    E[j] = df_dot_raw<NE>(u, ch, cl);
   }
 #pragma unroll
   for (int j = 0; j < NH; ++j) {
@@ -140,14 +146,14 @@ __device__ __forceinline__ void df_eo_bwd_fast(df* u) {
       ch[r] = c_tf[K].Be[NE + r][j];
       cl[r] = c_tflo[K].Be[NE + r][j];
     }
-    O[j] = df_dot<NH>(u + NE, ch, cl);
+    O[j] = df_dot_raw<NH>(u + NE, ch, cl);
   }
 #pragma unroll
   for (int j = 0; j < NH; ++j) {
     u[j] = df_add(E[j], O[j]);
     u[N - 1 - j] = df_sub(E[j], O[j]);
   }
-  if (N % 2) u[NH] = E[NH];
+  if (N % 2) u[NH] = df_norm(E[NH].hi, E[NH].lo);
 }
 
 // I_p (TRANS: transposed) on one df line, by the mirror identity of interp_line_reg

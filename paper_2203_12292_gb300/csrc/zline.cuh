@@ -60,19 +60,19 @@ __device__ __forceinline__ void zline(df* v, const float* ch, const float* cl) {
   df e[NE], o[NH];
 #pragma unroll
   for (int j = 0; j < NH; ++j) {
-    e[j] = df_add(v[j], v[K - j]);
-    o[j] = df_sub(v[j], v[K - j]);
+    e[j] = df_add_raw(v[j], v[K - j]);
+    o[j] = df_sub_raw(v[j], v[K - j]);
   }
   if (N % 2) e[NH] = v[NH];
 #pragma unroll
   for (int i = 0; i < NE; ++i) {
-    const df E = df_dot<NE>(e, ch + NE * i, cl + NE * i);
+    const df E = df_dot_raw<NE>(e, ch + NE * i, cl + NE * i);
     if (i < NH) {
-      const df O = df_dot<NH>(o, ch + NE * NE + NH * i, cl + NE * NE + NH * i);
+      const df O = df_dot_raw<NH>(o, ch + NE * NE + NH * i, cl + NE * NE + NH * i);
       v[i] = df_add(E, O);
       v[K - i] = df_sub(E, O);
     } else {
-      v[i] = E;
+      v[i] = df_norm(E.hi, E.lo);
     }
   }
 }
