@@ -409,16 +409,36 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 8 : 1) vmult_lanes(Lane
 // The passes over the 1D lines as one loop, so that each transform is one piece
 // of code: written out pass by pass, the kernel's instructions did not fit the
 // instruction caches (the largest stall was "no instruction", 57 % issue
-// active).  A pass takes the lines along direction D through, in this order,
-// C_e, the forward transform, the innermost direction's matrix (zline), the
-// backward transform, C_e^T.
-enum : uint8_t { DF_C = 4, DF_FWD = 8, DF_Z = 16, DF_BWD = 32, DF_CT = 64 };  // bits 0-1: D
-__constant__ uint8_t c_df_pass[2][9] = {
+// active).  A pass is one operation on the lines along direction D; its loop over
+// the warp's lines holds that operation alone, with the lines' first nodes from a
+// table: tests of the operation and divisions in every line's iteration cost 7 to 14
+// % (Q4 octant 479 -> 448 us, Q2 octant 98 -> 85 us).  Leaving out the barriers that a
+// plane per warp makes unnecessary was no faster (451 us), nor was one quarter of
+// the tiles in native fp64 (615 us) or five blocks per SM (451 us).
+enum : uint8_t { DF_C = 0, DF_FWD = 4, DF_Z = 8, DF_BWD = 12, DF_CT = 16 };  // bits 0-1: D
+__constant__ uint8_t c_df_pass[2][11] = {
     // tiles without hanging cells: x, y forward, z, y, x backward
-    {0 | DF_FWD, 1 | DF_FWD, 2 | DF_Z, 1 | DF_BWD, 0 | DF_BWD, 0, 0, 0, 0},
+    {0 | DF_FWD, 1 | DF_FWD, 2 | DF_Z, 1 | DF_BWD, 0 | DF_BWD, 0, 0, 0, 0, 0, 0},
     // with hanging cells: C_x, C_y, C_z and the sweeps in the order z, y, x, and back
-    {0 | DF_C, 1 | DF_C, 2 | DF_C | DF_FWD, 1 | DF_FWD, 0 | DF_Z, 1 | DF_BWD, 2 | DF_BWD | DF_CT,
-     1 | DF_CT, 0 | DF_CT}};
+    {0 | DF_C, 1 | DF_C, 2 | DF_C, 2 | DF_FWD, 1 | DF_FWD, 0 | DF_Z, 1 | DF_BWD, 2 | DF_BWD, 2 | DF_CT, 1 | DF_CT,
+     0 | DF_CT}};
+// first node of the warp's i-th line along D, times 32: [k][D][w][i]
+__constant__ uint16_t c_df_node[KMAX + 1][3][NMAX][8];
+
+// op(v, i) on the warp's lines, first node ptr + node[i], node stride S * 32
+template <int N, typename F>
+__device__ __forceinline__ void df_lines(df* cb, const uint16_t* node, int S, F&& op) {
+#pragma unroll 1
+  for (int i = 0; i < N; ++i) {
+    df* ptr = cb + node[i];
+    df v[N];
+#pragma unroll
+    for (int a = 0; a < N; ++a) v[a] = ptr[a * S];
+    op(v, i);
+#pragma unroll
+    for (int a = 0; a < N; ++a) ptr[a * S] = v[a];
+  }
+}
 
 template <int K>
 __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(LaneArgsT<double> A) {
@@ -506,27 +526,20 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(L
       for (int a = 0; a < N; ++a) cb[(N * c_ll.bl[K][w][i] + a) * 32 + lane] = v[i][a];
   }
   // the first pass takes the warp's own lines
-  const int npass = hang ? 9 : 5;
+  const int npass = hang ? 11 : 5;
 #pragma unroll 1
   for (int ps = 0; ps < npass; ++ps) {
     const int f = c_df_pass[hang][ps], D = f & 3;
-    const int S = D == 0 ? 1 : (D == 1 ? N : N2);
-    const uint32_t hl = (f & (DF_C | DF_CT)) ? hg->hl[D][lane] : 0u;
-    const int p = (m >> D) & 1;
-#pragma unroll 1
-    for (int i = 0; i < N; ++i) {
-      const int r = c_ll.bl[K][w][i];
-      const bool on = (hl >> r) & 1u;
-      // a pass of C_e or C_e^T alone touches the hanging lines only
-      if (!(f & (DF_FWD | DF_Z | DF_BWD)) && !on) continue;
-      const int q = D == 0 ? N * r : (D == 1 ? r % N + N2 * (r / N) : r);
-      df* ptr = cb + q * 32 + lane;
-      df v[N];
-#pragma unroll
-      for (int a = 0; a < N; ++a) v[a] = ptr[a * S * 32];
-      if ((f & DF_C) && on) interp_line_df<K, false>(v, p);
-      if (f & DF_FWD) df_eo_fwd_fast<K>(v);
-      if (f & DF_Z) {  // h (K + (lam + lam') M) on the line of modes r
+    const int S = 32 * (D == 0 ? 1 : (D == 1 ? N : N2));
+    const uint16_t* node = c_df_node[K][D][w];
+    df* cl = cb + lane;
+    if ((f & ~3) == DF_FWD) {
+      df_lines<N>(cl, node, S, [&](df* v, int) { df_eo_fwd_fast<K>(v); });
+    } else if ((f & ~3) == DF_BWD) {
+      df_lines<N>(cl, node, S, [&](df* v, int) { df_eo_bwd_fast<K>(v); });
+    } else if ((f & ~3) == DF_Z) {  // h (K + (lam + lam') M) on the line of modes r
+      df_lines<N>(cl, node, S, [&](df* v, int i) {
+        const int r = c_ll.bl[K][w][i];
         zline<K>(v, c_zl.h[K - 1][r], c_zl.l[K - 1][r]);
         if (h_pow2) {  // 2 operations per value instead of 7, the same result
 #pragma unroll
@@ -535,11 +548,24 @@ __global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(L
 #pragma unroll
           for (int c = 0; c < N; ++c) v[c] = df_mul(v[c], h);
         }
-      }
-      if (f & DF_BWD) df_eo_bwd_fast<K>(v);
-      if ((f & DF_CT) && on) interp_line_df<K, true>(v, p);
+      });
+    } else {  // the hanging lines only
+      const uint32_t hl = hg->hl[D][lane];
+      const int p = (m >> D) & 1;
+#pragma unroll 1
+      for (int i = 0; i < N; ++i) {
+        if (!((hl >> c_ll.bl[K][w][i]) & 1u)) continue;
+        df* ptr = cl + node[i];
+        df v[N];
 #pragma unroll
-      for (int a = 0; a < N; ++a) ptr[a * S * 32] = v[a];
+        for (int a = 0; a < N; ++a) v[a] = ptr[a * S];
+        if ((f & ~3) == DF_C)
+          interp_line_df<K, false>(v, p);
+        else
+          interp_line_df<K, true>(v, p);
+#pragma unroll
+        for (int a = 0; a < N; ++a) ptr[a * S] = v[a];
+      }
     }
     __syncthreads();
   }
@@ -798,6 +824,15 @@ void upload_tables_lanes() {
   fill_lane_lines(t);
   cudaMemcpyToSymbol(c_ll, &t, sizeof(t));
   upload_zlines();
+  static uint16_t node[KMAX + 1][3][NMAX][8];
+  for (int k = 1; k <= KMAX; ++k)
+    for (int D = 0; D < 3; ++D)
+      for (int w = 0; w <= k; ++w)
+        for (int i = 0; i <= k; ++i) {
+          const int n = k + 1, r = t.bl[k][w][i];
+          node[k][D][w][i] = (uint16_t)(32 * (D == 0 ? n * r : (D == 1 ? r % n + n * n * (r / n) : r)));
+        }
+  cudaMemcpyToSymbol(c_df_node, node, sizeof(node));
 }
 
 bool lanes_ok(const CellLaunch& L) { return L.lane_tiles && L.tc <= 32 && !L.geom && L.k >= 1 && L.k <= KMAX; }
