@@ -154,8 +154,26 @@ __device__ __forceinline__ void sweep_y(float* cb, int w, int lane) {
   }
 }
 
-template <int K>
-__global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 8 : 1) vmult_lanes(LaneArgs A) {
+// Blocks per SM that the registers are limited for: dense (many regular tiles: more
+// warps hide the block start's chain of loads, at the price of a few spills) or
+// roomy (what the code of hanging cells and a level of one wave prefer).  fp32, dense
+// against roomy: Q4 octant 108 / 112 us, Q3 octant 71 / 76.5 us, Q2 octant 30.1 / 31.5
+// us; Q4 sphere (hanging cells in most tiles) 60 / 56.4 us, Q4 cube of 32,768 cells
+// (one wave) 15.2 / 14.4 us, Q3 octant of 34,903 cells 16.8 / 15.8 us.  fp64: Q4 octant
+// 447 / 451 us, Q3 octant 233 / 242 us, Q2 octant 82.5 / 84.6 us; Q4 sphere 227 / 220
+// us, Q2 sphere 53.3 / 52.6 us.
+constexpr int lanes_blocks(int K, bool dense) { return K == 4 ? (dense ? 8 : 7) : !dense ? 1 : K == 3 ? 10 : 14; }
+constexpr int lanes_df_blocks(int K, bool dense) { return K == 4 ? (dense ? 6 : 5) : !dense ? 1 : K == 3 ? 8 : 10; }
+// blocks per SM of the roomy variants as built
+constexpr int lanes_roomy(int K) { return K == 4 ? 7 : K == 3 ? 8 : 12; }
+constexpr int lanes_df_roomy(int K) { return K == 4 ? 5 : K == 3 ? 6 : 10; }
+// by the level, not by the launch: every range of a level's tiles takes the same code
+bool lanes_dense(const CellLaunch& L, int roomy_blocks) {
+  return 2 * L.n_hang_tiles <= L.n_tiles && L.n_tiles > roomy_blocks * L.n_sm;
+}
+
+template <int K, bool DENSE>
+__global__ void __launch_bounds__((K + 1) * 32, lanes_blocks(K, DENSE)) vmult_lanes(LaneArgs A) {
   pdl_begin();
   constexpr int N = K + 1, N2 = N * N, NT = N * 32;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -440,8 +458,8 @@ __device__ __forceinline__ void df_lines(df* cb, const uint16_t* node, int S, F&
   }
 }
 
-template <int K>
-__global__ void __launch_bounds__((K + 1) * 32, K == 4 ? 6 : 1) vmult_lanes_df(LaneArgsT<double> A) {
+template <int K, bool DENSE>
+__global__ void __launch_bounds__((K + 1) * 32, lanes_df_blocks(K, DENSE)) vmult_lanes_df(LaneArgsT<double> A) {
   constexpr int N = K + 1, N2 = N * N, NT = N * 32;
   extern __shared__ __align__(16) unsigned char smem[];
   LaneTile* st = reinterpret_cast<LaneTile*>(smem);
@@ -799,9 +817,10 @@ size_t lanes_df_smem(int max_local) {
 template <int K>
 cudaError_t run_lanes_df(const CellLaunch& L, const LaneArgsT<double>& A, int n_tiles, cudaStream_t s) {
   const size_t sm = lanes_df_smem<K>(L.max_local);
-  cudaError_t e = smem_allow(vmult_lanes_df<K>, sm);
+  const auto kernel = lanes_dense(L, lanes_df_roomy(K)) ? vmult_lanes_df<K, true> : vmult_lanes_df<K, false>;
+  cudaError_t e = smem_allow(kernel, sm);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(vmult_lanes_df<K>, n_tiles, (K + 1) * 32, sm, s, A);
+  e = launch_pdl(kernel, n_tiles, (K + 1) * 32, sm, s, A);
   note_launches(1);
   return e;
 }
@@ -809,9 +828,10 @@ cudaError_t run_lanes_df(const CellLaunch& L, const LaneArgsT<double>& A, int n_
 template <int K>
 cudaError_t run_lanes(const CellLaunch& L, const LaneArgs& A, int n_tiles, cudaStream_t s) {
   const size_t sm = lanes_smem<K>(L.max_local);
-  cudaError_t e = smem_allow(vmult_lanes<K>, sm);
+  const auto kernel = lanes_dense(L, lanes_roomy(K)) ? vmult_lanes<K, true> : vmult_lanes<K, false>;
+  cudaError_t e = smem_allow(kernel, sm);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(vmult_lanes<K>, n_tiles, (K + 1) * 32, sm, s, A);
+  e = launch_pdl(kernel, n_tiles, (K + 1) * 32, sm, s, A);
   note_launches(1);
   return e;
 }
