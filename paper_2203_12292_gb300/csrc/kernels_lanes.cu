@@ -304,7 +304,8 @@ __global__ void __launch_bounds__((K + 1) * 32, lanes_blocks(K, DENSE)) vmult_la
     // G_e^T.  Nodes of two cells are one DoF only where every coordinate is
     // equal or both lie on the cell boundary: between planes only c = 0 and
     // c = k meet, so warp k adds after warp 0 (named barrier 1); within a
-    // plane the x-lines and their nodes add in program order.
+    // plane the x-lines and their nodes add in program order (add_turns keeps the
+    // lanes together from one slot to the next).
     if (w == K) named_bar_sync(1, 64);
 #pragma unroll
     for (int b = 0; b < N; ++b) {
@@ -314,10 +315,9 @@ __global__ void __launch_bounds__((K + 1) * 32, lanes_blocks(K, DENSE)) vmult_la
       float* p0 = reinterpret_cast<float*>(const_cast<char*>(in ? xB0 : xA0) + q0) + (in ? b - 1 : 0);
       float* p1 = reinterpret_cast<float*>(const_cast<char*>(in ? xB1 : xA1) + q1) + (in ? (b - 1) * (K - 1) : 0);
       float* p2 = reinterpret_cast<float*>(const_cast<char*>(in ? xB0 : xA0) + q2) + (in ? b - 1 : 0);
-      *p0 += u[N * b];
-#pragma unroll
-      for (int a = 1; a < K; ++a) p1[a - 1] += u[N * b + a];
-      *p2 += u[N * b + K];
+      add_turns<1>(p0, u + N * b, 0, 1);
+      if constexpr (K > 1) add_turns<K - 1>(p1, u + N * b + 1, 0, 1);
+      add_turns<1>(p2, u + N * b + K, 0, 1);
     }
     if (w == 0) named_bar_arrive(1, 64);
   } else {
@@ -776,7 +776,6 @@ __global__ void __launch_bounds__(RWPB * 32) vmult_q1(LaneArgsT<T> A, int n_tile
   for (int n = 0; n < N3; ++n) {
     const int slot = vertex_slot(n);
     add_turns<1>(xs + (ls[n][lane] >> 2), &u[n], hang ? lh->rank[slot][lane] : 0, hang ? lh->most[slot] : 1);
-    __syncwarp();
   }
   T* d = A.dst + ti.dof_begin;
   for (int i = lane; i < ti.n_owned; i += 32) {

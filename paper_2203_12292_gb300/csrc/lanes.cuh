@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "device.cuh"
+#include "turns.cuh"
 
 namespace gcmg {
 
@@ -50,28 +51,6 @@ __device__ __forceinline__ void interp_line_reg(float* v, int p) {
   }
 #pragma unroll
   for (int a = 0; a < N; ++a) v[a] = p ? y[K - a] : y[a];
-}
-
-// x[i] += v[i] for the C nodes of one slot: lanes whose slot starts at the same
-// DoF take turns in lane order (rank and turns come with the tile: finding the
-// lanes that meet with a match over the warp's addresses at every node was the
-// largest part of a hanging tile: Q4 sphere postsmoothing 311 -> 261 us with the
-// turns and the hanging lines dealt evenly to the warps)
-template <int C, typename T>
-__device__ __forceinline__ void add_turns(T* x, const T* v, int rank, int turns) {
-  if (turns <= 1) {  // uniform over the warp
-#pragma unroll
-    for (int i = 0; i < C; ++i) x[i] += v[i];
-    return;
-  }
-#pragma unroll 1
-  for (int q = 0; q < turns; ++q) {
-    if (rank == q) {
-#pragma unroll
-      for (int i = 0; i < C; ++i) x[i] += v[i];
-    }
-    __syncwarp();
-  }
 }
 
 __device__ __forceinline__ df df_sel(bool p, df a, df b) { return df{p ? a.hi : b.hi, p ? a.lo : b.lo}; }
