@@ -284,7 +284,7 @@ __global__ void __launch_bounds__((K + 1) * 32, lanes_blocks(K, DENSE)) vmult_la
       float v[N];
 #pragma unroll
       for (int c = 0; c < N; ++c) v[c] = p[c * N2 * 32];
-      zline<K>(v, c_zl.h[K - 1][i + N * w]);
+      zline<K>(v, c_zl.f[zline_row(K) + i + N * w], i == 0);
 #pragma unroll
       for (int c = 0; c < N; ++c) p[c * N2 * 32] = h * v[c];
     }
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__((K + 1) * 32, lanes_blocks(K, DENSE)) vmult_la
       float x[N];
 #pragma unroll
       for (int a = 0; a < N; ++a) x[a] = p[a * 32];
-      zline<K>(x, c_zl.h[K - 1][i + N * w]);
+      zline<K>(x, c_zl.f[zline_row(K) + i + N * w], i == 0);
 #pragma unroll
       for (int a = 0; a < N; ++a) p[a * 32] = h * x[a];
     }
@@ -558,7 +558,7 @@ __global__ void __launch_bounds__((K + 1) * 32, lanes_df_blocks(K, DENSE)) vmult
     } else if ((f & ~3) == DF_Z) {  // h (K + (lam + lam') M) on the line of modes r
       df_lines<N>(cl, node, S, [&](df* v, int i) {
         const int r = c_ll.bl[K][w][i];
-        zline<K>(v, c_zl.h[K - 1][r], c_zl.l[K - 1][r]);
+        zline<K>(v, c_zl.h[zline_row(K) + r], c_zl.l[zline_row(K) + r]);
         if (h_pow2) {  // 2 operations per value instead of 7, the same result
 #pragma unroll
           for (int c = 0; c < N; ++c) v[c] = df{v[c].hi * h.hi, v[c].lo * h.hi};
@@ -644,11 +644,11 @@ constexpr int RWPB = 4;  // tiles (warps) per block
 
 template <int K>
 __device__ __forceinline__ void reg_z(float* v, int q) {
-  zline<K>(v, c_zl.h[K - 1][q]);
+  zline<K>(v, c_zl.f[zline_row(K) + q], q == 0);
 }
 template <int K>
 __device__ __forceinline__ void reg_z(df* v, int q) {
-  zline<K>(v, c_zl.h[K - 1][q], c_zl.l[K - 1][q]);
+  zline<K>(v, c_zl.h[zline_row(K) + q], c_zl.l[zline_row(K) + q]);
 }
 
 template <int K, int D, bool FWD, typename V>

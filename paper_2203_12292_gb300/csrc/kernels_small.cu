@@ -106,8 +106,9 @@ __global__ void __launch_bounds__(SWPB * 32) cell_vectors(CellVecArgs<T> A) {
   const int q = lane / N2, r = lane - q * N2;     // the lane's cell and line
   const bool on = q < nc;
   uint16_t m = 0;
-  constexpr int NC = (N / 2) * (N / 2) + ((N + 1) / 2) * ((N + 1) / 2);
-  float zh[NC], zl[sizeof(T) == 8 ? NC : 1];      // K + (lam_a + lam_b) M on the z-line (a, b) = r
+  // K + (lam_a + lam_b) M on the z-line (a, b) = r: high and low parts, or the fp32 form and its t
+  constexpr int NC = zline_count(K) + (sizeof(T) == 4);
+  float zh[NC], zl[sizeof(T) == 8 ? NC : 1];
   V h = V(0);
   if (on) {
     const CellMeta& cm = A.meta[c0 + q];
@@ -117,8 +118,8 @@ __global__ void __launch_bounds__(SWPB * 32) cell_vectors(CellVecArgs<T> A) {
     h = V(hd);
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
-      zh[i] = g_zl.h[K - 1][r][i];
-      if (sizeof(T) == 8) zl[i] = g_zl.l[K - 1][r][i];
+      zh[i] = sizeof(T) == 8 ? g_zl.h[zline_row(K) + r][i] : g_zl.f[zline_row(K) + r][i];
+      if (sizeof(T) == 8) zl[i] = g_zl.l[zline_row(K) + r][i];
     }
   }
   const bool hang = __any_sync(0xffffffffu, (m & MASK_HANG) != 0);
@@ -147,7 +148,7 @@ __global__ void __launch_bounds__(SWPB * 32) cell_vectors(CellVecArgs<T> A) {
     if constexpr (sizeof(T) == 8)
       zline<K>(x, zh, zl);
     else
-      zline<K>(x, zh);
+      zline<K>(x, zh, true);
 #pragma unroll
     for (int c = 0; c < N; ++c) x[c] = x[c] * h;
 #pragma unroll

@@ -6,8 +6,17 @@
 // matrices.  That is one (k+1) x (k+1) matrix per pair of modes, symmetric under
 // reversal: in even-odd form 13 coefficients at k = 4.  Applying it costs half of
 // what the forward transform, the scaling by h (lam_a + lam_b + lam_c) and the
-// backward transform cost (26 instead of 44 operations per line in fp32, about
-// 235 instead of 470 in double-float), in fewer roundings.
+// backward transform cost (28 instead of 44 operations per line in fp32, about
+// 235 instead of 470 in double-float).
+//   In fp32 the matrix of the constant pair (lam_a + lam_b = 0, the stiffness
+// matrix alone) is applied to differences: its rows sum to zero, and rows rounded
+// entry by entry do not (-4.8e-7 at k = 4), which acts as a reaction term of one
+// sign in every cell.  With e_j - t e_mid in place of e_j (t = 2, without a middle
+// node 1) the middle column is the row sum, zero, and constants along the line give
+// zero whatever the rounding.  The other pairs have t = 0: the same instructions,
+// the same bits as without.  x^T A x on sin sin sin, degree 4, 32^3 cells, relative
+// error: sweeps and scaling 1.7e-7, the matrix rounded entry by entry 1.5e-5
+// (growing with h^-2), differences 2.4e-7.
 // fp32 operator of the octant meshes: Q3 84 -> 73 us (269,998 cells), Q4 115 -> 111
 // us (296,535 cells); a level of few cells (Q4, 4,712 cells) 14.5 -> 9.3 us in fp32,
 // 34 -> 24.5 us in fp64.
@@ -18,17 +27,23 @@
 
 namespace gcmg {
 
-// coefficients of degree k at [k - 1], line of modes i + (k+1) j (mode order of
-// DevTables::lame): the even block, rows of (k+2)/2, then the odd block
+// first row of degree k's lines, one row per line of modes i + (k+1) j (mode order
+// of DevTables::lame); a row: the even block, rows of (k+2)/2, then the odd block
+__host__ __device__ constexpr int zline_row(int k) { return k * (k + 1) * (2 * k + 1) / 6 - 1; }
 struct ZLines {
-  alignas(16) float h[KMAX][NMAX * NMAX][16];
-  alignas(16) float l[KMAX][NMAX * NMAX][16];  // low parts: h + l to about 2^-48
+  alignas(16) float f[zline_row(KMAX + 1)][16];  // fp32; then t
+  alignas(16) float h[zline_row(KMAX + 1)][16];
+  alignas(16) float l[zline_row(KMAX + 1)][16];  // low parts: h + l to about 2^-48
 };
 static __constant__ ZLines c_zl;  // one copy per translation unit (upload_zlines)
 
-// v <- (K + lam M) v with the coefficients c
+__host__ __device__ constexpr int zline_count(int k) { return ((k + 2) / 2) * ((k + 2) / 2) + ((k + 1) / 2) * ((k + 1) / 2); }
+
+// v <- (K + lam M) v with the coefficients c; constants: the line may be that of the
+// modes (0, 0) (differences on every line of the Q4 octant operator: 109.3 us, on those
+// of the first mode only 108.4 us, as without)
 template <int K>
-__device__ __forceinline__ void zline(float* v, const float* c) {
+__device__ __forceinline__ void zline(float* v, const float* c, bool constants) {
   constexpr int N = K + 1, NH = N / 2, NE = (N + 1) / 2;
   float e[NE], o[NH];
 #pragma unroll
@@ -37,6 +52,10 @@ __device__ __forceinline__ void zline(float* v, const float* c) {
     o[j] = v[j] - v[K - j];
   }
   if (N % 2) e[NH] = v[NH];
+  if (constants) {
+#pragma unroll
+    for (int j = 0; j < NE - 1; ++j) e[j] = fmaf(-c[zline_count(K)], e[NE - 1], e[j]);
+  }
 #pragma unroll
   for (int i = 0; i < NE; ++i) {
     float E = c[NE * i] * e[0];
@@ -95,11 +114,17 @@ static inline void upload_zlines() {
   fill_tables(td, tf);
   for (int k = 1; k <= KMAX; ++k)
     for (int q = 0; q < (k + 1) * (k + 1); ++q) {
+      const int nc = zline_count(k), nh = (k + 1) / 2, ne = (k + 2) / 2;
       double c[13] = {};
       zline_coefficients(basis(k), td[k].lame[q % (k + 1)] + td[k].lame[q / (k + 1)], c);
       for (int i = 0; i < 13; ++i) {
-        z.h[k - 1][q][i] = (float)c[i];
-        z.l[k - 1][q][i] = (float)(c[i] - (double)z.h[k - 1][q][i]);
+        z.h[zline_row(k) + q][i] = (float)c[i];
+        z.l[zline_row(k) + q][i] = (float)(c[i] - (double)z.h[zline_row(k) + q][i]);
+        z.f[zline_row(k) + q][i] = z.h[zline_row(k) + q][i];
+      }
+      if (q == 0 && ne > 1) {  // modes (0, 0): constants; lam = 0
+        for (int i = 0; i < ne; ++i) z.f[zline_row(k) + q][ne * i + ne - 1] = 0.f;
+        z.f[zline_row(k) + q][nc] = ne > nh ? 2.f : 1.f;
       }
     }
   cudaMemcpyToSymbol(c_zl, &z, sizeof(z));
