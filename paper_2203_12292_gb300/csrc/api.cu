@@ -409,7 +409,7 @@ void vcycle_level(Handle& H, int l, bool pending) {
   const bool f64 = !L.fp32;
   if (pending && (l == 0 || dense_usable(H, l))) launch_cell_sum(L.cl, f64, L.b.p, false, H.stream);
   if (dense_usable(H, l)) {
-    launch_dense_apply(f64, H.dense.p, (int)L.n(), L.b.p, L.x.p, H.stream);
+    launch_dense_apply(f64, H.dense.as<double>(), (int)L.n(), L.b.p, L.x.p, H.stream);
     return;
   }
   if (l == 0) {
@@ -639,13 +639,9 @@ void setup_dense(Handle& H) {
     }
     const double* M = dense_vcycle_matrix(n, A, L.dinv64.as<double>(), (int)coef.size() / 2, coef.data(), n_c, P, Mc,
                                           work.as<double>(), H.stream);
-    if (l < top)
-      ck(cudaMemcpyAsync(Mc, M, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToDevice, H.stream), "copy");
-    else {
-      const size_t bytes = (size_t)n * n * (L.fp32 ? sizeof(float) : sizeof(double));
-      if (H.dense.bytes != bytes) H.dense.alloc(bytes);
-      launch_dense_store(!L.fp32, M, H.dense.p, (int64_t)n * n, H.stream);
-    }
+    const size_t bytes = (size_t)n * n * sizeof(double);
+    if (l == top && H.dense.bytes != bytes) H.dense.alloc(bytes);
+    ck(cudaMemcpyAsync(l < top ? Mc : H.dense.p, M, bytes, cudaMemcpyDeviceToDevice, H.stream), "copy");
     n_c = n;
   }
   ck_launches("dense levels");

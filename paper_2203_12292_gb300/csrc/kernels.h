@@ -187,8 +187,8 @@ void launch_dense_prolongation(const TransferLaunch& T, int n_f, int n_c, int ce
 size_t dense_scratch_bytes(int n);
 double* dense_vcycle_matrix(int n, const double* A, const double* dinv, int steps, const double* coef, int n_c,
                             const double* P, const double* Mc, double* work, cudaStream_t s);
-void launch_dense_store(bool fp64, const double* M, void* out, int64_t n, cudaStream_t s);
-void launch_dense_apply(bool fp64, const void* M, int n, const void* b, void* x, cudaStream_t s);
+// x = M b, sums in fp64; fp64: of b and x
+void launch_dense_apply(bool fp64, const double* M, int n, const void* b, void* x, cudaStream_t s);
 
 // vector kernels
 void upload_tables();

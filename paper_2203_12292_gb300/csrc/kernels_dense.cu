@@ -7,13 +7,15 @@
 // builds M_l once, in fp64 and in a fixed order, from the level operators,
 // their Jacobi diagonals, the Chebyshev coefficients and the prolongations:
 //   X = p_pre(A) b, X += P M_{l-1} P^T (1 - A X), postsmoothing,  b = identity
-// and a cycle applies it as one matrix-vector product in the level's
-// precision.
+// and a cycle applies it as one matrix-vector product.  The matrix and the sums
+// are fp64 for fp32 levels too, rounded once into x: the exact solve on level 0
+// in it was fp64 level by level, and an fp32 matrix with fp32 sums lost that.
 // Q2 octant mesh (6,407 DoFs; the levels up to 659 DoFs in the matrix), solve
 // with fp64 V-cycle: 3.36 -> 1.69 ms; batch of 16 problems 14.9 -> 11.2 ms.  The
-// matrix of 659 DoFs costs 0.9 ms of set-up.  DENSE_MAX: at 1,024 DoFs the
-// product reads 4 MB in fp32, about 2 us, against 50 to 110 us level by level;
-// beyond it the set-up's products (n^2 row lengths) grow faster than the gain.
+// matrix of 659 DoFs costs 0.9 ms of set-up.  DENSE_MAX: at 927 DoFs the
+// product takes 7.1 us for an fp32 level (3.5 with an fp32 matrix and sums) and 5.8
+// for an fp64 one, against 50 to 110 us level by level; beyond it the set-up's
+// products (n^2 row lengths) grow faster than the gain.
 #include <algorithm>
 
 #include "device.cuh"
@@ -251,34 +253,43 @@ __global__ void __launch_bounds__(BLOCK) dense_product(DenseProduct G) {
   }
 }
 
+// x = M b, one warp per row, a lane's partial sums and the lanes in a fixed order.
+// The first 256 entries of the rows are loaded before the predecessor's completion
+// (the matrix is set-up data); an fp32 b is widened once per block, since a
+// conversion costs as much as a product on the FP64 pipe.
+constexpr int DROWS = 4;  // rows (warps) per block
 template <typename T>
-__global__ void __launch_bounds__(BLOCK) dense_store(const double* M, T* out, int64_t n) {
-  pdl_begin();
-  const int64_t t = blockIdx.x * (int64_t)BLOCK + threadIdx.x;
-  if (t < n) out[t] = (T)M[t];
-}
-
-// x = M b, one warp per row, a lane's partial sums and the lanes in a fixed order
-template <typename T>
-__global__ void __launch_bounds__(128) dense_apply(const T* __restrict__ M, int n, const T* __restrict__ b,
-                                                   T* __restrict__ x) {
-  pdl_begin();
-  const int i = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (i >= n) return;
-  const T* row = M + (size_t)i * n;
-  T s[8] = {};
-  int k = lane;
-  for (; k + 7 * 32 < n; k += 8 * 32) {
+__global__ void __launch_bounds__(DROWS * 32) dense_apply(const double* __restrict__ M, int n,
+                                                          const T* __restrict__ b, T* __restrict__ x) {
+  constexpr bool WIDEN = sizeof(T) == 4;
+  __shared__ double sb[WIDEN ? DENSE_MAX : 1];
+  const int i = blockIdx.x * DROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const double* row = M + (size_t)min(i, n - 1) * n;
+  double m[8], s[8] = {};
 #pragma unroll
-    for (int u = 0; u < 8; ++u) s[u] += row[k + 32 * u] * b[k + 32 * u];
+  for (int u = 0; u < 8; ++u) m[u] = lane + 32 * u < n ? row[lane + 32 * u] : 0.0;
+  pdl_wait();
+  if constexpr (WIDEN) {
+    for (int k = threadIdx.x; k < n; k += DROWS * 32) sb[k] = (double)b[k];
+    __syncthreads();
   }
+  auto in = [&](int k) -> double {
+    if constexpr (WIDEN)
+      return sb[k];
+    else
+      return b[k];
+  };
+  for (int k = lane; k < n; k += 8 * 32) {
 #pragma unroll
-  for (int u = 0; u < 8; ++u)
-    if (k + 32 * u < n) s[u] += row[k + 32 * u] * b[k + 32 * u];
-  T v = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+    for (int u = 0; u < 8; ++u)
+      if (k + 32 * u < n) s[u] += m[u] * in(k + 32 * u);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) m[u] = k + 32 * (u + 8) < n ? row[k + 32 * (u + 8)] : 0.0;
+  }
+  double v = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
 #pragma unroll
   for (int h = 16; h > 0; h >>= 1) v += __shfl_down_sync(0xffffffffu, v, h);
-  if (lane == 0) x[i] = v;
+  if (lane == 0 && i < n) x[i] = (T)v;
 }
 
 void product(const DenseProduct& G, int rows, cudaStream_t s) {
@@ -384,22 +395,13 @@ double* dense_vcycle_matrix(int n, const double* A, const double* dinv, int step
   return X;
 }
 
-void launch_dense_store(bool fp64, const double* M, void* out, int64_t n, cudaStream_t s) {
-  const unsigned nb = (unsigned)((n + BLOCK - 1) / BLOCK);
+void launch_dense_apply(bool fp64, const double* M, int n, const void* b, void* x, cudaStream_t s) {
   if (fp64)
-    launch_pdl(dense_store<double>, nb, BLOCK, 0, s, M, static_cast<double*>(out), n);
+    launch_pdl(dense_apply<double>, (n + DROWS - 1) / DROWS, DROWS * 32, 0, s, M, n, static_cast<const double*>(b),
+               static_cast<double*>(x));
   else
-    launch_pdl(dense_store<float>, nb, BLOCK, 0, s, M, static_cast<float*>(out), n);
-  note_launches(1);
-}
-
-void launch_dense_apply(bool fp64, const void* M, int n, const void* b, void* x, cudaStream_t s) {
-  if (fp64)
-    launch_pdl(dense_apply<double>, (n + 3) / 4, 128, 0, s, static_cast<const double*>(M), n,
-               static_cast<const double*>(b), static_cast<double*>(x));
-  else
-    launch_pdl(dense_apply<float>, (n + 3) / 4, 128, 0, s, static_cast<const float*>(M), n,
-               static_cast<const float*>(b), static_cast<float*>(x));
+    launch_pdl(dense_apply<float>, (n + DROWS - 1) / DROWS, DROWS * 32, 0, s, M, n, static_cast<const float*>(b),
+               static_cast<float*>(x));
   note_launches(1);
 }
 
