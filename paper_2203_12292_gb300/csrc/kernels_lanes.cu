@@ -160,7 +160,8 @@ __device__ __forceinline__ void sweep_y(float* cb, int w, int lane) {
 // against roomy: Q4 octant 108 / 112 us, Q3 octant 71 / 76.5 us, Q2 octant 30.1 / 31.5
 // us; Q4 sphere (hanging cells in most tiles) 60 / 56.4 us, Q4 cube of 32,768 cells
 // (one wave) 15.2 / 14.4 us, Q3 octant of 34,903 cells 16.8 / 15.8 us.  fp64: Q4 octant
-// 447 / 451 us, Q3 octant 233 / 242 us, Q2 octant 82.5 / 84.6 us; Q4 sphere 227 / 220
+// 447 / 451 us, Q3 octant 233 / 242 us, Q2 octant 82.5 / 84.6 us (438, 233, 84.2 with the
+// differences of zline.cuh); Q4 sphere 227 / 220
 // us, Q2 sphere 53.3 / 52.6 us.
 constexpr int lanes_blocks(int K, bool dense) { return K == 4 ? (dense ? 8 : 7) : !dense ? 1 : K == 3 ? 10 : 14; }
 constexpr int lanes_df_blocks(int K, bool dense) { return K == 4 ? (dense ? 6 : 5) : !dense ? 1 : K == 3 ? 8 : 10; }
@@ -284,7 +285,7 @@ __global__ void __launch_bounds__((K + 1) * 32, lanes_blocks(K, DENSE)) vmult_la
       float v[N];
 #pragma unroll
       for (int c = 0; c < N; ++c) v[c] = p[c * N2 * 32];
-      zline<K>(v, c_zl.f[zline_row(K) + i + N * w], i == 0);
+      zline<K>(v, c_zl.h[zline_row(K) + i + N * w], i == 0);
 #pragma unroll
       for (int c = 0; c < N; ++c) p[c * N2 * 32] = h * v[c];
     }
@@ -356,7 +357,7 @@ __global__ void __launch_bounds__((K + 1) * 32, lanes_blocks(K, DENSE)) vmult_la
       float x[N];
 #pragma unroll
       for (int a = 0; a < N; ++a) x[a] = p[a * 32];
-      zline<K>(x, c_zl.f[zline_row(K) + i + N * w], i == 0);
+      zline<K>(x, c_zl.h[zline_row(K) + i + N * w], i == 0);
 #pragma unroll
       for (int a = 0; a < N; ++a) p[a * 32] = h * x[a];
     }
@@ -558,7 +559,7 @@ __global__ void __launch_bounds__((K + 1) * 32, lanes_df_blocks(K, DENSE)) vmult
     } else if ((f & ~3) == DF_Z) {  // h (K + (lam + lam') M) on the line of modes r
       df_lines<N>(cl, node, S, [&](df* v, int i) {
         const int r = c_ll.bl[K][w][i];
-        zline<K>(v, c_zl.h[zline_row(K) + r], c_zl.l[zline_row(K) + r]);
+        zline<K>(v, c_zl.h[zline_row(K) + r], c_zl.l[zline_row(K) + r], r == 0);
         if (h_pow2) {  // 2 operations per value instead of 7, the same result
 #pragma unroll
           for (int c = 0; c < N; ++c) v[c] = df{v[c].hi * h.hi, v[c].lo * h.hi};
@@ -644,11 +645,11 @@ constexpr int RWPB = 4;  // tiles (warps) per block
 
 template <int K>
 __device__ __forceinline__ void reg_z(float* v, int q) {
-  zline<K>(v, c_zl.f[zline_row(K) + q], q == 0);
+  zline<K>(v, c_zl.h[zline_row(K) + q], q == 0);
 }
 template <int K>
 __device__ __forceinline__ void reg_z(df* v, int q) {
-  zline<K>(v, c_zl.h[zline_row(K) + q], c_zl.l[zline_row(K) + q]);
+  zline<K>(v, c_zl.h[zline_row(K) + q], c_zl.l[zline_row(K) + q], q == 0);
 }
 
 template <int K, int D, bool FWD, typename V>

@@ -106,8 +106,8 @@ __global__ void __launch_bounds__(SWPB * 32) cell_vectors(CellVecArgs<T> A) {
   const int q = lane / N2, r = lane - q * N2;     // the lane's cell and line
   const bool on = q < nc;
   uint16_t m = 0;
-  // K + (lam_a + lam_b) M on the z-line (a, b) = r: high and low parts, or the fp32 form and its t
-  constexpr int NC = zline_count(K) + (sizeof(T) == 4);
+  constexpr int NC = zline_count(K) + 1;
+  // K + (lam_a + lam_b) M on the z-line (a, b) = r
   float zh[NC], zl[sizeof(T) == 8 ? NC : 1];
   V h = V(0);
   if (on) {
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(SWPB * 32) cell_vectors(CellVecArgs<T> A) {
     h = V(hd);
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
-      zh[i] = sizeof(T) == 8 ? g_zl.h[zline_row(K) + r][i] : g_zl.f[zline_row(K) + r][i];
+      zh[i] = g_zl.h[zline_row(K) + r][i];
       if (sizeof(T) == 8) zl[i] = g_zl.l[zline_row(K) + r][i];
     }
   }
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(SWPB * 32) cell_vectors(CellVecArgs<T> A) {
 #pragma unroll
     for (int c = 0; c < N; ++c) x[c] = cl[r + N2 * c];
     if constexpr (sizeof(T) == 8)
-      zline<K>(x, zh, zl);
+      zline<K>(x, zh, zl, r == 0);
     else
       zline<K>(x, zh, true);
 #pragma unroll

@@ -8,15 +8,15 @@
 // what the forward transform, the scaling by h (lam_a + lam_b + lam_c) and the
 // backward transform cost (28 instead of 44 operations per line in fp32, about
 // 235 instead of 470 in double-float).
-//   In fp32 the matrix of the constant pair (lam_a + lam_b = 0, the stiffness
-// matrix alone) is applied to differences: its rows sum to zero, and rows rounded
-// entry by entry do not (-4.8e-7 at k = 4), which acts as a reaction term of one
-// sign in every cell.  With e_j - t e_mid in place of e_j (t = 2, without a middle
-// node 1) the middle column is the row sum, zero, and constants along the line give
-// zero whatever the rounding.  The other pairs have t = 0: the same instructions,
-// the same bits as without.  x^T A x on sin sin sin, degree 4, 32^3 cells, relative
-// error: sweeps and scaling 1.7e-7, the matrix rounded entry by entry 1.5e-5
-// (growing with h^-2), differences 2.4e-7.
+//   The matrix of the constant pair (lam_a + lam_b = 0, the stiffness matrix alone)
+// is applied to differences: its rows sum to zero, and rows rounded entry by entry
+// do not (-4.8e-7 at k = 4 in fp32), which acts as a reaction term of one sign in
+// every cell.  With e_j - t e_mid in place of e_j (t = 2, without a middle node 1)
+// the middle column is the row sum, zero, and constants along the line give zero
+// whatever the rounding.  x^T A x on sin sin sin, 32^3 cells, relative error of the
+// sweeps and scaling, the matrix rounded entry by entry (growing with h^-2), the
+// differences: fp32, degree 4: 1.7e-7, 1.5e-5, 2.4e-7; fp64, degree 3: 5.8e-13,
+// 1.9e-12, 6.7e-14.
 // fp32 operator of the octant meshes: Q3 84 -> 73 us (269,998 cells), Q4 115 -> 111
 // us (296,535 cells); a level of few cells (Q4, 4,712 cells) 14.5 -> 9.3 us in fp32,
 // 34 -> 24.5 us in fp64.
@@ -31,8 +31,7 @@ namespace gcmg {
 // of DevTables::lame); a row: the even block, rows of (k+2)/2, then the odd block
 __host__ __device__ constexpr int zline_row(int k) { return k * (k + 1) * (2 * k + 1) / 6 - 1; }
 struct ZLines {
-  alignas(16) float f[zline_row(KMAX + 1)][16];  // fp32; then t
-  alignas(16) float h[zline_row(KMAX + 1)][16];
+  alignas(16) float h[zline_row(KMAX + 1)][16];  // then t
   alignas(16) float l[zline_row(KMAX + 1)][16];  // low parts: h + l to about 2^-48
 };
 static __constant__ ZLines c_zl;  // one copy per translation unit (upload_zlines)
@@ -74,7 +73,7 @@ __device__ __forceinline__ void zline(float* v, const float* c, bool constants) 
 }
 
 template <int K>
-__device__ __forceinline__ void zline(df* v, const float* ch, const float* cl) {
+__device__ __forceinline__ void zline(df* v, const float* ch, const float* cl, bool constants) {
   constexpr int N = K + 1, NH = N / 2, NE = (N + 1) / 2;
   df e[NE], o[NH];
 #pragma unroll
@@ -83,6 +82,11 @@ __device__ __forceinline__ void zline(df* v, const float* ch, const float* cl) {
     o[j] = df_sub_raw(v[j], v[K - j]);
   }
   if (N % 2) e[NH] = v[NH];
+  if (constants) {
+    const float t = ch[zline_count(K)];
+#pragma unroll
+    for (int j = 0; j < NE - 1; ++j) e[j] = df_sub_raw(e[j], df{t * e[NE - 1].hi, t * e[NE - 1].lo});
+  }
 #pragma unroll
   for (int i = 0; i < NE; ++i) {
     const df E = df_dot_raw<NE>(e, ch + NE * i, cl + NE * i);
@@ -120,11 +124,10 @@ static inline void upload_zlines() {
       for (int i = 0; i < 13; ++i) {
         z.h[zline_row(k) + q][i] = (float)c[i];
         z.l[zline_row(k) + q][i] = (float)(c[i] - (double)z.h[zline_row(k) + q][i]);
-        z.f[zline_row(k) + q][i] = z.h[zline_row(k) + q][i];
       }
       if (q == 0 && ne > 1) {  // modes (0, 0): constants; lam = 0
-        for (int i = 0; i < ne; ++i) z.f[zline_row(k) + q][ne * i + ne - 1] = 0.f;
-        z.f[zline_row(k) + q][nc] = ne > nh ? 2.f : 1.f;
+        for (int i = 0; i < ne; ++i) z.h[zline_row(k)][ne * i + ne - 1] = z.l[zline_row(k)][ne * i + ne - 1] = 0.f;
+        z.h[zline_row(k)][nc] = ne > nh ? 2.f : 1.f;
       }
     }
   cudaMemcpyToSymbol(c_zl, &z, sizeof(z));
