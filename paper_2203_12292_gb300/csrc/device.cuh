@@ -680,8 +680,8 @@ __device__ __forceinline__ df df_norm(float hi, float lo) {  // |lo| small again
 // a + b as an unnormalised pair: the low part may exceed half an ulp of the
 // high part.  For values that the same thread's next df_dot or df_add takes: both
 // keep every low part to fp32 precision, and the normalisation comes at the end
-// (12 of 175 operations of a sweep line fewer; with the scaling by a power of
-// two the fp64 operator of the Q4 octant took 479 instead of 502 us)
+// (12 of 175 operations of a sweep line fewer).  It costs up to two bits of the
+// pair: errors and times at df_add_step
 __device__ __forceinline__ df df_add_raw(df a, df b) {
   const float s = __fadd_rn(a.hi, b.hi);
   const float z = __fsub_rn(s, a.hi);
@@ -697,7 +697,6 @@ __device__ __forceinline__ df df_add(df a, df b) {
 __device__ __forceinline__ df df_neg(df a) { return df{-a.hi, -a.lo}; }
 
 __device__ __forceinline__ df df_sub(df a, df b) { return df_add(a, df_neg(b)); }
-__device__ __forceinline__ df df_sub_raw(df a, df b) { return df_add_raw(a, df_neg(b)); }
 
 // a * (ch + cl)
 __device__ __forceinline__ df df_mulc(df a, float ch, float cl) {

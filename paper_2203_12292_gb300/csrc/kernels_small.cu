@@ -72,7 +72,7 @@ __device__ __forceinline__ void cell_sweep(V* cb, int r, bool on) {
     V x[N];
 #pragma unroll
     for (int a = 0; a < N; ++a) x[a] = cb[base + a * S];
-    eo_line<K, FWD>(x);
+    eo_line<K, FWD, (K >= 3)>(x);  // normalised pairs at k >= 3: df_add_step
 #pragma unroll
     for (int a = 0; a < N; ++a) cb[base + a * S] = x[a];
   }
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(SWPB * 32) cell_vectors(CellVecArgs<T> A) {
 #pragma unroll
     for (int c = 0; c < N; ++c) x[c] = cl[r + N2 * c];
     if constexpr (sizeof(T) == 8)
-      zline<K>(x, zh, zl, r == 0);
+      zline<K, (K >= 3)>(x, zh, zl, r == 0);
     else
       zline<K>(x, zh, true);
 #pragma unroll

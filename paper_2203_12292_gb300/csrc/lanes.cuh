@@ -84,9 +84,26 @@ __device__ __forceinline__ df df_dot(const df* x, const float* ch, const float* 
   return df_norm(s.hi, s.lo);
 }
 
+// pairs between two steps of a line: normalised (NORM), or as they come.  Error of
+// the fp64 operator on random vectors (uniform cube, 4,096 cells), as they come /
+// normalised / of the line-parallel kernel: k = 1 2.4 / 2.4 / 2.9e-15, k = 2 4.2 / 4.1 /
+// 4.4e-15, k = 3 6.3 / 5.6 / 6.1e-15, k = 4 6.1 / 5.7 / 5.7e-15; of vmult_lanes_df with
+// a forward sweep, the scaling and a backward sweep, all normalised, in place of the
+// z-line: k = 2 4.4, k = 3 6.4, k = 4 6.4e-15.  So whole tiles take them as they come
+// (Q4 octant 438 us, normalised 488), the cell vectors at k >= 3 normalised (4,096
+// cells, k = 4: 16.2 -> 16.3 us).
+template <bool NORM>
+__device__ __forceinline__ df df_add_step(df a, df b) {
+  return NORM ? df_add(a, b) : df_add_raw(a, b);
+}
+template <int T, bool NORM>
+__device__ __forceinline__ df df_dot_step(const df* x, const float* ch, const float* cl) {
+  return NORM ? df_dot<T>(x, ch, cl) : df_dot_raw<T>(x, ch, cl);
+}
+
 // even-odd forward transform with B (nodal -> modes in mode order) and its
 // backward transform, in double-float, rows as df_dot
-template <int K>
+template <int K, bool NORM = false>
 __device__ __forceinline__ void df_eo_fwd_fast(df* u) {
   constexpr int N = K + 1, NH = N / 2, NE = (N + 1) / 2;
   const float(&Bh)[NMAX][NMAX] = c_tf[K].Be;
@@ -94,8 +111,8 @@ __device__ __forceinline__ void df_eo_fwd_fast(df* u) {
   df e[NE], o[NH > 0 ? NH : 1];
 #pragma unroll
   for (int j = 0; j < NH; ++j) {
-    e[j] = df_add_raw(u[j], u[N - 1 - j]);
-    o[j] = df_sub_raw(u[j], u[N - 1 - j]);
+    e[j] = df_add_step<NORM>(u[j], u[N - 1 - j]);
+    o[j] = df_add_step<NORM>(u[j], df_neg(u[N - 1 - j]));
   }
   if (N % 2) e[NH] = u[NH];
 #pragma unroll
@@ -104,7 +121,7 @@ __device__ __forceinline__ void df_eo_fwd_fast(df* u) {
   for (int r = 0; r < NH; ++r) u[NE + r] = df_dot<NH>(o, Bh[NE + r], Bl[NE + r]);
 }
 
-template <int K>
+template <int K, bool NORM = false>
 __device__ __forceinline__ void df_eo_bwd_fast(df* u) {
   constexpr int N = K + 1, NH = N / 2, NE = (N + 1) / 2;
   df E[NE], O[NH > 0 ? NH : 1];
@@ -116,7 +133,7 @@ __device__ __forceinline__ void df_eo_bwd_fast(df* u) {
       ch[r] = c_tf[K].Be[r][j];
       cl[r] = c_tflo[K].Be[r][j];
     }
-    E[j] = df_dot_raw<NE>(u, ch, cl);
+    E[j] = df_dot_step<NE, NORM>(u, ch, cl);
   }
 #pragma unroll
   for (int j = 0; j < NH; ++j) {
@@ -125,7 +142,7 @@ __device__ __forceinline__ void df_eo_bwd_fast(df* u) {
       ch[r] = c_tf[K].Be[NE + r][j];
       cl[r] = c_tflo[K].Be[NE + r][j];
     }
-    O[j] = df_dot_raw<NH>(u + NE, ch, cl);
+    O[j] = df_dot_step<NH, NORM>(u + NE, ch, cl);
   }
 #pragma unroll
   for (int j = 0; j < NH; ++j) {
@@ -174,19 +191,19 @@ struct Arith<double> {
   static __device__ __forceinline__ double out(V x) { return df_to(x); }
 };
 
-template <int K, bool FWD>
+template <int K, bool FWD, bool NORM = false>
 __device__ __forceinline__ void eo_line(float* v) {
   if (FWD)
     eo_forward<K + 1, 0, 1>(v, tab<float>(K).Be);
   else
     eo_backward<K + 1, 0, 1>(v, tab<float>(K).Be);
 }
-template <int K, bool FWD>
+template <int K, bool FWD, bool NORM = false>
 __device__ __forceinline__ void eo_line(df* v) {
   if (FWD)
-    df_eo_fwd_fast<K>(v);
+    df_eo_fwd_fast<K, NORM>(v);
   else
-    df_eo_bwd_fast<K>(v);
+    df_eo_bwd_fast<K, NORM>(v);
 }
 template <int K, bool TRANS>
 __device__ __forceinline__ void hang_line(float* v, int p) {

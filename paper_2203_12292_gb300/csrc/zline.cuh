@@ -72,26 +72,26 @@ __device__ __forceinline__ void zline(float* v, const float* c, bool constants) 
   }
 }
 
-template <int K>
+template <int K, bool NORM = false>
 __device__ __forceinline__ void zline(df* v, const float* ch, const float* cl, bool constants) {
   constexpr int N = K + 1, NH = N / 2, NE = (N + 1) / 2;
   df e[NE], o[NH];
 #pragma unroll
   for (int j = 0; j < NH; ++j) {
-    e[j] = df_add_raw(v[j], v[K - j]);
-    o[j] = df_sub_raw(v[j], v[K - j]);
+    e[j] = df_add_step<NORM>(v[j], v[K - j]);
+    o[j] = df_add_step<NORM>(v[j], df_neg(v[K - j]));
   }
   if (N % 2) e[NH] = v[NH];
   if (constants) {
     const float t = ch[zline_count(K)];
 #pragma unroll
-    for (int j = 0; j < NE - 1; ++j) e[j] = df_sub_raw(e[j], df{t * e[NE - 1].hi, t * e[NE - 1].lo});
+    for (int j = 0; j < NE - 1; ++j) e[j] = df_add_step<NORM>(e[j], df{-t * e[NE - 1].hi, -t * e[NE - 1].lo});
   }
 #pragma unroll
   for (int i = 0; i < NE; ++i) {
-    const df E = df_dot_raw<NE>(e, ch + NE * i, cl + NE * i);
+    const df E = df_dot_step<NE, NORM>(e, ch + NE * i, cl + NE * i);
     if (i < NH) {
-      const df O = df_dot_raw<NH>(o, ch + NE * NE + NH * i, cl + NE * NE + NH * i);
+      const df O = df_dot_step<NH, NORM>(o, ch + NE * NE + NH * i, cl + NE * NE + NH * i);
       v[i] = df_add(E, O);
       v[K - i] = df_sub(E, O);
     } else {
