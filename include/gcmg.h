@@ -119,12 +119,13 @@ typedef struct {
                               not a multigrid level.  Requires
                               p_coarsening = 0; not combinable with the learned
                               smoother, a coefficient or the batch. */
-  int transfer_chunk;      /* coarse cells per chunk of the restriction kernel:
-                              0 = default (4 on levels whose coarse side has
-                              more than 4 tiles per SM, 8 on smaller ones),
-                              4 or 8 = that size on every level (the same
-                              operator; a test knob for the 4-cell variant
-                              on small meshes) */
+  int transfer_chunk;      /* restriction kernel: 0 = default (one warp per
+                              coarse cell); 4 or 8 = the general kernel with
+                              that many coarse cells per chunk, on every
+                              level (the same operator to rounding).  Tiles
+                              above 32 cells and the persistent batch take
+                              the general kernel by themselves.  The
+                              prolongation does not depend on it */
 } gcmg_config;
 
 int gcmg_config_default(gcmg_config* cfg);

@@ -438,8 +438,8 @@ void vcycle_level(Handle& H, int l, bool pending) {
   // b^(l-1) = R r; local smoothing: b^(l-1) += R (r_S, r_E) on top of the values Algorithm 1
   // copied to level l-1 (r_E = -A_ES x_S: b_E is zero on level l)
   // onto a level of few cells the result stays in its cell vectors until its presmoothing starts
-  // (local smoothing: added to the copied values now)
-  const bool to_cells = C.n() && cells_ok(C.cl) && lattice_prolong_ok(H.tr[l]->tl);
+  // (local smoothing: added to the copied values now); a set chunk size asks for the general kernel
+  const bool to_cells = C.n() && cells_ok(C.cl) && C.cl.chunk == 0 && lattice_prolong_ok(H.tr[l]->tl);
   if (to_cells) {
     launch_restrict_cells(H.tr[l]->tl, f64, L.t.p, formed ? nullptr : L.b.p, H.stream);
     if (H.ls) launch_cell_sum(C.cl, f64, C.b.p, true, H.stream);
