@@ -154,16 +154,25 @@ void upload_tables_lattice();
 // the operator of a level of few cells: cell vectors, then one pass over the
 // DoFs that adds them up and goes on (kernels_small.cu)
 // Levels that take them: those too small for 32-cell tiles (fewer than two tiles
-// per SM), and larger ones of low degree up to CELL_VEC_MAX entries.  Postsmoothing
-// in fp32, tiles -> cell vectors: Q4 4,712 cells 61 -> 56 us, 7,680 cells 76 -> 51;
-// Q1 37,871 cells (0.30 M entries) 46 -> 23, 82,776 cells (0.66 M) 58 -> 36; Q2
-// 21,512 cells (0.58 M) 59 -> 50, but 32,768 cells (0.88 M) 40 -> 45 and Q4 21,512
-// cells (2.7 M) 111 -> 128 (fp64 crosses at the same sizes)
+// per SM), and larger ones of low degree up to CELL_VEC_MAX entries.  Postsmoothing,
+// lane kernels -> cell vectors, fp32 / fp64 in us: Q1 61,440 cells (0.49 M entries)
+// 31.6 -> 21.7 / 53.8 -> 55.6, 82,776 cells (0.66 M) 42.0 -> 32.9 / 80.5 -> 71.5, but
+// 113,688 (0.91 M) 43.9 -> 39.2 / 89.6 -> 91.8; Q2 28,400 cells (0.77 M) 45.9 -> 39.4 /
+// 96.4 -> 98.6, but 34,903 (0.94 M) 39.7 -> 39.0 / 84.1 -> 98.0; Q3 12,608 cells (0.81 M)
+// 43.0 -> 29.4 / 94.4 -> 76.2, but 28,400 (1.8 M) 64.4 -> 62.1 / 164 -> 194; Q4 9,024
+// cells 56.0 -> 43.5 / 148 -> 125, but 9,864 (1.2 M) 63.3 -> 54.6 / 175 -> 185.
 constexpr int64_t CELL_VEC_MAX = 850000;
 inline bool cell_vectors_pay(int64_t cells, int k, int n_sm) {
   return cells < 2 * (int64_t)n_sm * 32 || cells * (k + 1) * (k + 1) * (k + 1) <= CELL_VEC_MAX;
 }
 bool cells_ok(const CellLaunch& L);
+// The operator on its own has no update to go on with.  fp64 at degrees 1 and 2: the
+// lane kernels from fewer entries on.  Lane kernels / cell vectors: Q1 28,400 cells (0.23
+// M) 14.2 / 11.9 us, 32,768 (0.26 M) 7.7 / 15.2, 37,871 (0.30 M) 13.4 / 13.2, 61,440
+// 13.6 / 16.7; Q2 9,864 (0.27 M) 18.7 / 15.5, 11,096 (0.30 M) 15.5 / 15.7, 28,400 27.4 /
+// 31.2.  fp32 and degrees 3 and 4 keep the level's choice (Q1 80,781 cells 9.2 / 8.0,
+// Q2 28,400 12.9 / 12.5; fp64 Q3 12,608 26.4 / 22.9, Q4 9,024 40.9 / 37.3).
+bool cells_operator_ok(const CellLaunch& L, bool fp64);
 void launch_cell_vectors(const CellLaunch& L, bool fp64, const void* src, cudaStream_t s);
 void launch_cell_sum(const CellLaunch& L, bool fp64, void* dst, bool add, cudaStream_t s);
 void launch_cell_sum_residual(const CellLaunch& L, bool fp64, const void* b, void* r, cudaStream_t s);

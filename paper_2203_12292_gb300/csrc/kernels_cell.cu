@@ -1597,9 +1597,15 @@ size_t cell_smem_bytes(int k, bool fp64, int tc, int max_local, bool mapped) {
               : smem_layout<float>(n3, tc, max_local, mapped, mapped).total;
 }
 
+bool cells_operator_ok(const CellLaunch& L, bool fp64) {
+  if (!cells_ok(L)) return false;
+  if (!fp64 || L.k > 2 || !L.use_lanes || !lanes_ok(L)) return true;
+  return L.k == 1 ? 8 * (int64_t)L.n_cells <= 250000 : 27 * (int64_t)L.n_cells <= 290000;
+}
+
 void launch_vmult(const CellLaunch& L, bool fp64, const void* src, void* dst, int add, cudaStream_t s) {
   if (L.n_tiles == 0) return;
-  if (cells_ok(L)) {  // a level of few cells
+  if (cells_operator_ok(L, fp64)) {  // a level of few cells
     launch_cell_vectors(L, fp64, src, s);
     launch_cell_sum(L, fp64, dst, add != 0, s);
     return;
@@ -1630,7 +1636,7 @@ void launch_vmult(const CellLaunch& L, bool fp64, const void* src, void* dst, in
 }
 
 bool vmult_tiles_ok(const CellLaunch& L, bool fp64) {
-  if (cells_ok(L)) return false;
+  if (cells_operator_ok(L, fp64)) return false;
   if (L.use_lanes && lanes_ok(L)) return true;
   return L.tc <= CHUNK && !L.geom && (fp64 || (L.use_lines && L.threads == BLOCK));
 }
