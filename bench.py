@@ -27,6 +27,8 @@ beside it, and two further parts of the method:
   stream with seed 12292), operator tile size and thread mapping from the
   autotuner, solved to 1e-8 by one CUDA-graph launch.
 
+The printed line holds the headline; the tables behind it (autotuner, stages, levels)
+go into bench_details.json beside this file.
 Under torchrun every rank solves its own copy (replicas, weak scaling);
 value sums the ranks.
 
@@ -468,6 +470,57 @@ def finite(v):
     return v
 
 
+DETAILS = "bench_details.json"  # beside this file: everything measured, the long tables included
+LINE_MAX = 2600  # characters: the end of the output is what a caller keeps
+
+
+def headline(res):
+    """The printed line: the headline and one short entry per part of the run, numbers
+    to six digits; the autotuner's, the stages' and the levels' tables stay in DETAILS."""
+    def pick(d, *keys):
+        return {k: d[k] for k in keys if k in d} if d else None
+
+    def short(v):
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items()}
+        return [short(x) for x in v] if isinstance(v, (list, tuple)) else v
+
+    out = pick(res, "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+               "vs_baseline", "dtype", "data", "config", "gpu_launches", "clocks", "setup_s")
+    out["e2e"] = pick(res["e2e"], "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "one_vector_per_call_gdofs")
+    out["roofline"] = pick(res["roofline"], "bound", "achieved", "peak", "unit", "frac", "traffic", "peak_kind", "alu_frac")
+    out["vcycle"] = pick(res["vcycle"], "ms", "gdofs", "frac")
+    out["cpu_baseline"] = pick(res["cpu_baseline"], "value", "unit", "cores", "kind")
+    out["solve"] = pick(res["solve"], "mixed_ms", "mixed_iterations", "mixed_rel_residual", "fp64_ms", "fp64_iterations",
+                        "fp64_rel_residual", "solution_rel_diff_mixed_vs_fp64")
+    out["vmult"] = pick(res["vmult"], "fp32_ms", "fp32_gdofs", "fp64_ms", "fp64_gdofs")
+    if res["configs"]:
+        out["configs"] = {k: pick(c, "mixed_ms", "mixed_iterations", "fp64_ms", "fp64_iterations")
+                          for k, c in res["configs"].items()}
+    if res["learned"]:
+        out["learned"] = {"kept": res["learned"].get("kept"),
+                          "ms": {v["name"]: v["ms"] for v in res["learned"].get("variants", [])}}
+    if res["batch"]:
+        out["batch"] = pick(res["batch"], "problems", "dofs", "solve_ms", "all_converged")
+        out["batch"]["persistent"] = pick(res["batch"].get("persistent"), "solve_ms", "all_converged",
+                                          "max_rel_diff_vs_graph_batch")
+    out["details"] = DETAILS
+    return short(out)
+
+
+def report(res):
+    """Everything into DETAILS, the headline as the last line of the output."""
+    res = finite(res)
+    try:
+        with open(os.path.join(os.path.dirname(os.path.abspath(__file__)), DETAILS), "w") as f:
+            json.dump(res, f, allow_nan=False, indent=1)
+    except OSError as exc:  # a read-only tree: the line is what counts
+        print(f"{DETAILS}: {exc}", file=sys.stderr)
+    print(json.dumps(headline(res), allow_nan=False), flush=True)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -713,7 +766,7 @@ def main():
             "learned": learned,
             "batch": batch,
         }
-        print(json.dumps(finite(res), allow_nan=False), flush=True)
+        report(res)
     if dist is not None:
         dist.destroy_process_group()
 
