@@ -439,7 +439,7 @@ void vcycle_level(Handle& H, int l, bool pending) {
   // copied to level l-1 (r_E = -A_ES x_S: b_E is zero on level l)
   // onto a level of few cells the result stays in its cell vectors until its presmoothing starts
   // (local smoothing: added to the copied values now); a set chunk size asks for the general kernel
-  const bool to_cells = C.n() && cells_ok(C.cl) && C.cl.chunk == 0 && lattice_prolong_ok(H.tr[l]->tl);
+  const bool to_cells = C.n() && cells_ok(C.cl) && C.cl.chunk == 0;
   if (to_cells) {
     launch_restrict_cells(H.tr[l]->tl, f64, L.t.p, formed ? nullptr : L.b.p, H.stream);
     if (H.ls) launch_cell_sum(C.cl, f64, C.b.p, true, H.stream);
@@ -684,21 +684,7 @@ void setup_numerics(Handle& H) {
 void cell_vector_lists(const LevelHost& L, std::vector<int32_t>& ptr, std::vector<int32_t>& pos) {
   const int n1 = L.k + 1, n3 = n1 * n1 * n1;
   std::vector<int> slot(n3), off(n3);
-  for (int n = 0; n < n3; ++n) {
-    const int x[3] = {n % n1, (n / n1) % n1, n / (n1 * n1)};
-    int s = 0, o = 0, ms = 1, mo = 1;
-    for (int d = 0; d < 3; ++d) {
-      const int c = x[d] == 0 ? 0 : (x[d] == L.k ? 2 : 1);
-      s += c * ms;
-      ms *= 3;
-      if (c == 1) {
-        o += (x[d] - 1) * mo;
-        mo *= L.k - 1;
-      }
-    }
-    slot[n] = s;
-    off[n] = o;
-  }
+  for (int n = 0; n < n3; ++n) host_node_slot(L.k, n % n1, (n / n1) % n1, n / (n1 * n1), slot[n], off[n]);
   const size_t nc = L.cells.size();
   ptr.assign((size_t)L.n_free + 1, 0);
   for (size_t c = 0; c < nc; ++c)

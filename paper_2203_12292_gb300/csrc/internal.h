@@ -202,4 +202,24 @@ std::vector<int32_t> refinement_edge_dofs(const LevelHost& L, const Octree& leve
 void local_copy_map(const LevelHost& active, const std::vector<const LevelHost*>& levels,
                     std::vector<std::vector<int32_t>>& g, std::vector<std::vector<int32_t>>& idx);
 
+// entity slot and offset of local node (a, b, c) of a degree-k cell
+// (the numbering of the level set-up: slot cx + 3 cy + 9 cz, DoFs of an
+// entity lexicographic over its interior axes)
+inline void host_node_slot(int k, int a, int b, int c, int& slot, int& off) {
+  const int ca = a == 0 ? 0 : (a == k ? 2 : 1), cbb = b == 0 ? 0 : (b == k ? 2 : 1),
+            cc = c == 0 ? 0 : (c == k ? 2 : 1);
+  slot = ca + 3 * cbb + 9 * cc;
+  int o = 0, mul = 1;
+  if (ca == 1) {
+    o += a - 1;
+    mul *= k - 1;
+  }
+  if (cbb == 1) {
+    o += (b - 1) * mul;
+    mul *= k - 1;
+  }
+  if (cc == 1) o += (c - 1) * mul;
+  off = o;
+}
+
 }  // namespace gcmg

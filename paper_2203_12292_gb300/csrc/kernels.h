@@ -126,7 +126,7 @@ struct TransferLaunch {
   const uint32_t* own_f;    // fine cells
   const int32_t* gstart_c;  // coarse cells x 27
   const uint16_t* mask_c;   // coarse cells
-  const int32_t* lattice;   // h: entity table of the lattice kernels (null: not built)
+  const int32_t* lattice;   // h: entity table of the lattice kernels
   CellLaunch coarse;        // coarse level tiles (restriction scatter)
 };
 void launch_prolongate_add(const TransferLaunch& T, bool fp64, const void* coarse, void* fine, cudaStream_t s);
@@ -141,7 +141,6 @@ void launch_restrict_residual(const TransferLaunch& T, bool fp64, const void* b,
 // (lattice_table_words words) is built once per transfer from the other members
 size_t lattice_table_words(int k, int n_coarse);
 void launch_lattice_entities(const TransferLaunch& T, int32_t* table, cudaStream_t s);
-bool lattice_prolong_ok(const TransferLaunch& T);
 bool lattice_restrict_ok(const TransferLaunch& T);
 void launch_prolong_lattice(const TransferLaunch& T, bool fp64, const void* coarse, void* fine, cudaStream_t s);
 // coarse (+)= R fine, or R (rhs - fine) with rhs set
@@ -243,9 +242,9 @@ int64_t dot_noalloc_max_n();
 cudaError_t launch_dot_noalloc(const double* x, const double* y, int64_t n, double* result, cudaStream_t s);
 // CG updates with device scalars: scal[0] = rz, [1] = pq, [2] = rr, [3] = alpha, [4] = beta, [5] = rz_new,
 // [6] = r_{k+1}.z_k of flexible CG
-// rb != null: r is also written into the V-cycle's right-hand side (fp64 or rounded to fp32)
+// rb != null: r is also written into the V-cycle's right-hand side, rounded to fp32
 void launch_cg_update_xr(double* x, double* r, const double* p, const double* q, double* scal, int64_t n,
-                         double* scratch, cudaStream_t s, void* rb = nullptr, bool rb64 = false);
+                         double* scratch, cudaStream_t s, float* rb = nullptr);
 // CG as a loop inside a graph: further scalars.  cg_limits sets the limits of the
 // next solve, cg_start begins it (|b|^2 in scal[7]), the update of x and r ends
 // an iteration (it sets the WHILE node's condition h), cg_result writes

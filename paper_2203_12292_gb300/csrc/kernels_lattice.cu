@@ -96,7 +96,6 @@ struct LatArgs {
   const LaneHang* lh;
   T* halo;
   const int32_t* halo_pos;
-  int max_local;
 };
 
 // prolongation of one line: v[0..k] -> v[0..2k]
@@ -166,24 +165,6 @@ __device__ __forceinline__ void line_restrict(T* v) {
   v[K] += last;
 }
 
-template <int K, bool TRANS, typename T>
-__device__ __forceinline__ void interp_line(T* v, int p) {
-  constexpr int N = K + 1;
-  const DevTables<T>& tb = tab<T>(K);
-  T x[N], y[N];
-#pragma unroll
-  for (int a = 0; a < N; ++a) x[a] = p ? v[K - a] : v[a];
-#pragma unroll
-  for (int r = 0; r < N; ++r) {
-    T s = T(0);
-#pragma unroll
-    for (int a = 0; a < N; ++a) s += (TRANS ? tb.I[0][a][r] : tb.I[0][r][a]) * x[a];
-    y[r] = s;
-  }
-#pragma unroll
-  for (int a = 0; a < N; ++a) v[a] = p ? y[K - a] : y[a];
-}
-
 // lattice of one coarse cell of degree K: the children's (KF = 0, h transfer) or
 // the same cell's nodes of degree KF (p transfer)
 template <int K, int KF = 0>
@@ -241,6 +222,43 @@ struct Lat {
   }
 };
 
+// the three sweeps down on a warp's lattice: M^3 -> N^3 values, value i of the x-line
+// that starts at p to out(p, i, value)
+template <typename L, typename T, typename F>
+__device__ __forceinline__ void lattice_down(T* lat, int lane, F&& out) {
+  constexpr int N = L::N, M = L::M, M2 = L::M2;
+#pragma unroll 1
+  for (int q = lane; q < M2; q += 32) {  // z-lines
+    T v[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) v[i] = lat[q + M2 * i];
+    L::down(v);
+#pragma unroll
+    for (int i = 0; i < N; ++i) lat[q + M2 * i] = v[i];
+  }
+  __syncwarp();
+#pragma unroll 1
+  for (int q = lane; q < M * N; q += 32) {  // y-lines (x, c)
+    T* p = lat + q % M + M2 * (q / M);
+    T v[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) v[i] = p[M * i];
+    L::down(v);
+#pragma unroll
+    for (int i = 0; i < N; ++i) p[M * i] = v[i];
+  }
+  __syncwarp();
+  if (lane < N * N) {  // x-lines (b, c)
+    T* p = lat + M * (lane % N) + M2 * (lane / N);
+    T v[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) v[i] = p[i];
+    L::down(v);
+#pragma unroll
+    for (int i = 0; i < N; ++i) out(p, i, v[i]);
+  }
+}
+
 // shared memory: lane records, point tables, entity starts, then the cell
 // buffer, then the warps' lattices; the tile's accumulator takes the lattices'
 // place once every cell of the tile has been reduced
@@ -261,7 +279,7 @@ template <int K, typename T, int KF>
 __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
   using L = Lat<K, KF>;
   using SM = RestrictSmem<K, T, KF>;
-  constexpr int N = L::N, N2 = L::N2, N3 = L::N3, M = L::M, M2 = L::M2;
+  constexpr int N = L::N, N2 = L::N2, N3 = L::N3;
   constexpr int NT = WPB * 32;
   extern __shared__ __align__(16) unsigned char smem[];
   LaneTile* st = reinterpret_cast<LaneTile*>(smem);
@@ -321,36 +339,8 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
           if (b + u < L::NI) lat[pos[u]] = v[u];
       }
       __syncwarp();
-#pragma unroll 1
-      for (int q = lane; q < M2; q += 32) {  // z-lines
-        T v[M];
-#pragma unroll
-        for (int i = 0; i < M; ++i) v[i] = lat[q + M2 * i];
-        L::down(v);
-#pragma unroll
-        for (int i = 0; i < N; ++i) lat[q + M2 * i] = v[i];
-      }
-      __syncwarp();
-#pragma unroll 1
-      for (int q = lane; q < M * N; q += 32) {  // y-lines (x, c)
-        T* p = lat + q % M + M2 * (q / M);
-        T v[M];
-#pragma unroll
-        for (int i = 0; i < M; ++i) v[i] = p[M * i];
-        L::down(v);
-#pragma unroll
-        for (int i = 0; i < N; ++i) p[M * i] = v[i];
-      }
-      __syncwarp();
-      if (lane < N2) {  // x-lines (b, c), into the cell buffer
-        const T* p = lat + M * (lane % N) + M2 * (lane / N);
-        T v[M];
-#pragma unroll
-        for (int i = 0; i < M; ++i) v[i] = p[i];
-        L::down(v);
-#pragma unroll
-        for (int i = 0; i < N; ++i) cb[(N * lane + i) * CBS + j] = v[i];
-      }
+      // the x-lines' results into the cell buffer
+      lattice_down<L>(lat, lane, [&](T*, int i, T v) { cb[(N * lane + i) * CBS + j] = v; });
     } else {  // identity category (no fine cells: no owned slots, zeros)
 #pragma unroll
       for (int i = 0; i < L::NJ; ++i) {
@@ -381,7 +371,7 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
         T v[N];
 #pragma unroll
         for (int a = 0; a < N; ++a) v[a] = p[a * N2 * CBS];
-        interp_line<K, true>(v, (m >> 2) & 1);
+        interp_line_reg<K, true>(v, (m >> 2) & 1);
 #pragma unroll
         for (int a = 0; a < N; ++a) p[a * N2 * CBS] = v[a];
       }
@@ -393,7 +383,7 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
         T v[N];
 #pragma unroll
         for (int a = 0; a < N; ++a) v[a] = p[a * N * CBS];
-        interp_line<K, true>(v, (m >> 1) & 1);
+        interp_line_reg<K, true>(v, (m >> 1) & 1);
 #pragma unroll
         for (int a = 0; a < N; ++a) p[a * N * CBS] = v[a];
       }
@@ -409,7 +399,7 @@ __global__ void __launch_bounds__(WPB * 32) restrict_lattice(LatArgs<T> A) {
       T v[N];
 #pragma unroll
       for (int a = 0; a < N; ++a) v[a] = cb[(N * r + a) * CBS + lane];
-      if (hang && ((hg->hl[0][lane] >> r) & 1u)) interp_line<K, true>(v, m & 1);
+      if (hang && ((hg->hl[0][lane] >> r) & 1u)) interp_line_reg<K, true>(v, m & 1);
       const uint32_t li = c_ll.line[K][r];
       const int s0 = li & 0xff, o0 = (li >> 8) & 0xff, o1 = li >> 16;
       T* p0 = reinterpret_cast<T*>(xb + SC * (st->ls[s0][lane] + o0));
@@ -444,7 +434,7 @@ __device__ __forceinline__ void lattice_hang(T* lat, uint16_t m, int lane) {
   T x[L::N];
 #pragma unroll
   for (int a = 0; a < L::N; ++a) x[a] = p[a * S];
-  interp_line<K, TRANS>(x, (m >> D) & 1);
+  interp_line_reg<K, TRANS>(x, (m >> D) & 1);
 #pragma unroll
   for (int a = 0; a < L::N; ++a) p[a * S] = x[a];
 }
@@ -565,7 +555,7 @@ __global__ void __launch_bounds__(WPB * 32) prolong_lattice(LatArgs<T> A) {
 template <int K, typename T, int KF>
 __global__ void __launch_bounds__(WPB * 32) restrict_cells(LatArgs<T> A) {
   using L = Lat<K, KF>;
-  constexpr int N = L::N, N3 = L::N3, M = L::M, M2 = L::M2;
+  constexpr int N3 = L::N3;
   constexpr int NT = WPB * 32;
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -605,36 +595,7 @@ __global__ void __launch_bounds__(WPB * 32) restrict_cells(LatArgs<T> A) {
 #pragma unroll
     for (int i = 0; i < L::NI; ++i) lat[s_pt[lane + 32 * i] >> 12] = v[i];
     __syncwarp();
-#pragma unroll 1
-    for (int q = lane; q < M2; q += 32) {  // z-lines
-      T x[M];
-#pragma unroll
-      for (int i = 0; i < M; ++i) x[i] = lat[q + M2 * i];
-      L::down(x);
-#pragma unroll
-      for (int i = 0; i < N; ++i) lat[q + M2 * i] = x[i];
-    }
-    __syncwarp();
-#pragma unroll 1
-    for (int q = lane; q < M * N; q += 32) {  // y-lines (x, c)
-      T* p = lat + q % M + M2 * (q / M);
-      T x[M];
-#pragma unroll
-      for (int i = 0; i < M; ++i) x[i] = p[M * i];
-      L::down(x);
-#pragma unroll
-      for (int i = 0; i < N; ++i) p[M * i] = x[i];
-    }
-    __syncwarp();
-    if (lane < N * N) {  // x-lines (b, c)
-      T* p = lat + M * (lane % N) + M2 * (lane / N);
-      T x[M];
-#pragma unroll
-      for (int i = 0; i < M; ++i) x[i] = p[i];
-      L::down(x);
-#pragma unroll
-      for (int i = 0; i < N; ++i) p[i] = x[i];
-    }
+    lattice_down<L>(lat, lane, [](T* p, int i, T x) { p[i] = x; });
   } else {  // identity category (no fine cells: no owned slots, zeros)
 #pragma unroll
     for (int i = 0; i < L::NJ; ++i) {
@@ -802,7 +763,6 @@ LatArgs<T> lat_args(const TransferLaunch& L, const T* src, T* dst) {
   A.lh = static_cast<const LaneHang*>(L.coarse.lane_hang);
   A.halo = static_cast<T*>(L.coarse.halo);
   A.halo_pos = L.coarse.halo_pos;
-  A.max_local = L.coarse.max_local;
   return A;
 }
 
@@ -897,10 +857,7 @@ void launch_lattice_entities(const TransferLaunch& L, int32_t* ent, cudaStream_t
 // The restriction accumulates through the coarse level's lane records, which
 // exist for tiles of at most 32 cells, and reads its record per tile: larger
 // tiles keep restrict_h.
-bool lattice_prolong_ok(const TransferLaunch& L) { return L.kind == 1 || L.lattice; }
-bool lattice_restrict_ok(const TransferLaunch& L) {
-  return lattice_prolong_ok(L) && L.coarse.lane_tiles && L.coarse.tc <= 32;
-}
+bool lattice_restrict_ok(const TransferLaunch& L) { return L.coarse.lane_tiles && L.coarse.tc <= 32; }
 
 void launch_prolong_lattice(const TransferLaunch& L, bool fp64, const void* coarse, void* fine, cudaStream_t s) {
   if (fp64)

@@ -608,8 +608,7 @@ void restrict_p_run(const TransferLaunch& L, const T* src, T* dst, const T* rhs,
   launch_halo_add(L.coarse, sizeof(T) == 8, dst, s);
 }
 
-template <typename T>
-void prolong_any(const TransferLaunch& L, const T* src, T* dst, cudaStream_t s) {
+void prolong_any(const TransferLaunch& L, const float* src, float* dst, cudaStream_t s) {
   if (L.kind == 0) {
     switch (L.kf) {
       case 1: prolong_h_run<1>(L, src, dst, s); break;
@@ -648,23 +647,19 @@ void restrict_any(const TransferLaunch& L, const T* src, T* dst, const T* rhs, b
 }  // namespace
 
 #ifndef GCMG_BODIES_ONLY
-// The h transfer runs one warp per coarse cell (kernels_lattice.cu).  The
-// kernels of this file take the p transfer, the restriction onto tiles above 32
-// cells and with a set chunk size, and the recorded launches of the persistent
-// batch, whose blocks all have the layout of these kernels.
+// Both transfers run one warp per coarse cell (kernels_lattice.cu).  The kernels of
+// this file take the restriction onto tiles above 32 cells and with a set chunk
+// size, and the recorded launches of the persistent batch (fp32 only), whose blocks
+// all have the layout of these kernels.
 bool lattice_restrict(const TransferLaunch& L) {
   return lattice_restrict_ok(L) && L.coarse.chunk == 0 && !dwl_recording();
 }
 
 void launch_prolongate_add(const TransferLaunch& L, bool fp64, const void* coarse, void* fine, cudaStream_t s) {
-  if (lattice_prolong_ok(L) && !dwl_recording()) {
+  if (dwl_recording() && !fp64)
+    prolong_any(L, static_cast<const float*>(coarse), static_cast<float*>(fine), s);
+  else  // (recorded in fp64: refused there, as every fp64 level is)
     launch_prolong_lattice(L, fp64, coarse, fine, s);
-    return;
-  }
-  if (fp64)
-    prolong_any<double>(L, static_cast<const double*>(coarse), static_cast<double*>(fine), s);
-  else
-    prolong_any<float>(L, static_cast<const float*>(coarse), static_cast<float*>(fine), s);
 }
 
 void launch_restrict_add(const TransferLaunch& L, bool fp64, const void* fine, void* coarse, cudaStream_t s) {

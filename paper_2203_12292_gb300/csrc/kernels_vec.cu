@@ -695,22 +695,18 @@ void launch_dot(const double* x, const float* y, int64_t n, double* scratch, dou
 }
 
 void launch_cg_update_xr(double* x, double* r, const double* p, const double* q, double* scal, int64_t n,
-                         double* scratch, cudaStream_t s, void* rb, bool rb64) {
+                         double* scratch, cudaStream_t s, float* rb) {
   if (dwl_recording()) {
-    float* r32 = rb64 ? nullptr : static_cast<float*>(rb);
-    if (r32)
-      launch_pdl(cg_xr_b<true>, DOT_BLOCKS, BLOCK, 0, s, x, r, p, q, (const double*)scal, n, scratch, r32);
+    if (rb)
+      launch_pdl(cg_xr_b<true>, DOT_BLOCKS, BLOCK, 0, s, x, r, p, q, (const double*)scal, n, scratch, rb);
     else
-      launch_pdl(cg_xr_b<false>, DOT_BLOCKS, BLOCK, 0, s, x, r, p, q, (const double*)scal, n, scratch, r32);
+      launch_pdl(cg_xr_b<false>, DOT_BLOCKS, BLOCK, 0, s, x, r, p, q, (const double*)scal, n, scratch, rb);
     note_launches(1);
     launch_pdl(dot_final, 1, BLOCK, 0, s, scratch, DOT_BLOCKS, scal, 2, DOT_STORE);
     note_launches(1);
     return;
   }
-  if (rb64)
-    cg_xr_any(x, r, p, q, scal, n, scratch, static_cast<double*>(rb), 0, cudaGraphConditionalHandle{}, s);
-  else
-    cg_xr_any(x, r, p, q, scal, n, scratch, static_cast<float*>(rb), 0, cudaGraphConditionalHandle{}, s);
+  cg_xr_any(x, r, p, q, scal, n, scratch, rb, 0, cudaGraphConditionalHandle{}, s);
 }
 
 void launch_cg_update_xr_loop(double* x, double* r, const double* p, const double* q, double* scal, int64_t n,

@@ -35,16 +35,16 @@ static __constant__ LaneLines c_ll;  // one copy per translation unit (filled by
 // registers.  I_1[a][b] = I_0[k-a][k-b] (Gauss-Lobatto points and Lagrange
 // basis are symmetric under x -> 1 - x), so p = 1 reverses the line, applies
 // I_0 and reverses back: one set of constant-operand multiply-adds
-template <int K, bool TRANS>
-__device__ __forceinline__ void interp_line_reg(float* v, int p) {
+template <int K, bool TRANS, typename T>
+__device__ __forceinline__ void interp_line_reg(T* v, int p) {
   constexpr int N = K + 1;
-  const DevTables<float>& tb = tab<float>(K);
-  float x[N], y[N];
+  const DevTables<T>& tb = tab<T>(K);
+  T x[N], y[N];
 #pragma unroll
   for (int a = 0; a < N; ++a) x[a] = p ? v[K - a] : v[a];
 #pragma unroll
   for (int r = 0; r < N; ++r) {
-    float s = 0.f;
+    T s = T(0);
 #pragma unroll
     for (int a = 0; a < N; ++a) s += (TRANS ? tb.I[0][a][r] : tb.I[0][r][a]) * x[a];
     y[r] = s;
@@ -212,26 +212,6 @@ __device__ __forceinline__ void hang_line(float* v, int p) {
 template <int K, bool TRANS>
 __device__ __forceinline__ void hang_line(df* v, int p) {
   interp_line_df<K, TRANS>(v, p);
-}
-
-// host: entity slot and offset of local node (a, b, c) of a degree-k cell
-// (the numbering of the level set-up: slot cx + 3 cy + 9 cz, DoFs of an
-// entity lexicographic over its interior axes)
-inline void host_node_slot(int k, int a, int b, int c, int& slot, int& off) {
-  const int ca = a == 0 ? 0 : (a == k ? 2 : 1), cbb = b == 0 ? 0 : (b == k ? 2 : 1),
-            cc = c == 0 ? 0 : (c == k ? 2 : 1);
-  slot = ca + 3 * cbb + 9 * cc;
-  int o = 0, mul = 1;
-  if (ca == 1) {
-    o += a - 1;
-    mul *= k - 1;
-  }
-  if (cbb == 1) {
-    o += (b - 1) * mul;
-    mul *= k - 1;
-  }
-  if (cc == 1) o += (c - 1) * mul;
-  off = o;
 }
 
 // x-line tables: slots and offsets per line; the line classes (lines whose
