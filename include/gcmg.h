@@ -99,9 +99,11 @@ typedef struct {
   int tile_cells;          /* cells per tile on large levels, 0 = default (32);
                               levels with fewer than 2 * 152 tiles of that
                               size use halved tiles (down to 8 cells) */
-  int cell_kernel;         /* operator kernel: 0 = default (one lane per cell
-                              on levels with 32-cell tiles, fp32 and fp64;
-                              else line-parallel), 1 = line-parallel (one
+  int cell_kernel;         /* operator kernel: 0 = default (levels of few
+                              cells: one warp per cell writes the cell's
+                              result, one thread per DoF adds them up; else
+                              one lane per cell on levels with 32-cell
+                              tiles, fp32 and fp64; else line-parallel), 1 = line-parallel (one
                               thread per 1D line of a cell), 2 = slab threads
                               (fp32, k+1 threads per cell, z-slabs in
                               registers; tiles <= 64 cells), 3 = one lane per
@@ -242,6 +244,8 @@ int gcmg_get_coefficient(gcmg_handle* h, int level, double* nu);
 int gcmg_quadrature_points(gcmg_handle* h, double* xyz);
 /* lambda_max used by the Chebyshev smoother of a level (after the safety factor) */
 int gcmg_get_lambda(const gcmg_handle* h, int level, double* lam);
+/* Another value than the set-up's on a level of at most 1,024 DoFs: the cycle
+ * runs these levels one by one instead of as one matrix (gcmg_vcycle) until every one of them has the set-up's value again. */
 int gcmg_set_lambda(gcmg_handle* h, int level, double lam);
 /*
  * Chebyshev iteration around point Jacobi (Sec. 3.3) on a level:
@@ -257,7 +261,10 @@ int gcmg_restrict_add(gcmg_handle* h, int fine_level, int fp64, const void* fine
 int gcmg_coarse_solve(gcmg_handle* h, int fp64, const void* b, void* x);
 /*
  * x = V-cycle(b) (Algorithms 1-2): b, x are fp64 device vectors of the
- * finest level; the levels run in the configured precision.
+ * finest level; the levels run in the configured precision.  The levels of at
+ * most 1,024 DoFs are applied as one matrix, built in fp64 by the set-up and
+ * applied in fp64 (Cartesian cells, Chebyshev smoother, set-up's intervals,
+ * timers off; under local smoothing up to the first level with copied values).
  */
 int gcmg_vcycle(gcmg_handle* h, const double* b, double* x);
 /*
@@ -332,7 +339,15 @@ int gcmg_vmult_host_many(gcmg_handle* h, int level, int fp64, int n, const void*
 #define GCMG_STAGE_CG_VMULT 7    /* fp64 operator of CG on the finest level */
 #define GCMG_STAGE_CG_VECTOR 8   /* CG inner products, updates, precision casts */
 #define GCMG_STAGE_LEARNED 9     /* learned smoother: its residual and correction */
-/* switch the timers on/off; both reset the accumulated times */
+/*
+ * Switch the timers on/off; both reset the accumulated times.  A stage can only
+ * be timed where it is run on its own, so with timers on the cycle runs the levels
+ * of at most 1,024 DoFs one by one instead of as one matrix, and CG as a host
+ * loop around captured halves instead of one graph launch: the same results up to
+ * rounding, and a sum of stages above the time of a solve without timers.  On
+ * levels of few cells GCMG_STAGE_VMULT is the cells' part of an application; the
+ * pass that adds them up belongs to the stage it goes on with.
+ */
 int gcmg_set_profiling(gcmg_handle* h, int on);
 /* accumulated launches and milliseconds of one (level, stage); synchronises */
 int gcmg_get_profile(gcmg_handle* h, int level, int stage, int64_t* count, double* ms);
@@ -352,9 +367,11 @@ typedef struct {
 int gcmg_cg_solve(gcmg_handle* h, const double* b, double* x, double rtol, int maxit, gcmg_solve_stats* stats);
 
 /*
- * 1 (default): the V-cycle and the operator half of every CG iteration run as
- * CUDA graphs captured on first use; 0: plain stream launches.  Graphs are
- * re-captured after gcmg_set_lambda and gcmg_set_profiling.
+ * 1 (default): CUDA graphs captured on first use: a V-cycle is one, and a solve
+ * one with its iterations as a loop inside it (with timers or a learned smoother:
+ * the V-cycle and the operator half of an iteration one each); 0: plain stream
+ * launches.  Graphs are re-captured after gcmg_set_lambda, gcmg_set_profiling,
+ * gcmg_set_smoother, gcmg_set_coefficient and gcmg_set_geometry.
  */
 int gcmg_set_graphs(gcmg_handle* h, int on);
 

@@ -646,6 +646,8 @@ void setup_dense(Handle& H) {
   }
   ck_launches("dense levels");
   ck(cudaStreamSynchronize(H.stream), "dense levels");  // the scratch is freed on return
+  H.dense_lam.clear();
+  for (int l = 0; l <= top; ++l) H.dense_lam.push_back(H.lev[l]->lam);
   H.dense_top = top;
   H.dense_ok = true;
 }
@@ -1336,7 +1338,11 @@ int gcmg_set_lambda(gcmg_handle* h, int level, double lam) {
     if (!h || !(lam > 0)) throw Error(GCMG_ERR_ARG, "bad lambda");
     check_level(h->h, level);
     h->h.lev[level]->lam = lam;
-    if (level <= h->h.dense_top) h->h.dense_ok = false;  // that interval is not the matrix's: level by level from now on
+    Handle& H = h->h;
+    if (level <= H.dense_top) {  // level by level while an interval is not the matrix's
+      H.dense_ok = true;
+      for (int q = 1; q <= H.dense_top; ++q) H.dense_ok = H.dense_ok && H.lev[q]->lam == H.dense_lam[q];
+    }
     reset_graphs(h->h);
   });
 }

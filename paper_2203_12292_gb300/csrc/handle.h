@@ -98,6 +98,7 @@ struct Handle {
   // belongs to the levels' present operators and Chebyshev intervals
   int dense_top = -1;
   bool dense_ok = false;
+  std::vector<double> dense_lam;  // the intervals it was built with
   DevBuf dense;
   int top_mg = 0;               // finest multigrid level (lev.size() - 1 for global coarsening)
   bool in_batch = false;        // owned by a batch, whose graph holds the kernels' arguments
