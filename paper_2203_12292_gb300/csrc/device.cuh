@@ -646,10 +646,12 @@ __device__ __forceinline__ df df_from(double x) {
 
 __device__ __forceinline__ double df_to(df a) { return (double)a.hi + (double)a.lo; }
 
-// The same two conversions with integer operations on the bits, equal to the last
-// bit: the conversions and the addition above run on the FP64 pipe, which was
-// busy 57 % of vmult_lanes_df's time with nothing else.  Values outside the range
-// whose parts are normal floats take the conversions.
+// The same two conversions with integer operations on the bits: the conversions
+// and the addition above run on the FP64 pipe, which was busy 57 % of
+// vmult_lanes_df's time with nothing else.  df_to_bits equals df_to to the last
+// bit.  df_from_bits gives a pair of the same value hi + lo as df_from; where x
+// lies half way between two floats it rounds hi away from zero, df_from to even.
+// Values outside the range whose parts are normal floats take the conversions.
 __device__ __forceinline__ df df_from_bits(double x) {
   const uint64_t b = (uint64_t)__double_as_longlong(x);
   const uint32_t h0 = (uint32_t)(b >> 32);
