@@ -75,9 +75,9 @@ BYTES_PER_DOF = {"fp32": 9.8, "fp64": 17.8}
 # this workload, both of its launches, from one ncu capture of
 # dram__bytes_read.sum + dram__bytes_write.sum with caches flushed before each
 # kernel (ncu's default), mean of two applications: tile kernel vmult_lanes<4>
-# 138.4 MB read + 59.4 MB written, halo pass 60.0 MB + 0.1 MB; set to 0
+# 138.4 MB read + 59.8 MB written, halo pass 60.0 MB + 0.1 MB; set to 0
 # (reported as null) when the kernels change until they are captured again
-VMULT_TRAFFIC_BYTES = 257.9e6
+VMULT_TRAFFIC_BYTES = 258.4e6
 # V-cycle bytes per finest-level DoF (fp32): six operator applications and
 # five vector updates per level, the transfers, summed over the levels with
 # the 1/(1 - 1/8) factor of the coarser levels
