@@ -44,3 +44,25 @@ def test_route(gcmg, i):
     b.smooth(L, s[1], y, False)
     assert not torch.equal(s[0], s[1])
     assert float((s[0] - s[1]).norm()) <= 8e-12 * float(s[1].norm())
+
+
+@pytest.mark.parametrize("k,recipe", [(1, synth.sphere(6)), (1, synth.cube_octant(5, 1)), (2, synth.sphere(6)),
+                                      (3, synth.cube_octant(4, 1))])
+def test_cell_vectors_beyond_two_tiles_per_sm(gcmg, k, recipe):
+    """the larger levels of low degree that take the cell vectors, against one lane per cell"""
+    m = gcmg.Mesh.from_recipe(recipe)
+    a, b = gcmg.Multigrid(m, k), gcmg.Multigrid(m, k, cell_kernel=3)
+    L = a.finest
+    for dtype, tol in ((torch.float64, 2e-12), (torch.float32, 4e-6)):
+        gen = torch.Generator(device="cuda").manual_seed(21)
+        x, f = (torch.randn(a.n_free(L), dtype=dtype, device="cuda", generator=gen) for _ in range(2))
+        y, z = torch.empty_like(x), torch.empty_like(x)
+        a.vmult(L, x, y)
+        b.vmult(L, x, z)
+        assert float((y - z).double().norm()) <= tol * float(z.double().norm())
+        for zero in (False, True):  # three applications: four times the tolerance
+            s, t = x.clone(), x.clone()
+            a.smooth(L, s, f, zero)
+            b.smooth(L, t, f, zero)
+            assert not torch.equal(s, t)
+            assert float((s - t).double().norm()) <= 4 * tol * float(t.double().norm())
